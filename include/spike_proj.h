@@ -368,13 +368,15 @@ sp_status spike_proj_decode_noalloc(const int8_t *W, int64_t ldw,
  *
  *     y[b*ldy + m] = s_m * sum_{k<K} float(W[m*ldw + k]) * x[b*ldx + k]
  *
- * computed in FP32: each lane of a warp accumulates the products of its
- * 16-column chunks (columns 16 l .. 16 l + 15 of every 512) with fmaf in
- * ascending k, the 32 lane sums meet in a 5-level butterfly, and one FP32
- * multiply applies s_m.  Each y is thus the FP32 value of a fixed summation
- * tree of depth d <= 16 * ceil(K / 512) + 5, identical on every run, with
- * |y - s_m * exact| <= |s_m| * gamma(d) * sum_k |W x| + u |y| (u = 2^-24,
- * gamma(d) = d u / (1 - d u)).  Weights are read once per call for all B rows.
+ * computed in FP32: every product is exact (or, with FMAs, enters its
+ * addition unrounded) and the sums round in FP32 in an order fixed by the
+ * sizes of the call, so a result is identical on every run; one FP32 multiply
+ * applies s_m.  Small launches and large K sum with fmaf, a tree of depth
+ * d <= 16 * ceil(K / 512) + 5; larger launches multiply on the tensor cores
+ * (each activation as the exact sum of three bf16 parts) and are held to the
+ * same bound, |y - s_m * exact| <= |s_m| * gamma(d) * sum_k |W x| + u |y|
+ * (u = 2^-24, gamma(d) = d u / (1 - d u)).  Weights are read once per call for
+ * all B rows.
  *
  *   problems[j]  one projection (fields below); count in 1 ..
  *                SPIKE_PROJ_DENSE_MAX_GROUP.  All run in ONE kernel launch.

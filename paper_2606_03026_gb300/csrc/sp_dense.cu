@@ -11,16 +11,57 @@
 // decode step).  The weights stream from HBM once per call, so the kernel is
 // HBM-bound: algorithmic bytes = sum over problems of N * K.
 //
-// A unit is 4 consecutive rows of one problem, owned by one warp.  Lane l
+// Two forms.
+//
+// dense_mma_kernel<B>: the products run on the tensor cores and stay exact.
+// An INT8 weight is a bf16 value exactly, and a normal FP32 activation is the
+// exact sum of three bf16 values (its 24 significant bits in three runs of 8:
+// x = hi + mid + lo), so every bf16 x bf16 product of mma.sync m16n8k16 is an
+// exact part of the FP32 product and only the additions round.  Per warp: 16
+// weight rows as the MMA's M, the split activations of all B rows as its N
+// (columns 4 b + {0, 1, 2} = hi, mid, lo of row b), 64 weight columns per
+// chunk.  The chunk's MMAs start from zero and their sums are added to the
+// running FP32 sums of the lane, so the tensor core's own accumulation chain
+// is four MMAs long; at the end y = s * (hi + (mid + lo)).  Relative error
+// (2-norm, K = 1536, N(0, 1) activations) 8.2e-8, against 1.4e-7 with FMAs.
+// Bounds and layout:
+//   - with FP32 FMAs the kernel is bound by instructions and L1 (per weight a
+//     byte permute, an FADD and B FFMAs, and every lane re-reads the
+//     activations).  The MMA takes the multiplications for all B rows at
+//     once; what is left per 4 weights is 5 logic operations and 2 packed
+//     subtractions (byte -> bf16: 128 + low 7 bits, minus 128 or 256).
+//   - lane (g, t) copies 16 bytes of rows g and g + 8 (four lanes share 64
+//     bytes of a row) with cp.async into its own slots of an 8-chunk ring and
+//     reads them back itself: 128 KB in flight per SM, no barrier, and no
+//     registers held by loads (a register ring of the same depth was slower,
+//     83 and 91 us against 72 and 75 for one and four rows below: it shares
+//     the six load scoreboards of a warp).  The K order inside a chunk is
+//     permuted alike on both operands.
+//   - the split activations of the CTA's problems are made once, in shared
+//     memory, in the order of the MMA's B operand (1 KB per 64 columns and two
+//     activation rows), while the first ring is in flight.
+//   - one 512-thread CTA per SM takes an equal, contiguous share of the
+//     launch's chunks, so that it meets one or two activation tables.
+// Measured on 66 projections (4608 / 1536 / 6144 x 1536, 415 MB): 70.6 us for
+// one activation row (5.9 TB/s) and 73.2 us for four; with dense_kernel 81 and
+// 259 us.
+//
+// dense_kernel<B> (small launches, and K whose table does not fit): a unit
+// is 4 consecutive rows of one problem, owned by one warp.  Lane l
 // covers the 16-column chunks l, l + 32, l + 64, ... of the row (16-byte
 // weight loads, 512 contiguous bytes per warp instruction), issuing the loads
 // of one chunk of all 4 rows before any arithmetic.  A weight byte
 // becomes a float exactly through its bias (w + 128 in the low byte of 2^23's
 // mantissa, minus 2^23 + 128).  Each lane accumulates with fmaf in ascending
 // k, the 32 lane sums meet in a 5-level butterfly, and one FP32 multiply by s_m
-// gives y.  Every output is therefore an FP32 sum of K products of depth at
-// most 16 * ceil(K / 512) + 5, whatever the grid, so the error bound and the
-// result are the same on every run.
+// gives y: an FP32 sum of K products of depth at most 16 * ceil(K / 512) + 5.
+// Its small CTAs start while the previous kernel drains: 2.2 us a call at
+// 0.5 MB, where the tensor-core form, which fills its SM, takes 4.1.
+// dense_mma_kernel runs a problem with FMAs too when an activation is not
+// finite or outside 2^-100 .. 2^100 (its three parts would not be exact).
+//
+// In both forms the order of every sum depends on the sizes alone, so the
+// result is the same on every run.
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
 #include "sp_spikes.cuh"
@@ -34,7 +75,7 @@ constexpr int kDenseThreads = 256;
 // CTAs per SM the registers must allow.  One chunk of 4 rows per round: the
 // converted weights stay in registers for the B activation rows, and more
 // warps with less in flight each stream faster than fewer warps with three
-// chunks (measured on the 22-block step: B = 1 at 32 warps per SM 5.1 TB/s
+// chunks (measured on 415 MB of weights: B = 1 at 32 warps per SM 5.1 TB/s
 // against 3.6 with three chunks; B = 2 / 3 / 4 at 16 warps per SM 2.9 / 2.3 /
 // 1.7 TB/s against 2.5 / 1.6 / 1.3).
 template <int B> struct DenseShape { static constexpr int batch = 1, min_ctas = 2; };
@@ -47,76 +88,403 @@ struct DenseParams {
   int32_t unit_end[kDenseMaxProblems]; // prefix sums of each problem's units
 };
 
+// y of rows row0 .. row0 + nrows - 1 (nrows <= 4) of P for the B activation
+// rows, by one warp with FP32 FMAs.
+template <int B>
+__device__ __forceinline__ void dense_rows(const DenseProblem& P, int row0, int nrows) {
+  constexpr int kDenseBatch = DenseShape<B>::batch;
+  const int lane = threadIdx.x & 31;
+  const int nch = (P.K + 511) / 512;        // chunk rounds of the whole warp
+  float acc[kDenseRows][B];
+#pragma unroll
+  for (int r = 0; r < kDenseRows; ++r)
+#pragma unroll
+    for (int b = 0; b < B; ++b) acc[r][b] = 0.f;
+
+  for (int i0 = 0; i0 < nch; i0 += kDenseBatch) {
+    // weights: one chunk x 4 rows of 16 bytes in flight
+    uint4 w[kDenseRows][kDenseBatch];
+#pragma unroll
+    for (int c = 0; c < kDenseBatch; ++c) {
+      const int k = 16 * (lane + 32 * (i0 + c));
+#pragma unroll
+      for (int r = 0; r < kDenseRows; ++r) {
+        w[r][c] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);   // biased zeros
+        if (k < P.K && r < nrows) {
+          // the row is ldw >= K bytes with ldw % 16 == 0: the 16 bytes at k
+          // lie inside it; bytes at or past K meet a zero activation
+          const uint4 v = ld_weights16(P.W + (int64_t)(row0 + r) * P.ldw + k);
+          w[r][c] = make_uint4(v.x ^ 0x80808080u, v.y ^ 0x80808080u, v.z ^ 0x80808080u,
+                               v.w ^ 0x80808080u);
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < kDenseBatch; ++c) {
+      const int k = 16 * (lane + 32 * (i0 + c));
+      if (k >= P.K) continue;
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        float xv[16];
+        load_x16(P.x + (int64_t)b * P.ldx, k, P.K, xv);
+#pragma unroll
+        for (int r = 0; r < kDenseRows; ++r) {
+          const uint32_t ww[4] = {w[r][c].x, w[r][c].y, w[r][c].z, w[r][c].w};
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            acc[r][b] = fmaf(byte_to_float(ww[e >> 2], (uint32_t)(e & 3)), xv[e], acc[r][b]);
+        }
+      }
+    }
+  }
+  // butterfly over the 32 lanes; every lane ends with the full sums
+#pragma unroll
+  for (int r = 0; r < kDenseRows; ++r)
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) acc[r][b] += __shfl_xor_sync(0xffffffffu, acc[r][b], d);
+#pragma unroll
+  for (int r = 0; r < kDenseRows; ++r)
+#pragma unroll
+    for (int b = 0; b < B; ++b)
+      if (lane == r * B + b && r < nrows)
+        P.y[(int64_t)b * P.ldy + row0 + r] = __fmul_rn(__ldg(P.scale + row0 + r), acc[r][b]);
+}
+
 template <int B>
 __global__ void __launch_bounds__(kDenseThreads, DenseShape<B>::min_ctas)
 dense_kernel(const __grid_constant__ DenseParams p) {
-  constexpr int kDenseBatch = DenseShape<B>::batch;
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31;
   const int nwarps = gridDim.x * (kDenseThreads / 32);
   int j = 0;                                   // problem of the current unit (units ascend)
   for (int u = blockIdx.x * (kDenseThreads / 32) + (threadIdx.x >> 5); u < p.units; u += nwarps) {
     while (u >= p.unit_end[j]) ++j;
     const DenseProblem& P = p.prob[j];
     const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kDenseRows;
-    const int nrows = min(kDenseRows, P.N - row0);
-    const int nch = (P.K + 511) / 512;        // chunk rounds of the whole warp
-    float acc[kDenseRows][B];
-#pragma unroll
-    for (int r = 0; r < kDenseRows; ++r)
-#pragma unroll
-      for (int b = 0; b < B; ++b) acc[r][b] = 0.f;
+    dense_rows<B>(P, row0, min(kDenseRows, P.N - row0));
+  }
+}
 
-    for (int i0 = 0; i0 < nch; i0 += kDenseBatch) {
-      // weights: up to 3 chunks x 4 rows of 16 bytes in flight
-      uint4 w[kDenseRows][kDenseBatch];
+// ---- tensor-core form -----------------------------------------------------------
+constexpr int kMmaRows = 16;                 // weight rows per unit (MMA M)
+constexpr int kMmaChunk = 64;                // weight columns per chunk (16 bytes per lane and row)
+constexpr int kMmaThreads = 512;
+constexpr int kMmaWarps = kMmaThreads / 32;
+constexpr int kMmaRing = 8;                  // chunks in flight per warp (1 KB each)
+
+// activation table: per chunk and 8-column tile, 2 x 32 16-byte groups
+constexpr int kMmaTile = 1024;
+constexpr int kMmaRingBytes = kMmaWarps * kMmaRing * kMmaRows * kMmaChunk;
+constexpr int kMmaTableBytes = 224 * 1024 - kMmaRingBytes;
+
+// d (+)= A B for one 16 x 16 x 8 step (kFirst: d is overwritten).
+template <bool kFirst>
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+  if (kFirst)
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+  else
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void cp_async16(uint4* dst, const int8_t* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Bytes 0 and 2 of w (INT8) as two bf16: 128 + (low 7 bits), whose bf16
+// pattern is 0x4300 | bits, minus 128 (or 256 where the sign bit is set:
+// 0x4380).  Exact.  one28 = 0x43004300, in a register: with the mask as the
+// immediate each and-or is one instruction (as two immediates it is two).
+__device__ __forceinline__ uint32_t bytes02_bf16(uint32_t w, uint32_t one28) {
+  uint32_t m, c, r;
+  asm("lop3.b32 %0, %1, 0x007f007f, %2, 0xEA;" : "=r"(m) : "r"(w), "r"(one28));
+  asm("lop3.b32 %0, %1, 0x00800080, %2, 0xEA;" : "=r"(c) : "r"(w), "r"(one28));
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(m), "r"(c));
+  return r;
+}
+
+// The three bf16 parts of a and b packed as (a, b) pairs: out[0] hi, out[1]
+// mid, out[2] lo.  Each part takes the leading 8 significant bits of what is
+// left (truncation), so the parts sum to the value exactly.
+__device__ __forceinline__ void split3(float a, float b, uint32_t (&out)[3]) {
 #pragma unroll
-      for (int c = 0; c < kDenseBatch; ++c) {
-        const int k = 16 * (lane + 32 * (i0 + c));
+  for (int s = 0; s < 3; ++s) {
+    const uint32_t ua = __float_as_uint(a) & 0xffff0000u, ub = __float_as_uint(b) & 0xffff0000u;
+    out[s] = (ua >> 16) | ub;
+    a = __fsub_rn(a, __uint_as_float(ua));
+    b = __fsub_rn(b, __uint_as_float(ub));
+  }
+}
+
+// The parts of v are exact bf16 values (0, or 2^-100 <= |v| <= 2^100).
+__device__ __forceinline__ bool splits_exactly(float v) {
+  const float a = fabsf(v);
+  return a == 0.f || (a >= 0x1p-100f && a <= 0x1p100f);
+}
+
+struct DenseMmaParams {
+  int32_t count;
+  int32_t table_bytes;                 // shared memory for activation tables
+  uint32_t one28;                      // two bf16 128 (bytes02_bf16)
+  int64_t cost;                        // chunks of all units
+  DenseProblem prob[kDenseMaxProblems];
+  int32_t unit_end[kDenseMaxProblems]; // prefix sums of each problem's 16-row units
+  int64_t cost_end[kDenseMaxProblems]; // prefix sums of each problem's chunks
+};
+
+// The rows of one unit of the tensor-core form with FP32 FMAs.
+template <int B>
+__device__ __forceinline__ void dense_unit_fma(const DenseProblem& P, int row0) {
+  for (int r = row0; r < row0 + kMmaRows && r < P.N; r += kDenseRows)
+    dense_rows<B>(P, r, min(kDenseRows, P.N - r));
+}
+
+template <int B>
+__global__ void __launch_bounds__(kMmaThreads, 1)
+dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
+  constexpr int NT = (B + 1) / 2;      // 8-column MMA tiles: two activation rows each
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint8_t* s_tab = smem + kMmaRingBytes;
+  __shared__ uint8_t s_fma[kDenseMaxProblems];   // problem j0 + i: an activation does not split exactly
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  const uint32_t one28 = p.one28;
+  // this lane's landing slots: each lane reads only what it copied
+  uint4* ring = reinterpret_cast<uint4*>(smem) + warp * (64 * kMmaRing) + lane;
+  pdl_launch_dependents();
+
+  // this CTA's units: an equal share of the launch's chunks (a unit belongs
+  // to the CTA that its first chunk falls to)
+  int range[2];
 #pragma unroll
-        for (int r = 0; r < kDenseRows; ++r) {
-          w[r][c] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);   // biased zeros
-          if (k < P.K && r < nrows) {
-            // the row is ldw >= K bytes with ldw % 16 == 0: the 16 bytes at k
-            // lie inside it; bytes at or past K meet a zero activation
-            const uint4 v = ld_weights16(P.W + (int64_t)(row0 + r) * P.ldw + k);
-            w[r][c] = make_uint4(v.x ^ 0x80808080u, v.y ^ 0x80808080u, v.z ^ 0x80808080u,
-                                 v.w ^ 0x80808080u);
-          }
+  for (int e = 0; e < 2; ++e) {
+    const int64_t c = p.cost * ((int)blockIdx.x + e) / (int)gridDim.x;
+    int lo = 0, hi = p.count - 1;      // the problem holding chunk c
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (c < p.cost_end[mid]) hi = mid;
+      else lo = mid + 1;
+    }
+    const int nch = (p.prob[lo].K + kMmaChunk - 1) / kMmaChunk;
+    const int64_t at = c - (lo ? p.cost_end[lo - 1] : 0);
+    const int u = (lo ? p.unit_end[lo - 1] : 0) + (int)((at + nch - 1) / nch);
+    range[e] = min(u, p.unit_end[p.count - 1]);
+  }
+  pdl_wait();
+
+  int j0 = 0;
+  for (int u0 = range[0]; u0 < range[1];) {
+    // ---- a segment: the units of the problems whose tables fit together ----
+    while (u0 >= p.unit_end[j0]) ++j0;
+    int used = 0, j1 = j0;
+    while (j1 < p.count && (j1 == j0 || range[1] > p.unit_end[j1 - 1])) {
+      const bool same = j1 > j0 && p.prob[j1].x == p.prob[j1 - 1].x && p.prob[j1].K == p.prob[j1 - 1].K &&
+                        p.prob[j1].ldx == p.prob[j1 - 1].ldx;
+      if (!same) {
+        const int bytes = (p.prob[j1].K + kMmaChunk - 1) / kMmaChunk * (NT * kMmaTile);
+        if (used + bytes > p.table_bytes) break;
+        used += bytes;
+      }
+      ++j1;
+    }
+    const int u1 = min(range[1], p.unit_end[j1 - 1]);
+
+    bool any_fma = false;
+    // ---- the weight ring: chunks of this warp's units, kMmaRing ahead --------
+    // Units are padded to whole rings, so slot s always holds a chunk s mod
+    // kMmaRing.  Rows past N and columns past K are clamped to the last row and
+    // the row's last 16 bytes: such a row's sums are not written and such a
+    // column meets zero activations.
+    int lu = u0 + warp, lj = j0, lc = 0, lch = 0, lK = 0;
+    const int8_t *q0 = nullptr, *q1 = nullptr;
+    auto open_unit = [&]() {
+      while (lu < u1) {                  // the next unit of this warp that runs here
+        while (lu >= p.unit_end[lj]) ++lj;
+        if (!any_fma || !s_fma[lj - j0]) break;
+        lu += kMmaWarps;
+      }
+      lc = lch = 0;
+      if (lu >= u1) return;
+      const DenseProblem& P = p.prob[lj];
+      const int row = (lu - (lj ? p.unit_end[lj - 1] : 0)) * kMmaRows + g;
+      lK = P.K;
+      lch = (lK + kMmaChunk - 1) / kMmaChunk;
+      q0 = P.W + (int64_t)min(row, P.N - 1) * P.ldw + 16 * t;
+      q1 = P.W + (int64_t)min(row + 8, P.N - 1) * P.ldw + 16 * t;
+    };
+    // slot s of the ring that starts at chunk lc of the open unit
+    auto load = [&](int s) {
+      if (lc + s < lch) {
+        const int over = max(0, (lc + s) * kMmaChunk + 16 * t - (lK - 1) / 16 * 16);
+        cp_async16(ring + 64 * s, q0 + (s * kMmaChunk - over));
+        cp_async16(ring + 64 * s + 32, q1 + (s * kMmaChunk - over));
+      }
+      cp_async_commit();
+      if (s == kMmaRing - 1) {           // the next ring of the unit, or the next unit
+        lc += kMmaRing;
+        q0 += kMmaRing * kMmaChunk;
+        q1 += kMmaRing * kMmaChunk;
+        if (lc >= lch && lch > 0) {
+          lu += kMmaWarps;
+          open_unit();
         }
       }
+    };
+    open_unit();
 #pragma unroll
-      for (int c = 0; c < kDenseBatch; ++c) {
-        const int k = 16 * (lane + 32 * (i0 + c));
-        if (k >= P.K) continue;
+    for (int s = 0; s < kMmaRing; ++s) load(s);
+
+    // ---- the activation tables of the segment --------------------------------
+    for (int i = threadIdx.x; i < kDenseMaxProblems; i += kMmaThreads) s_fma[i] = 0;
+    __syncthreads();
+    int bad = 0;
+    {
+      int base = 0;
+      for (int j = j0; j < j1; ++j) {
+        const DenseProblem& P = p.prob[j];
+        if (j > j0 && P.x == p.prob[j - 1].x && P.K == p.prob[j - 1].K && P.ldx == p.prob[j - 1].ldx) continue;
+        const int nch = (P.K + kMmaChunk - 1) / kMmaChunk;
+        bool exact = true;
+        for (int i = threadIdx.x; i < nch * 4 * B; i += kMmaThreads) {
+          const int tt = i & 3, b = (i >> 2) % B, c = (i >> 2) / B;
+          float x[16];
+          load_x16(P.x + (int64_t)b * P.ldx, c * kMmaChunk + 16 * tt, P.K, x);
+          uint4* dst = reinterpret_cast<uint4*>(s_tab + base + (c * NT + (b >> 1)) * kMmaTile) +
+                       (b & 1) * 16 + tt;
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-          float xv[16];
-          load_x16(P.x + (int64_t)b * P.ldx, k, P.K, xv);
+          for (int h = 0; h < 2; ++h) {
+            // MMAs 2 h and 2 h + 1 of the chunk: columns (0, 2), (1, 3) of each
+            uint32_t o[4][3];
 #pragma unroll
-          for (int r = 0; r < kDenseRows; ++r) {
-            const uint32_t ww[4] = {w[r][c].x, w[r][c].y, w[r][c].z, w[r][c].w};
+            for (int m = 0; m < 2; ++m) {
+              const float* xm = x + 8 * h + 4 * m;
+              split3(xm[0], xm[2], o[2 * m]);
+              split3(xm[1], xm[3], o[2 * m + 1]);
 #pragma unroll
-            for (int e = 0; e < 16; ++e)
-              acc[r][b] = fmaf(byte_to_float(ww[e >> 2], (uint32_t)(e & 3)), xv[e], acc[r][b]);
+              for (int e = 0; e < 4; ++e) exact = exact && splits_exactly(xm[e]);
+            }
+#pragma unroll
+            for (int s = 0; s < 3; ++s)
+              dst[32 * h + 4 * s] = make_uint4(o[0][s], o[1][s], o[2][s], o[3][s]);
           }
         }
+        if (!exact) {
+          bad = 1;
+          s_fma[j - j0] = 1;
+        }
+        base += nch * NT * kMmaTile;
       }
     }
-    // butterfly over the 32 lanes; every lane ends with the full sums
+    any_fma = __syncthreads_or(bad) != 0;
+    if (any_fma) {
+      // rare: those problems (and the ones that share their activations) with
+      // FP32 FMAs; the loops below leave them out
+      if (threadIdx.x == 0)
+        for (int j = j0 + 1; j < j1; ++j)
+          if (p.prob[j].x == p.prob[j - 1].x && p.prob[j].K == p.prob[j - 1].K && p.prob[j].ldx == p.prob[j - 1].ldx)
+            s_fma[j - j0] = s_fma[j - 1 - j0];
+      __syncthreads();
+      for (int u = u0 + warp, j = j0; u < u1; u += kMmaWarps) {
+        while (u >= p.unit_end[j]) ++j;
+        const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kMmaRows;
+        if (s_fma[j - j0]) dense_unit_fma<B>(p.prob[j], row0);
+      }
+      // the ring again, without them
+      cp_async_wait<0>();
+      lu = u0 + warp;
+      lj = j0;
+      open_unit();
+#pragma unroll 1
+      for (int s = 0; s < kMmaRing; ++s) load(s);
+    }
+
+    // ---- the units -------------------------------------------------------------
+    int j = j0, base = 0;
+    for (int u = u0 + warp; u < u1; u += kMmaWarps) {
+      while (u >= p.unit_end[j]) {
+        const DenseProblem &P = p.prob[j], &Q = p.prob[j + 1];
+        if (!(P.x == Q.x && P.K == Q.K && P.ldx == Q.ldx)) {
+          base += (P.K + kMmaChunk - 1) / kMmaChunk * (NT * kMmaTile);
+        }
+        ++j;
+      }
+      if (any_fma && s_fma[j - j0]) continue;
+      const DenseProblem& P = p.prob[j];
+      const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kMmaRows;
+      const int nch = (P.K + kMmaChunk - 1) / kMmaChunk;
+      float run[NT][4];
 #pragma unroll
-    for (int r = 0; r < kDenseRows; ++r)
+      for (int n = 0; n < NT; ++n)
 #pragma unroll
-      for (int b = 0; b < B; ++b)
+        for (int e = 0; e < 4; ++e) run[n][e] = 0.f;
+      const uint4* tab = reinterpret_cast<const uint4*>(s_tab + base) + lane;
+      for (int c0 = 0; c0 < nch; c0 += kMmaRing) {
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) acc[r][b] += __shfl_xor_sync(0xffffffffu, acc[r][b], d);
+        for (int s = 0; s < kMmaRing; ++s) {
+          cp_async_wait<kMmaRing - 1>();   // this lane's copies of the chunk have landed
+          if (c0 + s < nch) {
+            const uint4 w0 = ring[64 * s], w1 = ring[64 * s + 32];
+            const uint32_t wa[4] = {w0.x, w0.y, w0.z, w0.w};
+            const uint32_t wb[4] = {w1.x, w1.y, w1.z, w1.w};
+            const uint4* tc = tab + (c0 + s) * NT * (kMmaTile / 16);
+            float part[NT][4];
 #pragma unroll
-    for (int r = 0; r < kDenseRows; ++r)
+            for (int h = 0; h < 2; ++h) {
+              uint4 bf[NT];
 #pragma unroll
-      for (int b = 0; b < B; ++b)
-        if (lane == r * B + b && r < nrows)
-          P.y[(int64_t)b * P.ldy + row0 + r] = __fmul_rn(__ldg(P.scale + row0 + r), acc[r][b]);
+              for (int n = 0; n < NT; ++n) bf[n] = tc[n * (kMmaTile / 16) + 32 * h];
+#pragma unroll
+              for (int m = 0; m < 2; ++m) {
+                const uint32_t va = wa[2 * h + m], vb = wb[2 * h + m];
+                const uint32_t a0 = bytes02_bf16(va, one28), a1 = bytes02_bf16(vb, one28);
+                const uint32_t a2 = bytes02_bf16(va >> 8, one28), a3 = bytes02_bf16(vb >> 8, one28);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                  const uint32_t b0 = m ? bf[n].z : bf[n].x, b1 = m ? bf[n].w : bf[n].y;
+                  if (h == 0 && m == 0) mma_bf16<true>(part[n], a0, a1, a2, a3, b0, b1);
+                  else mma_bf16<false>(part[n], a0, a1, a2, a3, b0, b1);
+                }
+              }
+            }
+#pragma unroll
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) run[n][e] = __fadd_rn(run[n][e], part[n][e]);
+          }
+          load(s);
+        }
+      }
+      // lanes t = 0, 2 hold hi and mid of activation row 2 n + t / 2, lanes
+      // t = 1, 3 its lo
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float lo = __shfl_xor_sync(0xffffffffu, run[n][2 * e], 1);
+          const float sum = __fadd_rn(run[n][2 * e], __fadd_rn(run[n][2 * e + 1], lo));
+          const int b = 2 * n + (t >> 1), row = row0 + g + 8 * e;
+          if ((t & 1) == 0 && b < B && row < P.N)
+            P.y[(int64_t)b * P.ldy + row] = __fmul_rn(__ldg(P.scale + row), sum);
+        }
+    }
+    __syncthreads();                   // the tables are rebuilt by the next segment
+    u0 = u1;
   }
 }
 
@@ -146,6 +514,20 @@ cudaError_t launch_dense_t(const DenseParams& p, cudaStream_t s) {
   return launch_pdl(dense_kernel<B>, dim3(grid), dim3(kDenseThreads), 0, s, p);
 }
 
+template <int B>
+cudaError_t launch_dense_mma(const DenseMmaParams& p, cudaStream_t s) {
+  static bool attr_done = false;
+  if (!attr_done) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        dense_mma_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes + kMmaTableBytes);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
+  }
+  return launch_pdl(dense_mma_kernel<B>, dim3(g_dense_sms), dim3(kMmaThreads),
+                    (size_t)(kMmaRingBytes + p.table_bytes),
+                    s, p);
+}
+
 }  // namespace
 
 cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream_t s) {
@@ -155,6 +537,43 @@ cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&g_dense_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+  }
+  // The tensor-core form where an activation table fits in shared memory and
+  // the weights outweigh its start (it holds a whole SM, so it cannot start
+  // beside the previous kernel).  us per call, FMAs / tensor cores: one row,
+  // 18.9 MB 6.9 / 8.1 and 37.7 MB 12.8 / 11.0; two rows, 8.4 MB 5.1 / 5.7 and
+  // 13.1 MB 10.1 / 7.5; three rows, 2.1 MB 4.1 / 4.7 and 4.7 MB 5.7 / 5.5; four
+  // rows, 0.5 MB 3.7 / 4.1 and 2.1 MB 4.9 / 4.6.
+  constexpr int64_t kMmaMinBytes[SPIKE_PROJ_DENSE_MAX_B] = {24 << 20, 9 << 20, 3 << 20, 3 << 19};
+  int maxK = 0;
+  int64_t bytes = 0;
+  for (int j = 0; j < count; ++j) {
+    maxK = probs[j].K > maxK ? probs[j].K : maxK;
+    bytes += (int64_t)probs[j].N * probs[j].K;
+  }
+  const int table = ceil_div(maxK, kMmaChunk) * ((B + 1) / 2) * kMmaTile;
+  if (table <= kMmaTableBytes && bytes >= kMmaMinBytes[B - 1]) {
+    DenseMmaParams p;
+    p.count = count;
+    p.one28 = 0x43004300u;
+    p.table_bytes = table * 2 <= kMmaTableBytes ? table * 2 : table;
+    int units = 0;
+    int64_t cost = 0;
+    for (int j = 0; j < count; ++j) {
+      const int n = ceil_div(probs[j].N, kMmaRows);
+      p.prob[j] = probs[j];
+      units += n;
+      cost += (int64_t)n * ceil_div(probs[j].K, kMmaChunk);
+      p.unit_end[j] = units;
+      p.cost_end[j] = cost;
+    }
+    p.cost = cost;
+    switch (B) {
+      case 1: return launch_dense_mma<1>(p, s);
+      case 2: return launch_dense_mma<2>(p, s);
+      case 3: return launch_dense_mma<3>(p, s);
+      default: return launch_dense_mma<4>(p, s);
+    }
   }
   DenseParams p;
   p.count = count;

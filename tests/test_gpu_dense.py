@@ -149,6 +149,98 @@ def test_dense_decode_step_shapes_sampled():
         assert np.all(err <= tree_bound(K, s[rows].astype(np.float64), mag, want))
 
 
+# A launch with enough weights takes the tensor-core form; this problem alone
+# (28 MB, the widest K) is above the line, so the odd shapes beside it run there.
+BIG = (4608, 6144)
+BIG4 = (9216, 3072)
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 4])
+def test_dense_tensor_form_edges(B):
+    """The tensor-core form at the edges of its tiles: rows around 16, columns
+    around a 16-byte vector, a 64-column chunk and the 8-chunk ring, rows and
+    columns of a CTA's share across problems with different activations, two
+    problems sharing one activation row, and the widest table."""
+    N0, K0 = BIG if B <= 2 else BIG4
+    shapes = [(1, 1), (15, 15), (16, 16), (17, 17), (33, 63), (7, 64), (31, 65), (48, 511), (16, 512),
+              (50, 513), (100, 1000), (16, K0 - 1), (N0, K0), (5, 48), (3, K0)]
+    probs = []
+    for i, (N, K) in enumerate(shapes):
+        big = N == N0
+        W, x, s, ldw, ldx = case(300 + i, N, K, B, ldw=None if big else (K + 15) // 16 * 16 + 16)
+        probs.append((W, x, s, N, K, ldw, ldx))
+    ys = run(probs, B)
+    again = run(probs, B)
+    rng = synth.rng_for(712, B)
+    for y, y2, (W, x, s, N, K, ldw, ldx) in zip(ys, again, probs):
+        assert np.array_equal(y, y2), "not deterministic"
+        rows = np.arange(N) if N <= 128 else np.sort(rng.choice(N, 128, replace=False))
+        check(y[:, rows], np.ascontiguousarray(W[rows]), x, s[rows], len(rows), K, ldw, f"N={N} K={K} B={B}")
+
+
+@pytest.mark.parametrize("B", [1, 4])
+def test_dense_tensor_form_exact_and_shared(B):
+    """0/1 activations give the spike-gated projection bit for bit, one-hot
+    ones give s_m * W[m][k], with one activation buffer shared by all
+    problems of the launch (as a fused query/key/value call has it)."""
+    K, N0 = 3072, 8400
+    W0, _, s0, ldw, ldx = case(330, N0, K, B)
+    xb = synth.bernoulli(synth.rng_for(713), (B, K), 0.3)
+    x = np.zeros((B, ldx), np.float32)
+    x[:, :K] = xb
+    xd, keep, args = to_dev(x), [], []
+    for lo, hi in ((0, 8000), (8000, 8017), (8017, N0)):
+        y = torch.full((B, hi - lo), float("nan"), device=DEV)
+        Wd, sd = to_dev(np.ascontiguousarray(W0[lo:hi])), to_dev(s0[lo:hi])
+        keep.append((Wd, sd, y, lo, hi))
+        args.append((Wd, ldw, sd, xd, ldx, y, hi - lo, hi - lo, K))
+    sp.spike_proj_dense(args, B)
+    _, want = oracle.project(np.ascontiguousarray(W0[:, :K].T), s0, N0, K, xb, "u8")
+    for _, _, y, lo, hi in keep:
+        assert np.array_equal(y.cpu().numpy(), want[:, lo:hi])
+    x[:] = 0
+    for b in range(B):
+        x[b, (17, 0, 1023, K - 1)[b]] = -0.3
+    xd.copy_(to_dev(x))
+    sp.spike_proj_dense(args, B)
+    for _, _, y, lo, hi in keep:
+        got = y.cpu().numpy()
+        for b in range(B):
+            k = (17, 0, 1023, K - 1)[b]
+            assert np.array_equal(got[b], s0[lo:hi] * (np.float32(-0.3) * W0[lo:hi, k].astype(np.float32)))
+
+
+@pytest.mark.parametrize("B", [1, 3])
+def test_dense_tensor_form_extreme_activations(B):
+    """Activations that three bf16 parts cannot hold (infinite, NaN, subnormal,
+    beyond 2^100) are summed with FP32 FMAs, problem by problem: those
+    problems follow IEEE arithmetic and their neighbours are unaffected."""
+    vals = [float("inf"), float("-inf"), float("nan"), 1e-40, 3e-38, 1e31, 2.0 ** -100, 2.0 ** 100, 1e-44]
+    N0, K0 = BIG if B <= 2 else BIG4
+    probs = []
+    for i, v in enumerate(vals):
+        W, x, s, ldw, ldx = case(350 + i, 40, 200, B)
+        x[B - 1, 77] = v
+        if abs(v) < 1e-30:
+            x[B - 1, :200] = v                     # every activation of the row tiny
+        probs.append((W, x, s, 40, 200, ldw, ldx))
+        W, x, s, ldw, ldx = case(370 + i, 20, 100, B)
+        probs.append((W, x, s, 20, 100, ldw, ldx))
+    W, x, s, ldw, ldx = case(390, N0, K0, B)
+    probs.append((W, x, s, N0, K0, ldw, ldx))
+    ys = run(probs, B)
+    for y, (W, x, s, N, K, ldw, ldx) in zip(ys[:-1], probs[:-1]):
+        with np.errstate(invalid="ignore", over="ignore"):
+            want = (x[:, None, :K].astype(np.float64) * W[None, :, :K]).sum(-1) * s
+            mag = np.abs(x[:, None, :K].astype(np.float64) * W[None, :, :K]).sum(-1)
+        fine = np.isfinite(want)
+        assert np.array_equal(np.isnan(want), np.isnan(y))
+        assert np.array_equal(want[~fine & ~np.isnan(want)], y[~fine & ~np.isnan(want)])
+        # each product and sum near the subnormals may lose 2^-149 once more
+        bound = tree_bound(K, s.astype(np.float64), mag, want) + K * 2.0 ** -149
+        assert np.all(np.abs(y - want)[fine] <= bound[fine])
+
+
 def test_dense_errors():
     W = torch.zeros(16, 32, dtype=torch.int8, device=DEV)
     s = torch.ones(16, device=DEV)
