@@ -1,5 +1,5 @@
 // sp_head.cu -- vocabulary head with INT8 activations and candidate-row
-// verification (Section 5, trace configuration; Appendix D), one launch per
+// verification (Section 5, trace configuration; Appendix D), two launches per
 // call for up to 4 hidden states:
 //
 //   1. s_x = max(max_k |h_k|, 1e-8) / 127, q_k = clip(rint(h_k / s_x), +-127)
@@ -20,28 +20,41 @@
 // usual FP32 dot-product bound of the exact value.
 //
 // Layout of the work.  The weights stream from HBM once (V * K bytes) and
-// dominate the traffic, so the kernel is HBM-bound.  Every CTA builds the
-// INT8 codes of all hidden states in shared memory.  A warp owns units of 4
-// consecutive rows; lane l reads the 16-byte chunks l, l + 32, ... of each
-// row and accumulates __dp4a products with the codes.  Each z becomes a
-// 64-bit key (z's order-preserving bits, then the complement of the row, so
-// that one unsigned comparison orders by z descending and row ascending;
-// keys are distinct) and the warp keeps its best 64 keys in a sorted list
-// (bitonic sort of 32 new keys, then a bitonic merge with the list).
+// dominate the traffic.  Projection (head_kernel, one 512-thread CTA per SM):
+// every CTA builds the INT8 codes of all hidden states in shared memory.  A
+// pair of warps owns units of 16 consecutive rows, each warp half of the
+// unit's 64-column chunks: lane (g, t) copies 16 bytes of rows g and g + 8
+// with cp.async into its own slots of a 6-chunk ring (96 KB in flight per SM,
+// no barrier and no registers held by loads) and reads them back itself.  One
+// hidden state takes __dp4a; several take mma.sync m16n8k32 on INT8 with the
+// weights as A and the states as B, so that a weight byte is read from shared
+// memory once whatever B.  (Units of whole rows per warp left the last of 1.5
+// rounds to half the warps: 8 us of 29; halves make about three rounds.)  A
+// per-B dp4a form cost 61 us at B = 4: 128 registers, 16 warps, and 80
+// shuffles and 4 list insertions per 4 rows.
 //
-// Every key of the final 64 is in some CTA's list, so the CTA lists are all
-// that the selection reads.  Each projection CTA merges its 8 warp lists in
-// shared memory (a tree of pairwise bitonic merges), writes one list to the
-// workspace, and counts the list's keys in a 4096-bin histogram of their 12
-// leading order bits.  A second kernel, one CTA launched as the programmatic
-// dependent of the first, takes as a lower bound T the histogram bin that
-// holds the 64th best listed key, and in the same round of loads the first
-// 4 keys of every list.  The keys >= T (about seventy) are gathered (the
-// rest of a list is fetched only when all 4 of its leading keys pass),
-// ordered by counting, gated, and the candidates recomputed, 4 rows per warp
-// with all their loads in flight.  The projection kernel has little shared
-// memory and no clusters: a larger shared-memory carve-out or a cluster
-// launch slowed its weight stream.
+// Each z becomes a 64-bit key (z's order-preserving bits, then the complement
+// of the row, so that one unsigned comparison orders by z descending and row
+// ascending; keys are distinct).  A pair keeps its best 64 keys: the first 64
+// as they come (a vocabulary of 57,344 has 48 rows per pair, and sorting
+// them cost 8 us a call at B = 4), later ones by a bitonic sort and merge.
+// At the end every list goes to the workspace, and the 8 best keys of each
+// CTA beside it.
+//
+// Selection (head_select_kernel, a cluster of 4 CTAs per hidden state, the
+// programmatic dependent of the projection): the bound T is the 64th largest
+// of the CTAs' best keys; the leading keys >= T (about eighty) are gathered
+// (the lists of a CTA are fetched only when all 8 of its leading keys pass),
+// ordered by counting, gated, and the candidates recomputed, two rows per
+// warp.  Its CTAs are small enough in registers, shared memory and carve-out
+// to run beside a projection CTA: the next call's projection starts while
+// the selection runs, and a projection CTA that had to wait for a
+// selection's SM held up the call by 7 us.
+//
+// Measured on 57,344 x 1536, back to back with three weight copies, us a call:
+// gate closed 21.7 (22.0 before this form: the weights 14 of it, the codes
+// 1.3, the selection and the two hand-offs 6), every call verified 24.9 (26.0);
+// four states, every call verified 30.7 (60.6); two states 27.9 (39.8).
 #include "sp_internal.h"
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
@@ -50,29 +63,37 @@
 namespace sp {
 namespace {
 
-constexpr int kHeadThreads = 256;
+constexpr int kHeadThreads = 512;
 constexpr int kHeadWarps = kHeadThreads / 32;
-constexpr int kHeadRows = 4;                  // rows per unit (one warp)
-constexpr int kHeadList = SPIKE_PROJ_HEAD_MAX_CAND;   // keys per sorted list
-constexpr int kSelThreads = 512;              // threads of the selection CTA
+constexpr int kHeadRegs = 80;                 // registers per thread: the selection's CTAs fit beside the projection's
+constexpr int kHeadRows = 16;                 // rows per unit (a pair of warps)
+constexpr int kHeadChunk = 64;                // columns of one ring slot (a 16-byte vector of two rows per lane)
+constexpr int kHeadRing = 6;                  // slots in flight per warp (1 KB each)
+constexpr int kCodePad = 64;                  // bytes between the states' codes (their reads then miss each other's banks)
+constexpr size_t kHeadRingBytes = (size_t)kHeadWarps * kHeadRing * kHeadRows * kHeadChunk;
+constexpr int kHeadLists = kHeadWarps / 2;    // lists of a projection CTA (one per pair of warps)
+constexpr int kHeadList = SPIKE_PROJ_HEAD_MAX_CAND;   // keys per list
+constexpr int kHeadMaxGrid = 160;             // projection CTAs of one call
+constexpr int kSelThreads = 256;              // threads of a selection CTA
 constexpr int kSelWarps = kSelThreads / 32;
-constexpr int kLead = 4;                      // leading keys of each list read first
-constexpr int kHistBits = 12;                 // histogram bins: the keys' leading order bits
-constexpr int kHistWords = 1 << kHistBits;    // bins of one hidden state
-constexpr int kHeadMaxGrid = 1024;            // projection CTAs (lists) of one call
+constexpr int kSelCluster = 4;                // selection CTAs of one hidden state
+constexpr int kCtaLead = 8;                   // leading keys of each projection CTA read first
+constexpr int kSelCand = 512;                 // keys that the bound may pass
+constexpr int kSelLong = 16;                  // projection CTAs read in full
 static_assert(kHeadList == 64, "a list is two keys per lane");
-static_assert(SPIKE_PROJ_HEAD_MAX_K % (4 * 256) == 0, "the codes phase covers K in float4 per thread");
-static_assert(kSelThreads * 8 == kHistWords, "hist_bound: 8 bins per selection thread");
-static_assert(kHeadList == 4 * kSelWarps, "four candidates per selection warp");
+static_assert(kHeadRingBytes + SPIKE_PROJ_HEAD_MAX_B * (SPIKE_PROJ_HEAD_MAX_K + kCodePad) <= 212 * 1024, "shared memory per CTA");
+static_assert((size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadLists * kHeadList * 8 <= kHeadRingBytes, "the lists fit the ring");
+static_assert(kHeadLists * kCtaLead == 64, "the pairs' leading keys: two per lane of one warp");
+static_assert(kHeadMaxGrid <= kSelThreads, "one projection CTA per selection thread");
+static_assert(kHeadList == 2 * kSelWarps * kSelCluster, "two candidates per selection warp");
 
 typedef unsigned long long hkey;
 
-// Workspace: the CTA lists (projection CTA c's list of hidden state b is
-// list b * nlists + c), then per hidden state the histogram of the listed
-// keys' 12 leading order bits (4096 bins, an eighth of an octave of z
-// each), zero between calls.
-constexpr size_t kListBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadMaxGrid * kHeadList * 8;
-constexpr size_t kHistBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHistWords * 4;
+// Workspace: the lists (pair q of projection CTA c, hidden state b: list
+// (b * nctas + c) * kHeadLists + q), then each CTA's leading keys; all of it
+// is rewritten by every call.
+constexpr size_t kListBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadMaxGrid * kHeadLists * kHeadList * 8;
+constexpr size_t kLeadBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadMaxGrid * kCtaLead * 8;
 
 struct HeadParams {
   const int8_t* W;
@@ -91,9 +112,9 @@ struct HeadParams {
   float* z;
   int64_t ld_z;
   int32_t B;
-  hkey* lists;             // one 64-key list per projection CTA and hidden state
-  uint32_t* hist;          // [B][kHistWords]
-  int32_t nlists;          // CTAs of the projection kernel
+  hkey* lists;             // one 64-key list per pair of projection warps and hidden state
+  hkey* lead;              // the kCtaLead best keys of each projection CTA and hidden state
+  int32_t nctas;           // CTAs of the projection kernel
 };
 
 // Order-preserving bits of z (both zeros map to the bits of +0).
@@ -143,33 +164,70 @@ __device__ __forceinline__ void warp_merge64(hkey& a, hkey& b, int lane) {
   }
 }
 
-// List (a, b) <- the best 64 of the list and the 32 keys n (one per lane).
-// For descending A and B of equal length, max(A_i, B_{63-i}) holds the best
-// 64 of both as a bitonic sequence; n is B with 32 empty keys appended.
-__device__ __forceinline__ void list_insert32(hkey& a, hkey& b, hkey n, int lane) {
-  n = warp_sort32(n, lane);
-  b = kmax(b, __shfl_sync(0xffffffffu, n, 31 - lane));
+// The 64 keys of (a, b), any order, sorted descending.
+__device__ __forceinline__ void sort64(hkey& a, hkey& b, int lane) {
+  a = warp_sort32(a, lane);
+  b = __shfl_sync(0xffffffffu, warp_sort32(b, lane), 31 - lane);   // descending, then ascending: bitonic
   warp_merge64(a, b, lane);
 }
 
-// Merges the n sorted lists s[0 .. n) (64 keys each, in shared memory) in
-// place, pairwise by the CTA's nw warps; the result is s[0].  Every thread
-// calls it.
-__device__ void tree_merge(hkey* s, int n, int nw) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int stride = 1; stride < n; stride <<= 1) {
-    for (int q = warp; q * 2 * stride + stride < n; q += nw) {
-      hkey* A = s + (size_t)(q * 2 * stride) * kHeadList;
-      const hkey* Bl = A + (size_t)stride * kHeadList;
-      hkey a = kmax(A[lane], Bl[63 - lane]);
-      hkey b = kmax(A[32 + lane], Bl[31 - lane]);
-      warp_merge64(a, b, lane);
-      __syncwarp();
-      A[lane] = a;
-      A[32 + lane] = b;
-    }
-    __syncthreads();
+// The kCtaLead largest of the 64 keys of (a, b), any order: lane r < kCtaLead
+// gets the r-th (the warp's maximum by two integer reductions each time).
+__device__ __forceinline__ hkey best_of64(hkey a, hkey b, int lane) {
+  hkey mine = 0ull;
+#pragma unroll
+  for (int r = 0; r < kCtaLead; ++r) {
+    const hkey m = kmax(a, b);
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(m >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(m >> 32) == hi ? (uint32_t)m : 0u);
+    const hkey best = (hkey)hi << 32 | lo;
+    if (lane == r) mine = best;
+    if (a == best) a = 0ull;                     // keys are distinct, the empty one apart
+    else if (b == best) b = 0ull;
   }
+  return mine;
+}
+
+// List (a, b) <- the best 64 of the list and the 32 keys n (one per lane), the
+// insert number `held`.  The first 64 keys stay as they come; from the third
+// insert on the list is kept sorted, and 32 keys below its last one are
+// dropped at once.  For descending A and B of equal length, max(A_i, B_{63-i})
+// holds the best 64 of both as a bitonic sequence; n is B with 32 empty keys
+// appended.
+__device__ __forceinline__ void list_add32(hkey& a, hkey& b, hkey n, int held, int lane) {
+  if (held == 0) {
+    a = n;
+  } else if (held == 1) {
+    b = n;
+  } else {
+    if (held == 2) sort64(a, b, lane);
+    if (!__any_sync(0xffffffffu, n > __shfl_sync(0xffffffffu, b, 31))) return;
+    n = warp_sort32(n, lane);
+    b = kmax(b, __shfl_sync(0xffffffffu, n, 31 - lane));
+    warp_merge64(a, b, lane);
+  }
+}
+
+// (a, b) <- the best 64 of the two sorted lists (a, b) and (c, d), sorted.
+__device__ __forceinline__ void list_merge(hkey& a, hkey& b, hkey c, hkey d, int lane) {
+  a = kmax(a, __shfl_sync(0xffffffffu, d, 31 - lane));
+  b = kmax(b, __shfl_sync(0xffffffffu, c, 31 - lane));
+  warp_merge64(a, b, lane);
+}
+
+// Keys of buf[0 .. C) above k.
+__device__ __forceinline__ int count_larger(const hkey* buf, int C, hkey k) {
+  int larger = 0;
+  int j = 0;
+  for (; j + 8 <= C; j += 8) {                   // 8 loads in flight
+    hkey v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = buf[j + e];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) larger += v[e] > k;
+  }
+  for (; j < C; ++j) larger += buf[j] > k;
+  return larger;
 }
 
 // out[0 .. 64) <- the best min(C, 64) of the C distinct keys buf[0 .. C),
@@ -178,72 +236,25 @@ __device__ void rank_place(const hkey* buf, int C, hkey* out) {
   const int t = threadIdx.x, nt = blockDim.x;
   for (int i = C + t; i < kHeadList; i += nt) out[i] = 0ull;
   for (int i = t; i < C; i += nt) {
-    const hkey ki = buf[i];
-    int larger = 0;
-    int j = 0;
-    for (; j + 8 <= C; j += 8) {                 // 8 loads in flight
-      hkey v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = buf[j + e];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) larger += v[e] > ki;
-    }
-    for (; j < C; ++j) larger += buf[j] > ki;
-    if (larger < kHeadList) out[larger] = ki;
+    const int larger = count_larger(buf, C, buf[i]);
+    if (larger < kHeadList) out[larger] = buf[i];
   }
   __syncthreads();
 }
 
-// The lower bound of the leading order bits of the histogram bin that holds
-// the need-th largest key, from a kHistWords-bin histogram (bin i counts the
-// keys whose leading bits are i): thread t of a kSelThreads-thread CTA holds
-// bins 8t .. 8t + 7 in c (loaded by the caller, so that the loads can be in
-// flight with others), and the suffix sums meet in two barriers.  0 when
-// the histogram holds fewer than need keys.  Every thread calls it.
-__device__ uint32_t hist_bound(const uint32_t (&c)[8], uint32_t need, uint32_t* s_wtot,
-                               uint32_t& s_bin) {
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  uint32_t sum = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) sum += c[i];
-  uint32_t S = sum;                              // keys in the bins of lanes >= this one
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t o = __shfl_down_sync(0xffffffffu, S, d);
-    if (lane + d < 32) S += o;
-  }
-  if (lane == 0) s_wtot[warp] = S;
-  if (t == 0) s_bin = 0u;
-  __syncthreads();
-  for (int w = warp + 1; w < (int)(blockDim.x >> 5); ++w) S += s_wtot[w];
-  if (S >= need && S - sum < need) {             // this thread's bins hold the need-th key
-    uint32_t cum = S - sum;
-#pragma unroll
-    for (int i = 7; i >= 0; --i) {
-      if (cum + c[i] >= need) {
-        s_bin = (uint32_t)(8 * t + i) << (32 - kHistBits);
-        break;
-      }
-      cum += c[i];
-    }
-  }
-  __syncthreads();
-  return s_bin;
-}
-
-// r of up to 4 candidate rows (rows[j], j < n) for hidden state hb, by one
+// r of up to 2 candidate rows (rows[j], j < n) for hidden state hb, by one
 // warp: per row, lane l sums the 16-byte chunks l, l + 32, ... in ascending k
 // with fmaf, then the 5-level butterfly (the continuous-input kernel's
 // order); the loads of all the rows and of up to 4 chunks are in flight
 // together.
-__device__ __forceinline__ void verify_rows4(const HeadParams& p, const float* hb, const int (&rows)[4],
-                                             int n, int lane, float (&out)[4]) {
+__device__ __forceinline__ void verify_rows2(const HeadParams& p, const float* hb, const int (&rows)[2],
+                                             int n, int lane, float (&out)[2]) {
   const int nch = (p.K + 511) / 512;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  float acc[2] = {0.f, 0.f};
   for (int c0 = 0; c0 < nch; c0 += 4) {
-    uint4 v[4][4];
+    uint4 v[2][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const int k = 16 * (lane + 32 * (c0 + t));
@@ -256,7 +267,7 @@ __device__ __forceinline__ void verify_rows4(const HeadParams& p, const float* h
         float x[16];
         load_x16(hb, k, p.K, x);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < 2; ++j) {
           if (j < n) {
             const uint32_t ww[4] = {v[j][t].x ^ 0x80808080u, v[j][t].y ^ 0x80808080u,
                                     v[j][t].z ^ 0x80808080u, v[j][t].w ^ 0x80808080u};
@@ -269,374 +280,459 @@ __device__ __forceinline__ void verify_rows4(const HeadParams& p, const float* h
     }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < 2; ++j) {
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], d);
     out[j] = j < n ? __fmul_rn(__ldg(p.scale + rows[j]), acc[j]) : 0.f;
   }
 }
 
-// Step 1 for every hidden state: thread t holds h[4t + 1024 i .. +3], i < NV,
-// in registers (one read of h); the CTA's maximum |h| meets in one barrier
-// and every thread derives s_x; the codes go to shared memory four to a word.
-template <int B, int NV>
+// Step 1: the CTA's warps are dealt out over the hidden states (kHeadThreads /
+// G threads each, G = B rounded up to a power of two); each group finds its
+// state's maximum |h|, and after one barrier every thread derives s_x and
+// writes codes four to a word, zero from K to Kpad.  h is read again for the
+// codes (from L1): kept in registers it made the code larger, and as the code
+// runs once per CTA its size showed (2.3 us instead of 1.3).
+template <int B>
 __device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes, float* s_red, float* s_sx) {
+  constexpr int G = B == 1 ? 1 : B == 2 ? 2 : 4;
+  constexpr int T = kHeadThreads / G;            // threads of one hidden state
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll 1
-  for (int b = 0; b < B; ++b) {
-    const float* hb = p.h + (int64_t)b * p.ldh;
-    float4 hv[NV];
-    float mx = 0.f;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int k = 4 * (int)threadIdx.x + 4 * kHeadThreads * i;
-      hv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k + 4 <= p.K) {
-        hv[i] = __ldg(reinterpret_cast<const float4*>(hb + k));   // h 16-byte aligned, ldh % 4 == 0
-      } else if (k < p.K) {
-        hv[i].x = hb[k];
-        if (k + 1 < p.K) hv[i].y = hb[k + 1];
-        if (k + 2 < p.K) hv[i].z = hb[k + 2];
-      }
-      mx = fmaxf(mx, fmaxf(fmaxf(fabsf(hv[i].x), fabsf(hv[i].y)), fmaxf(fabsf(hv[i].z), fabsf(hv[i].w))));
+  const int b = (int)threadIdx.x / T, tt = (int)threadIdx.x % T;
+  const float* hb = p.h + (int64_t)(b < B ? b : 0) * p.ldh;
+  const auto load4 = [&](int k) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k + 4 <= p.K) {
+      v = __ldg(reinterpret_cast<const float4*>(hb + k));   // h 16-byte aligned, ldh % 4 == 0
+    } else if (k < p.K) {
+      v.x = __ldg(hb + k);
+      if (k + 1 < p.K) v.y = __ldg(hb + k + 1);
+      if (k + 2 < p.K) v.z = __ldg(hb + k + 2);
     }
+    return v;
+  };
+  const auto pack = [&](const float4& v, int k, float sx) {
+    const float e[4] = {v.x, v.y, v.z, v.w};
+    uint32_t packed = 0;
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-    if (lane == 0) s_red[warp] = mx;
-    __syncthreads();
-    float a = s_red[0];
-#pragma unroll
-    for (int w = 1; w < kHeadWarps; ++w) a = fmaxf(a, s_red[w]);
-    const float sx = __fdiv_rn(fmaxf(a, 1e-8f), 127.0f);
-    if (threadIdx.x == 0) s_sx[b] = sx;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int k = 4 * (int)threadIdx.x + 4 * kHeadThreads * i;
-      if (k < p.Kpad) {
-        const float e[4] = {hv[i].x, hv[i].y, hv[i].z, hv[i].w};
-        uint32_t packed = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int c = 0;
-          if (k + j < p.K) c = (int)fminf(fmaxf(rintf(__fdiv_rn(e[j], sx)), -127.0f), 127.0f);
-          packed |= ((uint32_t)c & 0xffu) << (8 * j);
-        }
-        *reinterpret_cast<uint32_t*>(s_codes + b * p.Kpad + k) = packed;
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int c = k + j < p.K ? (int)fminf(fmaxf(rintf(__fdiv_rn(e[j], sx)), -127.0f), 127.0f) : 0;
+      packed |= ((uint32_t)c & 0xffu) << (8 * j);
     }
-    __syncthreads();                             // s_red is rewritten by the next hidden state
+    *reinterpret_cast<uint32_t*>(s_codes + b * (p.Kpad + kCodePad) + k) = packed;
+  };
+  float mx = 0.f;
+#pragma unroll 4
+  for (int k = 4 * tt; k < p.K; k += 4 * T) {
+    const float4 v = load4(k);
+    mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
   }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+  if (lane == 0) s_red[warp] = mx;
+  __syncthreads();
+  float a = s_red[b * (T / 32)];
+#pragma unroll
+  for (int w = 1; w < T / 32; ++w) a = fmaxf(a, s_red[b * (T / 32) + w]);
+  const float sx = __fdiv_rn(fmaxf(a, 1e-8f), 127.0f);
+  if (b < B) {
+    if (tt == 0) s_sx[b] = sx;
+#pragma unroll 1
+    for (int k = 4 * tt; k < p.Kpad; k += 4 * T) pack(load4(k), k, sx);
+  }
+  __syncthreads();
 }
 
-template <int B> struct HeadShape { static constexpr int min_ctas = 2; };
-template <> struct HeadShape<1> { static constexpr int min_ctas = 4; };
+__device__ __forceinline__ void cp_async16(uint4* dst, const int8_t* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// d += A B for 16 rows x 32 columns of weights and 32 columns of 8 states.
+__device__ __forceinline__ void mma_s8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                       uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
 
 // Steps 1-2 and the CTA's lists.
 template <int B>
-__global__ void __launch_bounds__(kHeadThreads, HeadShape<B>::min_ctas)
+__global__ void __maxnreg__(kHeadRegs)
 head_kernel(const __grid_constant__ HeadParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  hkey* s_all = reinterpret_cast<hkey*>(smem);             // [8][64]
-  int8_t* s_codes = reinterpret_cast<int8_t*>(s_all + kHeadWarps * kHeadList);   // [B][Kpad]
+  uint4* s_ring = reinterpret_cast<uint4*>(smem);          // [warp][slot][2][32 lanes]
+  int8_t* s_codes = reinterpret_cast<int8_t*>(smem + kHeadRingBytes);   // [B][Kpad]
   __shared__ float s_red[kHeadWarps];
   __shared__ float s_sx[B];
+  __shared__ hkey s_lead[B][kHeadLists * kCtaLead];
+  __shared__ int4 s_sum[2][kHeadWarps / 2][32];
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = gridDim.x * kHeadWarps;
-  const int wg = blockIdx.x * kHeadWarps + warp;
-  // The weights are constant (no kernel writes them): the rows of this warp's
-  // first unit are prefetched into L2 before the dependency wait.
-  if (wg < p.units) {
-    for (int r = 0; r < kHeadRows; ++r) {
-      const int row = wg * kHeadRows + r;
-      if (row >= p.V) break;
-      for (int off = lane * 128; off < p.K; off += 32 * 128)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p.W + (int64_t)row * p.ldw + off));
+  const int g = lane >> 2, t = lane & 3;
+  const int nch = p.Kpad / kHeadChunk;
+  // this lane's codes: of the one state, or of the MMA column g (any state for
+  // the columns past B)
+  const int8_t* codes = s_codes + (B == 1 ? 0 : g % B) * (p.Kpad + kCodePad) + 16 * t;
+  uint4* ring = s_ring + warp * (kHeadRing * 64) + lane;
+
+  // The weight ring: a pair of warps takes a unit, each warp half of its
+  // chunks, so that the units of a call fill about three rounds (rows past V
+  // and columns past K are clamped: their logits are not kept, their codes
+  // are 0).
+  const int half = warp & 1;
+  const int c0 = half ? (nch + 1) / 2 : 0;                 // this warp's chunks c0 .. c0 + nc - 1
+  const int nc = half ? nch / 2 : (nch + 1) / 2;
+  const int nslot = max(nc, kHeadRing);                    // ring slots of a unit: the loader is at most one unit ahead
+  const int first = (warp >> 1) * (int)gridDim.x + (int)blockIdx.x;
+  const int stride = (int)gridDim.x * (kHeadWarps / 2);
+  int lu = first, lc = 0, lslot = 0;                       // the loader's unit, chunk and slot
+  const int last16 = (p.K - 1) / 16 * 16;
+  const int8_t *lrow0, *lrow1;                             // this lane's rows of the loader's unit
+  const auto open_unit = [&]() {
+    lrow0 = p.W + (int64_t)min(lu * kHeadRows + g, p.V - 1) * p.ldw;
+    lrow1 = p.W + (int64_t)min(lu * kHeadRows + g + 8, p.V - 1) * p.ldw;
+  };
+  open_unit();
+  const auto load = [&]() {
+    if (lu < p.units && lc < nc) {
+      const int k = min((c0 + lc) * kHeadChunk + 16 * t, last16);
+      uint4* dst = ring + lslot * 64;
+      cp_async16(dst, lrow0 + k);
+      cp_async16(dst + 32, lrow1 + k);
     }
-  }
+    cp_async_commit();
+    if (++lslot == kHeadRing) lslot = 0;
+    if (++lc == nslot) {                                   // on to the next unit
+      lc = 0;
+      lu += stride;
+      open_unit();
+    }
+  };
+  // The first ring is issued before the dependency wait: of the kernels that
+  // may still be running then (those of this library, which alone let their
+  // successors start early) none writes the weights, and whatever else may
+  // have written them on the stream has completed.
+#pragma unroll 1
+  for (int s = 0; s < kHeadRing; ++s) load();
   pdl_wait();
+  // One state: the selection's CTAs fit beside this kernel's; resident early,
+  // they start as soon as the last list is written (with several states they
+  // come after the weight stream, below: 30 against 32 us a call for four).
+  if constexpr (B == 1) pdl_launch_dependents();
 
-  // 1. activation scale and INT8 codes of each hidden state (zero past K);
-  // a compact form for K <= 2048 (the code runs once per CTA, and its size
-  // shows in the start-up)
-  if (p.K <= 2 * 4 * kHeadThreads) head_codes<B, 2>(p, s_codes, s_red, s_sx);
-  else head_codes<B, SPIKE_PROJ_HEAD_MAX_K / (4 * kHeadThreads)>(p, s_codes, s_red, s_sx);
+  // 1. activation scale and INT8 codes of each hidden state
+  head_codes<B>(p, s_codes, s_red, s_sx);
 
-  // 2. approximate logits; each warp keeps its best 64 keys per hidden state
+  // 2. approximate logits; the even warp of each pair keeps the pair's best 64
+  // keys per hidden state
   hkey la[B], lb[B], pend[B];
 #pragma unroll
   for (int b = 0; b < B; ++b) la[b] = lb[b] = pend[b] = 0ull;
-  int slot = 0;                                  // units since the last insert
-  const int nch = (p.K + 511) / 512;
-  for (int u = wg; u < p.units; u += nwarps) {
-    const int row0 = u * kHeadRows;
-    const int nrows = min(kHeadRows, p.V - row0);
-    int acc[kHeadRows][B];
-#pragma unroll
-    for (int r = 0; r < kHeadRows; ++r)
-#pragma unroll
-      for (int b = 0; b < B; ++b) acc[r][b] = 0;
-    for (int c = 0; c < nch; ++c) {
-      const int k = 16 * (lane + 32 * c);
-      if (k >= p.K) continue;
-      // the row is ldw >= K bytes with ldw % 16 == 0: the 16 bytes at k lie
-      // inside it; bytes at or past K meet zero codes
-      uint4 w[kHeadRows];
-#pragma unroll
-      for (int r = 0; r < kHeadRows; ++r)
-        w[r] = r < nrows ? ld_weights16(p.W + (int64_t)(row0 + r) * p.ldw + k) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-      for (int b = 0; b < B; ++b) {
-        const uint4 q = *reinterpret_cast<const uint4*>(s_codes + b * p.Kpad + k);
-#pragma unroll
-        for (int r = 0; r < kHeadRows; ++r) {
-          int a = acc[r][b];
-          a = __dp4a((int)w[r].x, (int)q.x, a);
-          a = __dp4a((int)w[r].y, (int)q.y, a);
-          a = __dp4a((int)w[r].z, (int)q.z, a);
-          a = __dp4a((int)w[r].w, (int)q.w, a);
-          acc[r][b] = a;
+  int nu = 0;                                    // units since the last insert
+  int held = 0;                                  // inserts
+  int cslot = 0, buf = 0;
+  for (int u = first; u < p.units; u += stride) {
+    const int row0 = u * kHeadRows + g, row1 = row0 + 8;
+    const float sc0 = __ldg(p.scale + min(row0, p.V - 1)), sc1 = __ldg(p.scale + min(row1, p.V - 1));
+    // one state: each lane's share of rows g, g + 8; several: the MMA's
+    // accumulators (state 2 t + e of row g + 8 h in acc[2 h + e])
+    int acc[4] = {0, 0, 0, 0};
+#pragma unroll 1
+    for (int c = 0; c < nslot; ++c) {
+      cp_async_wait<kHeadRing - 1>();            // this lane's copies of the chunk have landed
+      if (c < nc) {
+        const uint4 w0 = ring[cslot * 64], w1 = ring[cslot * 64 + 32];
+        const uint4 q = *reinterpret_cast<const uint4*>(codes + (c0 + c) * kHeadChunk);
+        if constexpr (B == 1) {
+          acc[0] = __dp4a((int)w0.x, (int)q.x, acc[0]);
+          acc[1] = __dp4a((int)w1.x, (int)q.x, acc[1]);
+          acc[0] = __dp4a((int)w0.y, (int)q.y, acc[0]);
+          acc[1] = __dp4a((int)w1.y, (int)q.y, acc[1]);
+          acc[0] = __dp4a((int)w0.z, (int)q.z, acc[0]);
+          acc[1] = __dp4a((int)w1.z, (int)q.z, acc[1]);
+          acc[0] = __dp4a((int)w0.w, (int)q.w, acc[0]);
+          acc[1] = __dp4a((int)w1.w, (int)q.w, acc[1]);
+        } else {
+          mma_s8(acc, w0.x, w1.x, w0.y, w1.y, q.x, q.y);
+          mma_s8(acc, w0.z, w1.z, w0.w, w1.w, q.z, q.w);
         }
+      }
+      if (++cslot == kHeadRing) cslot = 0;
+      load();
+    }
+    // the halves meet: the odd warp hands its sums to the even one (two
+    // buffers: a buffer is written again only after the even warp has reached
+    // the next unit's barrier)
+    int4* sum = &s_sum[buf][warp >> 1][lane];
+    buf ^= 1;
+    if (half) *sum = make_int4(acc[0], acc[1], acc[2], acc[3]);
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp >> 1)) : "memory");
+    if (half) continue;
+    {
+      const int4 o = *sum;
+      acc[0] += o.x;
+      acc[1] += o.y;
+      acc[2] += o.z;
+      acc[3] += o.w;
+    }
+    if constexpr (B == 1) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], 1);
+        acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], 2);
       }
     }
 #pragma unroll
-    for (int r = 0; r < kHeadRows; ++r)
-#pragma unroll
-      for (int b = 0; b < B; ++b)
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) acc[r][b] += __shfl_xor_sync(0xffffffffu, acc[r][b], d);
-#pragma unroll
-    for (int r = 0; r < kHeadRows; ++r) {
-      if (r < nrows) {
-        const float s = __ldg(p.scale + row0 + r);
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-          const float zv = __fmul_rn(s, __fmul_rn(s_sx[b], __int2float_rn(acc[r][b])));
-          if (p.z && lane == r * B + b) p.z[(int64_t)b * p.ld_z + row0 + r] = zv;
-          if (lane == slot * kHeadRows + r) pend[b] = make_key(zv, row0 + r);
-        }
+    for (int b = 0; b < B; ++b) {
+      int a0 = acc[0], a1 = acc[1];
+      if constexpr (B > 1) {
+        const int src = (lane & ~3) | (b >> 1);
+        a0 = __shfl_sync(0xffffffffu, acc[b & 1], src);
+        a1 = __shfl_sync(0xffffffffu, acc[2 + (b & 1)], src);
       }
+      const float z0 = __fmul_rn(sc0, __fmul_rn(s_sx[b], __int2float_rn(a0)));
+      const float z1 = __fmul_rn(sc1, __fmul_rn(s_sx[b], __int2float_rn(a1)));
+      if (p.z && t == b) {
+        float* zb = p.z + (int64_t)b * p.ld_z;
+        if (row0 < p.V) zb[row0] = z0;
+        if (row1 < p.V) zb[row1] = z1;
+      }
+      // lanes t = 0, 1 keep the rows g, g + 8 of the first of two units, lanes
+      // t = 2, 3 those of the second
+      const int row = t & 1 ? row1 : row0;
+      if ((t >> 1) == nu && row < p.V) pend[b] = make_key(t & 1 ? z1 : z0, row);
     }
-    if (++slot == 32 / kHeadRows) {             // 32 pending keys: insert them
+    if (++nu == 2) {                             // 32 pending keys
 #pragma unroll
       for (int b = 0; b < B; ++b) {
-        list_insert32(la[b], lb[b], pend[b], lane);
+        list_add32(la[b], lb[b], pend[b], held, lane);
         pend[b] = 0ull;
       }
-      slot = 0;
+      ++held;
+      nu = 0;
     }
   }
-  if (slot) {
+  if (nu) {
 #pragma unroll
-    for (int b = 0; b < B; ++b) list_insert32(la[b], lb[b], pend[b], lane);
+    for (int b = 0; b < B; ++b) list_add32(la[b], lb[b], pend[b], held, lane);
   }
-  // the selection kernel may become resident once every CTA is here (not
-  // earlier: its CTAs would take slots from the weight stream)
-  pdl_launch_dependents();
-
-  // 3. the CTA's list per hidden state, into the workspace
-#pragma unroll
-  for (int b = 0; b < B; ++b) {
-    s_all[warp * kHeadList + lane] = la[b];
-    s_all[warp * kHeadList + 32 + lane] = lb[b];
+  // 3. every pair's list into the workspace; the CTA's best keys (of the
+  // pairs' best) into its leading keys.  With several states all the warps
+  // share the pairs' lists, through shared memory (the ring is idle).
+  if constexpr (B > 1) {
+    pdl_launch_dependents();
+    cp_async_wait<0>();
     __syncthreads();
-    tree_merge(s_all, kHeadWarps, kHeadWarps);
-    const int64_t slot = (int64_t)b * p.nlists + blockIdx.x;
-    if (threadIdx.x < kHeadList) {
-      const hkey k = s_all[threadIdx.x];
-      __stcg(p.lists + slot * kHeadList + threadIdx.x, k);
-      // the listed keys into the histogram (equal bins of a warp summed
-      // first): every key of the final selection is a listed key
-      const uint32_t real = __ballot_sync(0xffffffffu, k != 0ull);
-      if (k != 0ull) {
-        const uint32_t bin = (uint32_t)(k >> (64 - kHistBits));
-        const uint32_t mb = __match_any_sync(real, bin);
-        if (lane == __ffs(mb) - 1) atomicAdd(p.hist + (int64_t)b * kHistWords + bin, (uint32_t)__popc(mb));
+  }
+  if (!half) {
+    const int pair = warp >> 1;
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      hkey* list = p.lists + (((int64_t)b * p.nctas + blockIdx.x) * kHeadLists + pair) * kHeadList;
+      __stcg(list + lane, la[b]);
+      __stcg(list + 32 + lane, lb[b]);
+      if constexpr (B == 1) {
+        const hkey k = best_of64(la[b], lb[b], lane);
+        if (lane < kCtaLead) s_lead[b][pair * kCtaLead + lane] = k;
+      } else {
+        hkey* mine = reinterpret_cast<hkey*>(smem) + (b * kHeadLists + pair) * kHeadList;
+        mine[lane] = la[b];
+        mine[32 + lane] = lb[b];
       }
     }
+  }
+  __syncthreads();
+  if constexpr (B > 1) {
+    for (int i = warp; i < B * kHeadLists; i += kHeadWarps) {
+      const hkey* list = reinterpret_cast<const hkey*>(smem) + i * kHeadList;
+      const hkey k = best_of64(list[lane], list[32 + lane], lane);
+      if (lane < kCtaLead) s_lead[i / kHeadLists][i % kHeadLists * kCtaLead + lane] = k;
+    }
     __syncthreads();
+  }
+  if (warp < B) {
+    const hkey k = best_of64(s_lead[warp][lane], s_lead[warp][32 + lane], lane);
+    if (lane < kCtaLead) __stcg(p.lead + ((int64_t)warp * p.nctas + blockIdx.x) * kCtaLead + lane, k);
   }
 }
 
-// Steps 3-6, one CTA of kSelThreads threads, per hidden state: the bound T
-// and the leading keys of every list (one round of loads for both), the
-// keys >= T, the best 64 of them by counting, the gate, the candidates
-// recomputed (warp w: candidates w, w + 16, w + 32, w + 48), the token.  When
-// the bound does not narrow the keys to at most kSelThreads (an adversarial
-// spread, e.g. equal logits everywhere), or passes fewer than min(V, 64) (a
-// histogram left dirty by a call that never reached this kernel), every list
-// is merged instead, 15 at a time into a running best 64: slower, and exact
-// either way.
-__global__ void __launch_bounds__(kSelThreads, 1)
+// Steps 3-6, a cluster of kSelCluster CTAs per hidden state.  Every CTA of
+// the cluster makes the same selection: the bound T (the 64th largest of the
+// projection CTAs' best keys, so at least 64 keys reach it), the keys >= T,
+// the best 64 of them by counting, the gate.  A projection CTA whose kCtaLead
+// leading keys all pass may have others in its lists, which are then read in
+// full.  The candidates are shared out (warp w of rank r recomputes 8 r + w
+// and 32 + 8 r + w), their logits meet in rank 0's shared memory, and rank 0
+// picks the token.  When the bound does not narrow the keys to at most
+// kSelCand, or more than kSelLong CTAs would be read in full (an adversarial
+// spread, e.g. equal logits everywhere), the warps merge every list instead:
+// slower, and exact either way.
+__global__ void __launch_bounds__(kSelThreads)
 head_select_kernel(const __grid_constant__ HeadParams p) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  hkey* s_lead = reinterpret_cast<hkey*>(smem);            // [nlists][kLead]; 16 lists when merging
-  __shared__ hkey s_cand[kSelThreads];
+  __shared__ hkey s_cand[kSelCand];
   __shared__ hkey s_best[kHeadList];
+  __shared__ hkey s_merge[kSelWarps][kHeadList];
   __shared__ float s_r[kHeadList];
-  __shared__ int s_long[kSelThreads];
-  __shared__ uint32_t s_wtot[kSelWarps];
-  __shared__ uint32_t s_bin;
+  __shared__ int s_long[kSelLong];
+  __shared__ hkey s_bound;
   __shared__ int s_nc, s_nlong;
 
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int ks = p.k_sel, nl = p.nlists;
+  const int b = (int)blockIdx.x / kSelCluster;
+  const int rank = (int)blockIdx.x - b * kSelCluster;
+  const int ks = p.k_sel, nc = p.nctas;
+  asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // waited for before the first remote store
   pdl_launch_dependents();
-  pdl_wait();                                    // every CTA list and count is written
-  for (int b = 0; b < p.B; ++b) {
-    const hkey* lists = p.lists + (int64_t)b * nl * kHeadList;
-    // one round of loads: this thread's 8 histogram bins and the leading keys
-    // (32 bytes) of lists t and t + kSelThreads
-    const uint4* hq = reinterpret_cast<const uint4*>(p.hist + (int64_t)b * kHistWords) + 2 * t;
-    const uint4 h0 = __ldcg(hq), h1 = __ldcg(hq + 1);
-    ulonglong2 lead[2][2];
+  pdl_wait();                                    // every list and count is written
+  hkey lead[kCtaLead];                           // of projection CTA t
+  if (t < nc) {
+    const ulonglong2* src =
+        reinterpret_cast<const ulonglong2*>(p.lead + ((int64_t)b * nc + t) * kCtaLead);
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int l = t + q * kSelThreads;
-      if (l < nl) {
-        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(lists + (int64_t)l * kHeadList);
-        lead[q][0] = __ldcg(src);
-        lead[q][1] = __ldcg(src + 1);
-      }
+    for (int q = 0; q < kCtaLead / 2; ++q) {
+      const ulonglong2 k = __ldcg(src + q);
+      lead[2 * q] = k.x;
+      lead[2 * q + 1] = k.y;
     }
-    for (int l = t + 2 * kSelThreads; l < nl; l += kSelThreads) {   // more than 1024 lists: never
-      const ulonglong2* src = reinterpret_cast<const ulonglong2*>(lists + (int64_t)l * kHeadList);
-      const ulonglong2 k01 = __ldcg(src), k23 = __ldcg(src + 1);
-      s_lead[l * kLead] = k01.x;
-      s_lead[l * kLead + 1] = k01.y;
-      s_lead[l * kLead + 2] = k23.x;
-      s_lead[l * kLead + 3] = k23.y;
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int l = t + q * kSelThreads;
-      if (l < nl) {
-        s_lead[l * kLead] = lead[q][0].x;
-        s_lead[l * kLead + 1] = lead[q][0].y;
-        s_lead[l * kLead + 2] = lead[q][1].x;
-        s_lead[l * kLead + 3] = lead[q][1].y;
-      }
-    }
-    if (t == 0) {
-      s_nc = 0;
-      s_nlong = 0;
-    }
-    // the bound (its barriers also complete the stores above)
-    const uint32_t hc[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-    const uint32_t tb = hist_bound(hc, kHeadList, s_wtot, s_bin);
-    const hkey T = tb ? (hkey)tb << 32 : 1ull;   // no bound: every key passes
-    for (int l = t; l < nl; l += kSelThreads) {
-      int n = 0;
-#pragma unroll
-      for (int e = 0; e < kLead; ++e) {
-        const hkey k = s_lead[l * kLead + e];
-        if (k >= T) {
-          const int i = atomicAdd(&s_nc, 1);
-          if (i < kSelThreads) s_cand[i] = k;
-          ++n;
-        }
-      }
-      if (n == kLead) {                          // the list may continue past its leading keys
-        const int j = atomicAdd(&s_nlong, 1);
-        if (j < kSelThreads) s_long[j] = l;
-      }
-    }
-    __syncthreads();
-    const int nlong = s_nlong;
-    for (int j = warp; j < min(nlong, kSelThreads); j += kSelWarps) {
-      const hkey* L = lists + (int64_t)s_long[j] * kHeadList;
-      for (int e = kLead + lane; e < kHeadList; e += 32) {
-        const hkey k = __ldcg(L + e);
-        if (k >= T) {
-          const int i = atomicAdd(&s_nc, 1);
-          if (i < kSelThreads) s_cand[i] = k;
-        }
-      }
-    }
-    __syncthreads();
-    const int C = s_nc;
-    if (C <= kSelThreads && nlong <= kSelThreads && C >= min(p.V, kHeadList)) {
-      rank_place(s_cand, C, s_best);
-    } else {
-      hkey* s16 = s_lead;                        // 16 lists: the running best, then 15 more
-      for (int i = t; i < kHeadList; i += kSelThreads) s16[i] = 0ull;
-      for (int base = 0; base < nl; base += 15) {
-        const int cnt = min(15, nl - base);
-        for (int e = t; e < 15 * kHeadList; e += kSelThreads)
-          s16[kHeadList + e] = e / kHeadList < cnt ? __ldcg(lists + (int64_t)base * kHeadList + e) : 0ull;
-        __syncthreads();
-        tree_merge(s16, 16, kSelWarps);
-      }
-      for (int i = t; i < kHeadList; i += kSelThreads) s_best[i] = s16[i];
-      __syncthreads();
-    }
-    const float g = __fsub_rn(key_z(s_best[0]), key_z(s_best[1]));
-    const bool open = g < p.tau;
-    if (open) {
-      const float* hb = p.h + (int64_t)b * p.ldh;
-      int rows[4];
-      int n = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = warp + kSelWarps * j;
-        rows[j] = i < ks ? key_row(s_best[i]) : 0;
-        if (i < ks) n = j + 1;
-      }
-      if (n > 0) {
-        float rv[4];
-        verify_rows4(p, hb, rows, n, lane, rv);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (j < n && lane == 0) s_r[warp + kSelWarps * j] = rv[j];
-      }
-      __syncthreads();
-    }
-    if (warp == 0) {
-      int token = key_row(s_best[0]);
-      if (open) {
-        // largest r, equal r: lower row (starting from candidate 0, so the
-        // token is always a candidate)
-        float br = s_r[0];
-        int bm = token;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int i = lane + 32 * q;
-          if (i < ks) {
-            const float rv = s_r[i];
-            const int m = key_row(s_best[i]);
-            if (rv > br || (rv == br && m < bm)) {
-              br = rv;
-              bm = m;
-            }
-            if (p.r) p.r[(int64_t)b * ks + i] = rv;
-          }
-        }
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-          const float orv = __shfl_xor_sync(0xffffffffu, br, d);
-          const int om = __shfl_xor_sync(0xffffffffu, bm, d);
-          if (orv > br || (orv == br && om < bm)) {
-            br = orv;
-            bm = om;
-          }
-        }
-        token = bm;
-      }
-      if (lane == 0) {
-        p.token[b] = token;
-        if (p.verified) p.verified[b] = open ? 1 : 0;
-        if (p.gap) p.gap[b] = g;
-      }
-    }
-    if (p.cand && t < ks) p.cand[(int64_t)b * ks + t] = key_row(s_best[t]);
-    __syncthreads();                             // s_lead, s_cand, s_best, s_r are rewritten next
   }
-  // the histograms are read: clear them for the next call
-  for (int i = t; i < p.B * kHistWords; i += kSelThreads) p.hist[i] = 0u;
+  if (t == 0) {
+    s_nc = 0;
+    s_nlong = 0;
+    s_bound = 1ull;                              // no bound: every key passes
+  }
+  // the bound: the 64th largest of the CTAs' best keys (of all their leading
+  // keys where there are fewer than 64 CTAs), found by counting the larger ones
+  const int per = nc >= kHeadList ? 1 : kCtaLead;
+  if (t < nc) {
+#pragma unroll
+    for (int e = 0; e < kCtaLead; ++e)
+      if (e < per) s_cand[t * per + e] = lead[e];
+  }
+  __syncthreads();
+  for (int i = t; i < nc * per; i += kSelThreads)
+    if (count_larger(s_cand, nc * per, s_cand[i]) == kHeadList - 1 && s_cand[i] != 0ull) s_bound = s_cand[i];
+  __syncthreads();
+  const hkey T = s_bound;
+  if (t < nc) {
+    int n = 0;
+#pragma unroll
+    for (int e = 0; e < kCtaLead; ++e) n += lead[e] >= T;
+    if (n == kCtaLead) {                         // its lists may hold more
+      const int j = atomicAdd(&s_nlong, 1);
+      if (j < kSelLong) s_long[j] = t;
+    } else if (n > 0) {
+      const int i = atomicAdd(&s_nc, n);
+#pragma unroll
+      for (int e = 0; e < kCtaLead - 1; ++e)
+        if (e < n && i + e < kSelCand) s_cand[i + e] = lead[e];
+    }
+  }
+  __syncthreads();
+  const hkey* lists = p.lists + (int64_t)b * nc * kHeadLists * kHeadList;
+  const int nlong = s_nlong;
+  if (nlong <= kSelLong) {
+    for (int j = 0; j < nlong; ++j) {
+      const hkey* L = lists + (int64_t)s_long[j] * kHeadLists * kHeadList;
+#pragma unroll
+      for (int e = 0; e < kHeadLists * kHeadList / kSelThreads; ++e) {
+        const hkey k = __ldcg(L + t + e * kSelThreads);
+        if (k >= T) {
+          const int i = atomicAdd(&s_nc, 1);
+          if (i < kSelCand) s_cand[i] = k;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const int C = s_nc;
+  if (C <= kSelCand && nlong <= kSelLong && C >= min(p.V, kHeadList)) {
+    rank_place(s_cand, C, s_best);
+  } else {
+    hkey a = 0ull, c = 0ull;
+    for (int l = warp; l < nc * kHeadLists; l += kSelWarps) {
+      const hkey* L = lists + (int64_t)l * kHeadList;
+      hkey la = __ldcg(L + lane), lb = __ldcg(L + 32 + lane);
+      sort64(la, lb, lane);                      // (lists of up to 64 keys are as they came)
+      list_merge(a, c, la, lb, lane);
+    }
+    s_merge[warp][lane] = a;
+    s_merge[warp][32 + lane] = c;
+    __syncthreads();
+    if (warp == 0) {
+      for (int w = 1; w < kSelWarps; ++w) list_merge(a, c, s_merge[w][lane], s_merge[w][32 + lane], lane);
+      s_best[lane] = a;
+      s_best[32 + lane] = c;
+    }
+    __syncthreads();
+  }
+  const float g = __fsub_rn(key_z(s_best[0]), key_z(s_best[1]));
+  const bool open = g < p.tau;
+  asm volatile("barrier.cluster.wait;" ::: "memory");   // rank 0 is running
+  if (open) {
+    const float* hb = p.h + (int64_t)b * p.ldh;
+    const int i0 = rank * kSelWarps + warp, i1 = i0 + kHeadList / 2;
+    const int n = i1 < ks ? 2 : i0 < ks ? 1 : 0;
+    if (n > 0) {
+      const int rows[2] = {key_row(s_best[i0]), n > 1 ? key_row(s_best[i1]) : 0};
+      float rv[2];
+      verify_rows2(p, hb, rows, n, lane, rv);
+      if (lane < n)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(&s_r[lane ? i1 : i0], 0)),
+                     "f"(lane ? rv[1] : rv[0])
+                     : "memory");
+    }
+  }
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  if (rank != 0) return;
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // every logit is in
+  if (warp == 0) {
+    int token = key_row(s_best[0]);
+    if (open) {
+      // largest r, equal r: lower row (starting from candidate 0, so the
+      // token is always a candidate)
+      float br = s_r[0];
+      int bm = token;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = lane + 32 * q;
+        if (i < ks) {
+          const float rv = s_r[i];
+          const int m = key_row(s_best[i]);
+          if (rv > br || (rv == br && m < bm)) {
+            br = rv;
+            bm = m;
+          }
+          if (p.r) p.r[(int64_t)b * ks + i] = rv;
+        }
+      }
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) {
+        const float orv = __shfl_xor_sync(0xffffffffu, br, d);
+        const int om = __shfl_xor_sync(0xffffffffu, bm, d);
+        if (orv > br || (orv == br && om < bm)) {
+          br = orv;
+          bm = om;
+        }
+      }
+      token = bm;
+    }
+    if (lane == 0) {
+      p.token[b] = token;
+      if (p.verified) p.verified[b] = open ? 1 : 0;
+      if (p.gap) p.gap[b] = g;
+    }
+  }
+  if (p.cand && t < ks) p.cand[(int64_t)b * ks + t] = key_row(s_best[t]);
 }
 
 int g_head_sms = 0;
-size_t g_select_smem = 0;       // dynamic shared-memory limit set on head_select_kernel
 
 template <typename Kern>
 cudaError_t raise_smem(Kern kernel, size_t bytes, size_t& set_bytes) {
@@ -648,40 +744,46 @@ cudaError_t raise_smem(Kern kernel, size_t bytes, size_t& set_bytes) {
 
 template <int B>
 cudaError_t launch_head_t(HeadParams p, cudaStream_t s) {
+  // The largest shared-memory carve-out for the selection too: with a smaller
+  // one its SM could not take a projection CTA beside it (the next call's,
+  // which starts while the selection runs), and the late CTA held up the call.
+  static bool carve_done = false;
+  if (!carve_done) {
+    const cudaError_t e = cudaFuncSetAttribute(head_select_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                               (int)cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    carve_done = true;
+  }
   static size_t set_proj = 0;    // per instance: head_kernel<B> is a kernel of its own
-  const size_t smem = (size_t)kHeadWarps * kHeadList * 8 + (size_t)B * p.Kpad;
+  const size_t smem = kHeadRingBytes + (size_t)B * (p.Kpad + kCodePad);
   cudaError_t e = raise_smem(head_kernel<B>, smem, set_proj);
   if (e != cudaSuccess) return e;
-  // resident CTAs per SM, queried once per shared-memory size (a driver
-  // call of about a microsecond)
-  static int per_sm = 0;
-  static size_t per_sm_smem = 0;
-  if (per_sm == 0 || per_sm_smem != smem) {
-    int n = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, head_kernel<B>, kHeadThreads, smem);
-    if (e != cudaSuccess) return e;
-    per_sm = n < 1 ? 1 : n;
-    per_sm_smem = smem;
-  }
-  // one wave: every CTA resident at once
-  int grid = g_head_sms * per_sm;
-  const int need = (p.units + kHeadWarps - 1) / kHeadWarps;
-  if (grid > need) grid = need;
+  // one wave, one CTA per SM
+  int grid = g_head_sms;
+  if (grid > p.units) grid = p.units;
   if (grid > kHeadMaxGrid) grid = kHeadMaxGrid;
-  if (grid < 1) grid = 1;
-  p.nlists = grid;
+  p.nctas = grid;
   e = launch_pdl(head_kernel<B>, dim3((unsigned)grid), dim3(kHeadThreads), smem, s, p);
   if (e != cudaSuccess) return e;
-
-  const size_t sel_smem = (size_t)(grid * kLead > 16 * kHeadList ? grid * kLead : 16 * kHeadList) * 8;
-  e = raise_smem(head_select_kernel, sel_smem, g_select_smem);   // one kernel for every B
-  if (e != cudaSuccess) return e;
-  return launch_pdl(head_select_kernel, dim3(1), dim3(kSelThreads), sel_smem, s, p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(B * kSelCluster, 1, 1);
+  cfg.blockDim = dim3(kSelThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kSelCluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, head_select_kernel, p);
 }
 
 }  // namespace
 
-size_t head_workspace_bytes() { return kListBytes + kHistBytes; }
+size_t head_workspace_bytes() { return kListBytes + kLeadBytes; }
 
 cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
   if (g_head_sms == 0) {
@@ -697,7 +799,7 @@ cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
   p.scale = a.scale;
   p.V = a.V;
   p.K = a.K;
-  p.Kpad = (a.K + 511) / 512 * 512;
+  p.Kpad = (a.K + kHeadChunk - 1) / kHeadChunk * kHeadChunk;
   p.units = (a.V + kHeadRows - 1) / kHeadRows;
   p.h = a.h;
   p.ldh = a.ldh;
@@ -712,8 +814,8 @@ cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
   p.ld_z = a.ld_z;
   p.B = a.B;
   p.lists = static_cast<hkey*>(a.ws);
-  p.hist = reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(a.ws) + kListBytes);
-  p.nlists = 0;
+  p.lead = reinterpret_cast<hkey*>(static_cast<unsigned char*>(a.ws) + kListBytes);
+  p.nctas = 0;
   switch (a.B) {
     case 1: return launch_head_t<1>(p, s);
     case 2: return launch_head_t<2>(p, s);

@@ -169,7 +169,7 @@ cudaError_t launch_lif_rows(const float* vin, float* vout, const float* I, const
                             int64_t ld_bits, cudaStream_t s);
 
 // One vocabulary-head call (see spike_proj_head); ws is the head's workspace
-// of head_workspace_bytes(), zero when created (the kernels leave it so).
+// of head_workspace_bytes() (rewritten by every call).
 struct HeadArgs {
   const int8_t* W;
   int64_t ldw;

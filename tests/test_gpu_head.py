@@ -173,6 +173,34 @@ def test_head_full_size(k_sel):
               f"full k={k_sel} tau={tau}")
 
 
+@pytest.mark.parametrize("B", [1, 3, 4])
+def test_head_long_lists(B):
+    """More than 64 rows per list (the lists are then kept sorted) and K below
+    the ring's depth: a wide vocabulary of short rows."""
+    V, K = 150_001, 40
+    Q, s = small_case(5, V, K)
+    head = sp.Head(to_dev(Q), to_dev(s), K=K)
+    h = synth.rng_for(7811, B).standard_normal((B, K)).astype(np.float32)
+    for tau, k_sel in ((0.0, 64), (np.inf, 64)):
+        check(run_head(head, h, tau, k_sel, V), Q, s, V, K, h, tau, k_sel, f"V={V} B={B}")
+
+
+@pytest.mark.parametrize("V,K", [(57344, 64), (9000, 64), (600, 512)])
+def test_head_candidates_in_few_units(V, K):
+    """The best rows crowded into a few 16-row units, spread by the number of
+    SMs, so that one or several CTAs hold more candidates than their leading
+    keys show and their lists are read in full (or every list is merged)."""
+    Q, s = small_case(6, V, K)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    grid = min(sms, -(-V // 16))
+    unit = np.arange(V) // 16
+    h = synth.rng_for(7812, V).standard_normal((2, K)).astype(np.float32)
+    for ctas in (1, 5, 40):
+        sc = np.where(unit % grid < ctas, s * np.float32(50), s).astype(np.float32)
+        head = sp.Head(to_dev(Q), to_dev(sc), K=K)
+        check(run_head(head, h, np.inf, 64, V), Q, sc, V, K, h, np.inf, 64, f"V={V} ctas={ctas}")
+
+
 def test_head_outputs_optional():
     V, K = 1000, 128
     Q, s = small_case(6, V, K)
