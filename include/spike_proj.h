@@ -107,7 +107,8 @@ typedef enum sp_fmt {
  *   SP_AUTO    count the active spikes on the device, read the count back
  *              (one stream synchronisation) and pick SP_GATHER or, on a plan
  *              made with SP_PLAN_GEMM, SP_GEMM when its modelled time is
- *              lower (large batches and dense prefill).
+ *              lower (large batches and dense prefill).  Where SP_GEMM is
+ *              picked whatever the count, the call does not wait for it.
  *   SP_GATHER  per-token active-column gather (the batch-1 kernel per row).
  *   SP_UNION   one fetch of each column in the union of the rows' active sets,
  *              added into every row whose spike is set.
@@ -206,7 +207,8 @@ sp_status spike_proj_prefill(sp_plan_t plan, const uint8_t *X, int32_t T,
 
 /* Strategy and total active count (sum over rows of |A|) of the last
  * batched / prefill call with SP_AUTO on this plan; the count is -1 when the
- * last call did not measure it. */
+ * last call did not measure it.  Synchronises the device if the kernel that
+ * counts has not finished. */
 sp_status spike_proj_last_dispatch(sp_plan_t plan, sp_kernel *chosen,
                                    int32_t *active_count);
 

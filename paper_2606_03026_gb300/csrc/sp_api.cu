@@ -35,8 +35,10 @@ struct sp_plan_s {
   uint32_t* tickets = nullptr;    // zero between calls
   size_t n_tickets = 0;
   int* err = nullptr;             // device error word
-  int32_t* d_counts = nullptr;    // density probe result [2]
-  int32_t* h_counts = nullptr;    // page-locked copy
+  int32_t* d_counts = nullptr;    // spike count in progress and its tickets (SpikeCount)
+  int32_t* h_counts = nullptr;    // page-locked: the last count, the sequence number it is of
+  int32_t count_seq = 0;          // counts asked for
+  bool count_pending = false;     // last_active is still to be read from h_counts
   // tensor-core path
   uint8_t* Wq = nullptr;          // [N][2 Kp] e4m3 weight planes (16 h, l)
   uint8_t* Xs = nullptr;          // [xs_rows][Kp] 0/1 spike staging
@@ -288,11 +290,14 @@ sp_status run_union(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
   return SP_OK;
 }
 
+// count: asked for with SP_AUTO (else count.dev is null); the spikes are
+// counted by the staging pass where there is one.
 sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld, int32_t* acc,
-                   float* y, cudaStream_t s) {
+                   float* y, const SpikeCount& count, cudaStream_t s) {
   if (!(p->flags & SP_PLAN_GEMM)) return SP_EUNSUPPORTED;
   // a few rows: the transposed small-T form reads the spike rows in place
   if (const int S = gemm_small_splits(T, p->N, p->Kp)) {
+    if (count.dev) SP_CUDA(launch_density(spikes, fmt, ld, T, p->K, count, s));
     GemmSmallArgs g;
     g.spikes = spikes;
     g.fmt = fmt;
@@ -317,6 +322,7 @@ sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld,
   const bool in_place = fmt == SP_SPIKES_BOOL8 && aligned(spikes, 16) && ld % 16 == 0;
   const int S = gemm_splits(T, p->N, p->Kp, p->part_units);
   if (in_place) {
+    if (count.dev) SP_CUDA(launch_density(spikes, fmt, ld, T, p->K, count, s));
     if (spikes != p->rows_ptr || ld != p->rows_ld || T != p->rows_T) {
       SP_CUDA(gemm_make_rows_map(spikes, ld, T, p->K, &p->rows_map));
       p->rows_ptr = spikes;
@@ -324,7 +330,7 @@ sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld,
       p->rows_T = T;
     }
   } else {
-    SP_CUDA(launch_spikes_to_01(spikes, fmt, ld, T, p->K, p->Kp, p->Xs, s));
+    SP_CUDA(launch_spikes_to_01(spikes, fmt, ld, T, p->K, p->Kp, p->Xs, count, s));
   }
   GemmParams g;
   g.scale = p->scale;
@@ -375,18 +381,40 @@ sp_kernel choose(const sp_plan_s* p, int B, int32_t total) {
 
 sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld, int32_t* acc,
                     float* y, sp_kernel strategy, cudaStream_t s) {
+  SpikeCount count = {};
   if (strategy == SP_AUTO) {
-    SP_CUDA(launch_density(spikes, fmt, ld, B, p->K, p->d_counts, s));
-    SP_CUDA(cudaMemcpyAsync(p->h_counts, p->d_counts, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    count.dev = p->d_counts;
+    count.host = p->h_counts;
+    count.seq = ++p->count_seq;
+    // Where the GEMM is modelled faster than a gather of no column at all,
+    // the count cannot change the choice: the GEMM is enqueued at once, the
+    // count comes with it (spike_proj_last_dispatch waits for it), and the
+    // host does not.  173 byte rows of 1990 columns: 31.9 us a call with the
+    // count, its copy and the synchronisation ahead of the GEMM, 14.0
+    // without.  A stream being captured takes the other way and is refused
+    // by its synchronisation.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (choose(p, B, 0) == SP_GEMM && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone) {
+      const sp_status st = run_gemm(p, spikes, fmt, B, ld, acc, y, count, s);
+      if (st == SP_OK) {
+        p->last_kernel = SP_GEMM;
+        p->count_pending = true;
+      }
+      return st;
+    }
+    SP_CUDA(launch_density(spikes, fmt, ld, B, p->K, count, s));
     SP_CUDA(cudaStreamSynchronize(s));
     strategy = choose(p, B, p->h_counts[0]);
     p->last_kernel = strategy;
     p->last_active = p->h_counts[0];
+    p->count_pending = false;
+    count = SpikeCount{};
   }
   switch (strategy) {
     case SP_GATHER: return run_gather(p, spikes, fmt, B, ld, acc, y, s);
     case SP_UNION: return run_union(p, spikes, fmt, B, ld, acc, y, s);
-    case SP_GEMM: return run_gemm(p, spikes, fmt, B, ld, acc, y, s);
+    case SP_GEMM: return run_gemm(p, spikes, fmt, B, ld, acc, y, count, s);
     default: return SP_EINVAL;
   }
 }
@@ -471,6 +499,7 @@ sp_status spike_proj_plan(sp_plan_t* plan, const int8_t* W, int64_t ldw, const f
     plan_free(p);
     return cuda_fail(e);
   }
+  p->h_counts[0] = p->h_counts[1] = 0;
   if (flags & SP_PLAN_GEMM) {
     p->Kp = gemm_k_pad(K);
     p->xs_rows = ceil_div(max_batch, 128) * 128;
@@ -540,6 +569,13 @@ sp_status spike_proj_prefill(sp_plan_t plan, const uint8_t* X, int32_t T, int64_
 
 sp_status spike_proj_last_dispatch(sp_plan_t plan, sp_kernel* chosen, int32_t* active_count) {
   if (!plan) return SP_EINVAL;
+  if (plan->count_pending) {
+    // the counting kernel of the last SP_AUTO call may still be running
+    const volatile int32_t* host = plan->h_counts;
+    if (host[1] != plan->count_seq) SP_CUDA(cudaDeviceSynchronize());
+    plan->last_active = host[0];
+    plan->count_pending = false;
+  }
   if (chosen) *chosen = plan->last_kernel;
   if (active_count) *active_count = plan->last_active;
   return SP_OK;
@@ -710,7 +746,7 @@ sp_status spike_proj_group_prefill(sp_group_t g, const void* const* X, sp_fmt fm
       }
       M.a = g->rows_map[j];
     } else {
-      SP_CUDA(launch_spikes_to_01(X[j], fmt, ldx, T, p->K, p->Kp, p->Xs, s));
+      SP_CUDA(launch_spikes_to_01(X[j], fmt, ldx, T, p->K, p->Kp, p->Xs, SpikeCount{}, s));
       M.a = p->maps.a;
     }
     M.b = cl == 2 ? p->maps.b128 : p->maps.b;

@@ -862,17 +862,41 @@ __global__ void w_to_e4m3_kernel(const int8_t* __restrict__ W, int64_t ldw, int 
   }
 }
 
+// Sixteen spike bytes at x (any alignment) as 0 / 1 bytes, from the five
+// aligned words that hold them; [lo, hi) bounds the words that may be read.
+// False where one of them is outside.
+__device__ __forceinline__ bool bytes16_to_01(const uint8_t* x, const uint8_t* lo, const uint8_t* hi,
+                                              uint4& o) {
+  const uint8_t* w0 = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(x) & ~(uintptr_t)3);
+  if (w0 < lo || w0 + 20 > hi) return false;
+  uint32_t w[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t*>(w0) + i);
+  const uint32_t sh = 8u * (uint32_t)(x - w0);
+  o = make_uint4(nonzero_bytes_to_01(__funnelshift_r(w[0], w[1], sh)),
+                 nonzero_bytes_to_01(__funnelshift_r(w[1], w[2], sh)),
+                 nonzero_bytes_to_01(__funnelshift_r(w[2], w[3], sh)),
+                 nonzero_bytes_to_01(__funnelshift_r(w[3], w[4], sh)));
+  return true;
+}
+
 // Spike rows (any format) -> 0/1 bytes [T][Kp], zero past K.  One thread per
 // 16 consecutive columns of a row: one 16-byte store.  kVec: byte rows are
 // 16-byte aligned (base and leading dimension), so whole 16-column groups
-// load as one vector.
+// load as one vector; other byte rows load the aligned words around a group
+// (single bytes only at the ends of the matrix and of a row).  The spikes are
+// counted on the way when a count is asked for: SP_AUTO then needs no pass of
+// its own over them.
 template <bool kVec>
 __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, int64_t ld, int T,
-                                    int K, int Kp, uint8_t* __restrict__ Xs) {
+                                    int K, int Kp, uint8_t* __restrict__ Xs, SpikeCount count) {
   pdl_launch_dependents();
   pdl_wait();
   const int per_row = Kp / 16;
   const int64_t total = (int64_t)T * per_row;
+  const uint8_t* lo = static_cast<const uint8_t*>(spikes);
+  const uint8_t* hi = lo + (int64_t)(T - 1) * ld + K;      // byte rows
+  int active = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int t = (int)(i / per_row);
@@ -880,16 +904,17 @@ __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, in
     uint4 o = make_uint4(0u, 0u, 0u, 0u);
     if (k < K) {
       const void* row = spike_row(spikes, fmt, t, ld);
+      const uint8_t* x = static_cast<const uint8_t*>(row) + k;
       if (fmt != SP_SPIKES_BITS32 && kVec && K - k >= 16) {
-        const uint4 w = __ldg(reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(row) + k));
+        const uint4 w = __ldg(reinterpret_cast<const uint4*>(x));
         o = make_uint4(nonzero_bytes_to_01(w.x), nonzero_bytes_to_01(w.y), nonzero_bytes_to_01(w.z),
                        nonzero_bytes_to_01(w.w));
+      } else if (fmt != SP_SPIKES_BITS32 && !kVec && K - k >= 16 && bytes16_to_01(x, lo, hi, o)) {
       } else {
         uint32_t bits = 0u;                  // spikes of columns k .. k+15
         if (fmt == SP_SPIKES_BITS32) {
           bits = (__ldg(reinterpret_cast<const uint32_t*>(row) + (k >> 5)) >> (k & 31)) & 0xffffu;
         } else {
-          const uint8_t* x = static_cast<const uint8_t*>(row) + k;
           const int n = K - k < 16 ? K - k : 16;
           for (int j = 0; j < n; ++j) bits |= (uint32_t)(__ldg(x + j) != 0) << j;
         }
@@ -903,8 +928,11 @@ __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, in
         o = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
+    // (the bytes are 0 / 1: adding the words keeps byte sums below 5)
+    active += (int)(((o.x + o.y + o.z + o.w) * 0x01010101u) >> 24);
     *reinterpret_cast<uint4*>(Xs + (int64_t)t * Kp + k) = o;
   }
+  if (count.dev) count_spikes(active, count);
 }
 
 int g_num_sms = 0;
@@ -1043,7 +1071,7 @@ cudaError_t launch_w_to_e4m3(const int8_t* W, int64_t ldw, int N, int K, uint8_t
 }
 
 cudaError_t launch_spikes_to_01(const void* spikes, int fmt, int64_t ld, int T, int K, int Kp,
-                                uint8_t* Xs, cudaStream_t s) {
+                                uint8_t* Xs, const SpikeCount& count, cudaStream_t s) {
   const int64_t total = (int64_t)T * (Kp / 16);
   const int threads = 256;
   int64_t blocks = (total + threads - 1) / threads;
@@ -1053,9 +1081,9 @@ cudaError_t launch_spikes_to_01(const void* spikes, int fmt, int64_t ld, int T, 
                    ld % 16 == 0;
   if (vec)
     return launch_pdl(spikes_to_01_kernel<true>, dim3((unsigned)blocks), dim3(threads), 0, s, spikes,
-                      fmt, ld, T, K, Kp, Xs);
+                      fmt, ld, T, K, Kp, Xs, count);
   return launch_pdl(spikes_to_01_kernel<false>, dim3((unsigned)blocks), dim3(threads), 0, s, spikes,
-                    fmt, ld, T, K, Kp, Xs);
+                    fmt, ld, T, K, Kp, Xs, count);
 }
 
 namespace {

@@ -222,11 +222,21 @@ cudaError_t launch_probe_gather(const uint8_t* base, const uint32_t* offsets16, 
 cudaError_t launch_gather(const GatherParams1& p, cudaStream_t s);
 cudaError_t launch_gather(const GatherParamsG& p, cudaStream_t s);
 cudaError_t launch_union(const UnionParams& p, cudaStream_t s);
-// Counts active spikes: out[0] = sum over the B rows of |A_t| (out[1] unused).
+// Where a kernel that counts active spikes (sum over the rows of |A_t|) leaves
+// the count: the grid's blocks add into dev[0] and take tickets from dev[1];
+// the last one writes host[0] = count, then host[1] = seq (page-locked memory,
+// visible without a copy), and leaves dev zero for the next call.
+struct SpikeCount {
+  int32_t* dev;           // two words, zero between launches; null: no count
+  int32_t* host;
+  int32_t seq;
+};
+// Counts active spikes.
 cudaError_t launch_density(const void* spikes, int fmt, int64_t ld, int B, int K,
-                           int32_t* out, cudaStream_t s);
-// Spike rows in any format -> bytes 0 / 1 [T][Kp] (zero past K).
+                           const SpikeCount& count, cudaStream_t s);
+// Spike rows in any format -> bytes 0 / 1 [T][Kp] (zero past K), counted on the
+// way when count.dev is set.
 cudaError_t launch_spikes_to_01(const void* spikes, int fmt, int64_t ld, int T, int K, int Kp,
-                                uint8_t* Xs, cudaStream_t s);
+                                uint8_t* Xs, const SpikeCount& count, cudaStream_t s);
 
 }  // namespace sp

@@ -55,6 +55,29 @@ __device__ __forceinline__ const void* spike_row(const void* base, int fmt, int6
              : static_cast<const void*>(reinterpret_cast<const uint8_t*>(base) + row * ld);
 }
 
+// Adds the calling thread's share of a launch's spike count and, in the last
+// block to arrive, publishes the total (SpikeCount).  Every thread of the
+// grid calls it once; blockDim.x is a multiple of 32, at most 1024.
+__device__ __forceinline__ void count_spikes(int mine, const SpikeCount& c) {
+  __shared__ int s_sum[32];
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = mine;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  int sum = 0;
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) sum += s_sum[w];
+  if (sum) atomicAdd(c.dev, sum);
+  __threadfence();
+  if (atomicAdd(c.dev + 1, 1) != (int)gridDim.x - 1) return;
+  __threadfence();
+  volatile int32_t* host = c.host;
+  host[0] = atomicExch(c.dev, 0);
+  c.dev[1] = 0;
+  __threadfence_system();
+  host[1] = c.seq;
+}
+
 // Warp-cooperative compaction of nw <= 32 words into ascending column
 // indices base_k + 32*i + bit.  Call with the whole warp; returns |list| to
 // every lane.

@@ -206,11 +206,9 @@ union_kernel(const __grid_constant__ UnionParams p) {
   }
 }
 
-// Density probe: out[0] += sum over rows of |A_t| (out zeroed by the caller).
-// One thread per (row, 32-column word), grid-stride; warp sums, one atomic
-// per warp.
+// Density probe: one thread per (row, 32-column word), grid-stride.
 __global__ void density_kernel(const void* spikes, int fmt, int64_t ld, int B, int K,
-                               int32_t* out) {
+                               SpikeCount count) {
   const int nw = ceil_div(K, 32);
   const int64_t total_words = (int64_t)nw * B;
   int total = 0;
@@ -220,9 +218,7 @@ __global__ void density_kernel(const void* spikes, int fmt, int64_t ld, int B, i
     const int w = (int)(i - (int64_t)t * nw);
     total += __popc(spike_word(spike_row(spikes, fmt, t, ld), fmt, K, 32 * w));
   }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) total += __shfl_xor_sync(0xffffffffu, total, d);
-  if ((threadIdx.x & 31) == 0 && total) atomicAdd(out, total);
+  count_spikes(total, count);
 }
 
 int g_union_grid = 0;
@@ -252,16 +248,14 @@ cudaError_t launch_union(const UnionParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_density(const void* spikes, int fmt, int64_t ld, int B, int K, int32_t* out,
-                           cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(int32_t), s);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_density(const void* spikes, int fmt, int64_t ld, int B, int K,
+                           const SpikeCount& count, cudaStream_t s) {
   const int64_t words = (int64_t)ceil_div(K, 32) * B;
   const int threads = 256;
   int64_t grid = (words + threads - 1) / threads;
   if (grid > 2048) grid = 2048;
   if (grid < 1) grid = 1;
-  density_kernel<<<(int)grid, threads, 0, s>>>(spikes, fmt, ld, B, K, out);
+  density_kernel<<<(int)grid, threads, 0, s>>>(spikes, fmt, ld, B, K, count);
   return cudaGetLastError();
 }
 

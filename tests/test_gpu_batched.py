@@ -261,3 +261,37 @@ def test_errors_on_device():
         sp.Plan(W, S, 64, 128, ldw=72)
     assert e.value.status == sp.SP_EALIGN
     assert plan.status() == sp.SP_OK
+
+
+@pytest.mark.parametrize("fmt", ["u8", "bool8", "bits"])
+@pytest.mark.parametrize("shift", [0, 1, 3, 16])
+def test_auto_counts_without_waiting(fmt, shift):
+    """SP_AUTO where the GEMM is picked whatever the count: the spikes are
+    counted by the staging pass (or beside the in-place rows), for rows at any
+    alignment and ragged widths, and the count is right when it is asked for
+    at once, after several calls in flight, and after an explicit strategy."""
+    N, K, T = 1040, 1990, 173
+    Qc, s, _ = synth.random_case(91, N, K, T=T)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=T, gemm=True)
+    rng = synth.rng_for(7301, shift)
+    acc = torch.empty(T, N, dtype=torch.int32, device=DEV)
+    y = torch.empty(T, N, dtype=torch.float32, device=DEV)
+    for p in (0.15, 0.0, 1.0, 0.4):
+        X = synth.bernoulli(rng, (T, K), p)
+        if fmt == "bits":
+            rows = synth.pack_bits(X)
+            buf = to_dev(np.concatenate([np.zeros(shift, rows.dtype), rows.reshape(-1)]).view(np.int32))
+            x, ld = buf[shift:], rows.shape[1]
+        else:
+            ld = 2000 if shift == 16 else K + (3 if shift == 3 else 0)   # 2000: in place for bool8
+            pad = np.full((T, ld), 1, np.uint8)                          # past K: never counted
+            pad[:, :K] = X * (rng.integers(1, 256, X.shape) if fmt == "u8" else 1)
+            buf = to_dev(np.concatenate([np.zeros(shift, np.uint8), pad.reshape(-1)[:(T - 1) * ld + K]]))
+            x = buf[shift:]
+        for _ in range(3):
+            plan.batched(x, fmt, T, ld, acc, y, "auto")
+        assert plan.last_dispatch() == ("gemm", int(X.astype(np.int64).sum()))
+        want_acc, want_y = oracle.project(Qc, s, N, K, X, "u8", ldq=Qc.shape[1])
+        assert_parity(acc, y, want_acc, want_y, f"auto {fmt} shift {shift} p {p}")
+        plan.batched(x, fmt, T, ld, acc, y, "gather")
+        assert plan.last_dispatch() == ("gemm", int(X.astype(np.int64).sum()))
