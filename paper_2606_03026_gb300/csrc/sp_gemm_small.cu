@@ -28,9 +28,10 @@
 //               spike rows (any input format) into 0 / 1 bytes in the
 //               64-byte-swizzled K-major layout the MMA reads (the layout a
 //               TMA box with 64-byte swizzle writes), K block by K block.
-//   warps 2-5   then read the accumulator (warp w: TMEM lane quarter w % 4,
-//               i.e. 32 channels x TN tokens) and reduce it over the
-//               cluster: the tokens form groups of 4, group g belongs to
+//               Blocks after the first are fenced and published in groups.
+//   warps 2-9   then read the accumulator (warp w: TMEM lane quarter w % 4,
+//               i.e. 32 channels, and every other 16 tokens) and reduce it
+//               over the cluster: the tokens form groups of 4, group g belongs to
 //               cluster rank g % S, every CTA pushes each group's 4 values of
 //               its 32 channels into the owner's shared memory with st.async
 //               (distributed shared memory), which counts the bytes on the
@@ -38,6 +39,13 @@
 //               alone, adds the S partials of its groups and writes acc / y
 //               (a warp's 32 lanes hold 32 consecutive channels of one
 //               token: 128-byte stores).
+// Measured (us per call, weights in L2, before and after blocks were fenced in
+// groups, byte rows published in phases, commits dropped where no slot is
+// refilled, and all 8 warps wrote the output): 1536 x 6144, 64 bit rows 9.2 ->
+// 8.5, 64 byte rows 11.8 -> 9.3, 16 bit rows 7.2 -> 7.05; 1536 x 1536, 64 rows
+// 6.2 -> 5.7.  What is left of the 8.5: 1.4 from the end of one launch to the
+// dependency wait of the next, 1.1 to the first block staged, 3 of MMAs (64-80
+// cycles each whatever N <= 64), 1.2 of exchange, 1.3 of output.
 // No workspace, no atomics, no flags: the inter-CTA waits are one cluster
 // barrier (every peer has staged its spike slice, so its receive area is
 // free) and the receive mbarriers.  Every mbarrier wait is bounded; on
@@ -63,6 +71,10 @@ constexpr int kSmGroups = kGemmSmallMaxT / 4;       // 4-token groups
 constexpr int kSmRecvSlots = kSmGroups;
 constexpr int kSmStageWarps = 8;              // warps 2-9 stage the spike operand
 constexpr int kSmThreads = 64 + 32 * kSmStageWarps;
+constexpr int kSmFenceBlocks = 4;             // K blocks staged behind one proxy fence
+constexpr int kSmPhases = kGemmSmallMaxKB / 4;   // byte rows: commit groups of four K blocks
+static_assert(kSmPhases == 4, "the waits of the byte rows' phases");
+static_assert(8 * kSmStageWarps >= kGemmSmallMaxT, "a row of every staging warp's pass");
 constexpr int kSmTmemCols = kGemmSmallMaxT;
 constexpr size_t kSmRing = (size_t)kSmStages * kSmWBytes;
 constexpr size_t kSmX = (size_t)kGemmSmallMaxKB * kSmXBlock;
@@ -117,28 +129,30 @@ __device__ __forceinline__ void load_planes(uint8_t* dst, const CUtensorMap* map
 }
 
 // The four MMAs of one K block (two 32-column K steps x the two weight
-// planes, one accumulator), the commit that frees its ring slot, and a
+// planes, one accumulator), the commit that frees its ring slot where a later
+// block refills it (a commit costs the issuing thread as much as an MMA), and a
 // non-blocking test of the NEXT block's full barrier issued ahead of them, so
 // that its shared-memory latency overlaps the MMA issue.  Returns the test.
 __device__ __forceinline__ bool mma_block(uint32_t tmem, uint64_t hd, uint64_t ld, uint64_t xd,
-                                          uint32_t idesc, bool accumulate, uint64_t* empty_bar,
+                                          uint32_t idesc, bool accumulate, bool refill, uint64_t* empty_bar,
                                           uint64_t* next_full, uint32_t next_phase) {
   uint32_t ready;
   asm volatile(
-      "{\n\t.reg .pred pn, pa, pt;\n\t"
+      "{\n\t.reg .pred pn, pa, pt, pc;\n\t"
       "mbarrier.test_wait.parity.shared::cta.b64 pn, [%1], %2;\n\t"
       "setp.ne.b32 pa, %3, 0;\n\t"
       "setp.eq.b32 pt, 0, 0;\n\t"
+      "setp.ne.b32 pc, %13, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%4], %5, %7, %9, pa;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%4], %6, %7, %9, pt;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%4], %10, %8, %9, pt;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%4], %11, %8, %9, pt;\n\t"
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%12];\n\t"
+      "@pc tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%12];\n\t"
       "selp.u32 %0, 1, 0, pn;\n\t}"
       : "=r"(ready)
       : "r"(smem_u32(next_full)), "r"(next_phase), "r"((uint32_t)accumulate), "r"(tmem), "l"(hd),
         "l"(ld), "l"(xd), "l"(xd + 2u), "r"(idesc), "l"(hd + 2u), "l"(ld + 2u),
-        "r"(smem_u32(empty_bar))
+        "r"(smem_u32(empty_bar)), "r"((uint32_t)refill)
       : "memory");
   return ready != 0;
 }
@@ -233,8 +247,8 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
   const int q = warp & 3;                  // TMEM lane quarter of an epilogue warp
   const int row = q * 32 + lane;           // channel within the tile
   const int m = mt * kSmM + row;
-  const bool epi = warp >= 2 && warp < 6;   // epilogue: TMEM lane quarters 2, 3, 0, 1
-  const bool stg = warp >= 2;              // staging warps
+  const bool epi = warp >= 2;              // staging and epilogue warps: TMEM lane quarters 2, 3, 0, 1 twice
+  const int half = (warp - 2) >> 2;        // which of the two warps of a lane quarter
   // the scale of this thread's channel, read now so that no load waits in the epilogue
   const float sc = (epi && a.y && m < a.N) ? __ldg(a.scale + m) : 0.f;
   if (warp == 0) {
@@ -286,7 +300,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
         const uint64_t xd = smem_desc(sX + (size_t)i * kSmXBlock, 512, kSwizzle64);
         const int nstage = stage + 1 == kSmStages ? 0 : stage + 1;
         const uint32_t nfph = nstage == 0 ? fph ^ 1u : fph;
-        have = mma_block(tmem, hd, ld, xd, idesc, i > 0, &empty[stage], &full[nstage], nfph);
+        have = mma_block(tmem, hd, ld, xd, idesc, i > 0, i + kSmStages < nk, &empty[stage], &full[nstage], nfph);
         stage = nstage;
         fph = nfph;
       }
@@ -336,79 +350,94 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
       asm volatile("bar.sync 1, %0;" ::"n"(32 * kSmStageWarps) : "memory");
       const int rr = lane >> 2, j = lane & 3;
       const int shift = 16 * (j & 1);
+      // The first block alone, so that the MMAs start early; then several
+      // blocks behind one proxy fence (a fence per block held the MMAs of
+      // the first seven blocks back: 700 cycles a block instead of 450).
+      // Groups of 2 / 4 / 6 / 16: 8.62 / 8.52 / 8.61 / 8.96 us at 64 rows.
 #pragma unroll 1
-      for (int b = 0; b < nk; ++b) {
-        const int k = (kb0 + b) * 64 + 16 * j;
-        const int rem = a.K - k;
-        const uint32_t mask = rem >= 16 ? 0xffffu : (rem > 0 ? (1u << rem) - 1u : 0u);
-        const uint32_t* src = scratch + 2 * b + (j >> 1);
-        uint8_t* dst = sX + b * kSmXBlock;
+      for (int b0 = 0; b0 < nk;) {
+        const int b1 = min(nk, b0 == 0 ? 1 : b0 + kSmFenceBlocks);
 #pragma unroll 2
-        for (int r = 8 * e + rr; r < TN; r += 8 * kSmStageWarps) {
-          const uint32_t bits = (src[r * kScr] >> shift) & mask;
-          uint4 o;
-          o.x = ((bits & 0xfu) * 0x204081u) & 0x01010101u;
-          o.y = (((bits >> 4) & 0xfu) * 0x204081u) & 0x01010101u;
-          o.z = (((bits >> 8) & 0xfu) * 0x204081u) & 0x01010101u;
-          o.w = ((bits >> 12) * 0x204081u) & 0x01010101u;
-          *reinterpret_cast<uint4*>(dst + r * 64 + ((j ^ ((r >> 1) & 3)) << 4)) = o;
+        for (int b = b0; b < b1; ++b) {
+          const int k = (kb0 + b) * 64 + 16 * j;
+          const int rem = a.K - k;
+          const uint32_t mask = rem >= 16 ? 0xffffu : (rem > 0 ? (1u << rem) - 1u : 0u);
+          const uint32_t* src = scratch + 2 * b + (j >> 1);
+          uint8_t* dst = sX + b * kSmXBlock;
+          const int r = 8 * e + rr;
+          if (r < TN) {
+            const uint32_t bits = (src[r * kScr] >> shift) & mask;
+            uint4 o;
+            o.x = ((bits & 0xfu) * 0x204081u) & 0x01010101u;
+            o.y = (((bits >> 4) & 0xfu) * 0x204081u) & 0x01010101u;
+            o.z = (((bits >> 8) & 0xfu) * 0x204081u) & 0x01010101u;
+            o.w = ((bits >> 12) * 0x204081u) & 0x01010101u;
+            *reinterpret_cast<uint4*>(dst + r * 64 + ((j ^ ((r >> 1) & 3)) << 4)) = o;
+          }
         }
         // generic-proxy stores -> visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(&xready[b]);
+        if (lane < b1 - b0) mbar_arrive(&xready[b0 + lane]);
+        b0 = b1;
       }
     } else {
+      // Byte rows: one 16-byte copy per lane and K block, in kSmPhases commit
+      // groups of blocks; a phase is folded (U8) and published as soon as its
+      // own copies have landed.
       const int rr = lane >> 2, j = lane & 3;
-      const int groups = TN / 8;
-      bool any_async = false;
-#pragma unroll 1
-      for (int it = e; it < nk * groups; it += kSmStageWarps) {
-        const int b = it / groups;
-        const int r = (it - b * groups) * 8 + rr;
+      const int r = 8 * e + rr;
+      const uint8_t* row = r < a.T ? static_cast<const uint8_t*>(spike_row(a.spikes, a.fmt, r, a.ld)) : nullptr;
+      uint8_t* slot = sX + r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
+      const auto copied = [&](int b, const uint8_t*& src) {   // block b of this lane goes by cp.async
         const int k = (kb0 + b) * 64 + 16 * j;
-        uint8_t* dst = sX + b * kSmXBlock + r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
-        const uint8_t* src = r < a.T && k < a.K
-                                 ? static_cast<const uint8_t*>(spike_row(a.spikes, a.fmt, r, a.ld)) + k
-                                 : nullptr;
-        if (src && a.K - k >= 16 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
-                       : "memory");
-          any_async = true;
-        } else {
-          *reinterpret_cast<uint4*>(dst) = src ? spikes16(a, r, k) : make_uint4(0u, 0u, 0u, 0u);
-        }
-      }
-      asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
-      if (any_async && a.fmt == SP_SPIKES_U8) {   // any nonzero byte -> 1 (this lane's copies)
+        src = row && k < a.K ? row + k : nullptr;
+        return src && a.K - k >= 16 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
+      };
 #pragma unroll 1
-        for (int it = e; it < nk * groups; it += kSmStageWarps) {
-          const int b = it / groups;
-          const int r = (it - b * groups) * 8 + rr;
-          const int k = (kb0 + b) * 64 + 16 * j;
-          if (r < a.T && k + 16 <= a.K) {
-            uint4* p = reinterpret_cast<uint4*>(sX + b * kSmXBlock + r * 64 +
-                                                ((j ^ ((r >> 1) & 3)) << 4));
-            const uint4 v = *p;
-            *p = make_uint4(nonzero_bytes_to_01(v.x), nonzero_bytes_to_01(v.y),
-                            nonzero_bytes_to_01(v.z), nonzero_bytes_to_01(v.w));
+      for (int ph = 0; ph < kSmPhases; ++ph) {
+#pragma unroll 1
+        for (int b = 4 * ph; b < min(nk, 4 * ph + 4) && r < TN; ++b) {
+          const uint8_t* src;
+          if (copied(b, src))
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + b * kSmXBlock)), "l"(src)
+                         : "memory");
+          else
+            *reinterpret_cast<uint4*>(slot + b * kSmXBlock) =
+                src ? spikes16(a, r, (kb0 + b) * 64 + 16 * j) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+#pragma unroll
+      for (int ph = 0; ph < kSmPhases; ++ph) {
+        if (ph == 0) asm volatile("cp.async.wait_group 3;" ::: "memory");
+        else if (ph == 1) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (ph == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (a.fmt == SP_SPIKES_U8) {         // any nonzero byte -> 1 (this lane's copies)
+#pragma unroll 1
+          for (int b = 4 * ph; b < min(nk, 4 * ph + 4) && r < TN; ++b) {
+            const uint8_t* src;
+            if (copied(b, src)) {
+              uint4* p = reinterpret_cast<uint4*>(slot + b * kSmXBlock);
+              const uint4 v = *p;
+              *p = make_uint4(nonzero_bytes_to_01(v.x), nonzero_bytes_to_01(v.y), nonzero_bytes_to_01(v.z),
+                              nonzero_bytes_to_01(v.w));
+            }
           }
         }
+        // generic-proxy stores -> visible to the tensor core (async proxy)
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (4 * ph + lane < min(nk, 4 * ph + 4)) mbar_arrive(&xready[4 * ph + lane]);
       }
-    }
-    if (a.fmt != SP_SPIKES_BITS32) {
-      // generic-proxy stores -> visible to the tensor core (async proxy)
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0)
-        for (int b = 0; b < nk; ++b) mbar_arrive(&xready[b]);
     }
   }
   // Every CTA of the cluster arrives once its slice is staged (the receive
   // area held the BITS32 scratch) and waits, below, before its first store
   // into a peer's shared memory.
   if (S > 1) {
-    if (stg) asm volatile("bar.sync 1, %0;" ::"n"(32 * kSmStageWarps) : "memory");   // every staging warp is done
+    if (epi) asm volatile("bar.sync 1, %0;" ::"n"(32 * kSmStageWarps) : "memory");   // every staging warp is done
     asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
   }
 
@@ -432,7 +461,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
     asm volatile("barrier.cluster.wait;" ::: "memory");   // every peer has staged its slice
     if (epi && ok) {
 #pragma unroll 1
-      for (int c = 0; c < TN / 16; ++c) {
+      for (int c = half; c < TN / 16; c += 2) {
         float f[16];
         acc_chunk(trow, c, f);
 #pragma unroll
@@ -461,10 +490,10 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
       if (threadIdx.x == 64) atomicExch(a.err, kErrInjected);
     } else {
 #pragma unroll 1
-      for (int g = rank; g < G; g += S) {
+      for (int g = rank + half * S; g < G; g += 2 * S) {
         float f[4] = {0.f, 0.f, 0.f, 0.f};
         if (S > 1) {
-#pragma unroll 1
+#pragma unroll 4
           for (int s = 0; s < S; ++s) {
             const uint4 p = recv[(s * gpo + g / S) * kSmM + row];
             f[0] += __uint_as_float(p.x);
