@@ -31,7 +31,7 @@
 //               thread; tcgen05.commit frees ring slots and publishes
 //               accumulators
 //   warps 2-9   epilogue: warp w reads TMEM lane quarter w % 4 (32 rows);
-//               with K whole, warps 2-5 write 32-column chunks; with K split,
+//               with K whole, warps 2-5 write 16-column blocks; with K split,
 //               warps 2-5 and 6-9 take alternate chunks of the partial and
 //               the two 16-column halves of every owned chunk
 // Whole K (enough output tiles for every SM): one CTA per SM, persistent over
@@ -67,11 +67,9 @@ constexpr int B_BYTES = BN * BK * 2;          // 32 KB: the 16h and l planes
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int TMEM_COLS = 2 * BN;             // double-buffered accumulator
 constexpr int kGemmThreads = 320;             // TMA, MMA and 8 epilogue warps
-constexpr int TR_STRIDE = 33;                 // padded transpose rows (words)
 constexpr size_t SMEM_RING = (size_t)STAGES * STAGE_BYTES;
-constexpr int TR16_STRIDE = 17;               // padded 16-column transpose rows
-constexpr size_t SMEM_TR = (size_t)8 * 32 * TR16_STRIDE * 4 > (size_t)4 * 32 * TR_STRIDE * 4
-                               ? (size_t)8 * 32 * TR16_STRIDE * 4 : (size_t)4 * 32 * TR_STRIDE * 4;
+constexpr int TR16_STRIDE = 20;               // padded 16-column transpose rows (words, 16-byte aligned)
+constexpr size_t SMEM_TR = (size_t)8 * 32 * TR16_STRIDE * 4;
 constexpr size_t SMEM_BARS = 256;
 constexpr size_t kGemmSmem = 1024 + SMEM_RING + SMEM_TR + SMEM_BARS;
 static_assert(kGemmSmem <= 227 * 1024, "shared memory per CTA");
@@ -119,83 +117,66 @@ __device__ __forceinline__ float column_scale(const GemmParams& p, int n) {
   return (p.y && n < p.N) ? __ldg(p.scale + n) : 0.f;
 }
 
-// One warp writes a 32-row x 32-column chunk of fp32 sums in accumulator
-// units (v[i] = column col0 + i of row row0 + lane): transposed through shared
-// memory so that each store instruction covers 32 consecutive columns of one
-// row; acc = the exact integer, y = s * float(acc) with sc = the scale of
-// column col0 + lane.
-__device__ __forceinline__ void store_chunk(const GemmParams& p, uint32_t* tr,
-                                            const uint32_t (&v)[32], int row0, int col0,
-                                            float sc) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) tr[lane * TR_STRIDE + i] = v[i];
-  __syncwarp();
-  const int n = col0 + lane;
-  const int nrows = p.T - row0 < 32 ? p.T - row0 : 32;
-  if (n < p.N) {
-    int32_t* acc = p.acc ? p.acc + (int64_t)row0 * p.N + n : nullptr;
-    float* y = p.y ? p.y + (int64_t)row0 * p.N + n : nullptr;
-    if (nrows == 32) {
-      // full chunk: all 32 shared-memory reads into registers before the
-      // first global store, so no store orders a later read
-      int val[32];
-#pragma unroll
-      for (int rr = 0; rr < 32; ++rr)
-        val[rr] = __float2int_rn(__uint_as_float(tr[rr * TR_STRIDE + lane]) * kUnitsPerSpike);
-      if (acc) {
-#pragma unroll
-        for (int rr = 0; rr < 32; ++rr) acc[(int64_t)rr * p.N] = val[rr];
-      }
-      if (y) {
-#pragma unroll
-        for (int rr = 0; rr < 32; ++rr) y[(int64_t)rr * p.N] = scale_out(sc, val[rr]);
-      }
-    } else {
-      for (int rr = 0; rr < nrows; ++rr) {
-        const int val = __float2int_rn(__uint_as_float(tr[rr * TR_STRIDE + lane]) * kUnitsPerSpike);
-        if (acc) acc[(int64_t)rr * p.N] = val;
-        if (y) y[(int64_t)rr * p.N] = scale_out(sc, val);
-      }
-    }
-  }
-  __syncwarp();
-}
-
 // One warp writes a 32-row x 16-column block of fp32 sums in accumulator
-// units (v[i] = column col0 + i of row row0 + lane) through a shared-memory
-// transpose: lane l then holds column col0 + (l & 15) of rows 2 rr + (l >> 4),
-// so each store instruction covers 64 contiguous bytes of two rows.  sc = the
-// scale of column col0 + (lane & 15).
+// units (v[i] = column col0 + i of row row0 + lane; col0 and N are multiples of
+// 16) through a shared-memory transpose: lane l then holds columns 4 (l & 3) ..
+// + 3 of rows (l >> 2) + 8 i, so each store instruction writes 16 bytes per
+// lane, 64 contiguous bytes of 8 rows.  acc = the exact integer, y = s *
+// float(acc); sc = the scale of column col0 + (lane & 15).  (With 4-byte stores
+// of two rows the 16 stores per block and array bounded the epilogue: 11 us
+// for a 128 x 256 tile.)
 __device__ __forceinline__ void store_block16(const GemmParams& p, uint32_t* tr,
                                               const uint32_t (&v)[16], int row0, int col0,
                                               float sc) {
   const int lane = threadIdx.x & 31;
+  uint4* w = reinterpret_cast<uint4*>(tr + lane * TR16_STRIDE);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) tr[lane * TR16_STRIDE + i] = v[i];
+  for (int i = 0; i < 4; ++i) w[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
   __syncwarp();
-  const int col = lane & 15, sub = lane >> 4;
-  const int n = col0 + col;
-  int val[16];
+  const int c4 = 4 * (lane & 3), r8 = lane >> 2;
+  int4 val[4];
 #pragma unroll
-  for (int r2 = 0; r2 < 16; ++r2)
-    val[r2] = __float2int_rn(__uint_as_float(tr[(2 * r2 + sub) * TR16_STRIDE + col]) * kUnitsPerSpike);
+  for (int i = 0; i < 4; ++i) {
+    const uint4 x = *reinterpret_cast<const uint4*>(tr + (r8 + 8 * i) * TR16_STRIDE + c4);
+    val[i] = make_int4(__float2int_rn(__uint_as_float(x.x) * kUnitsPerSpike),
+                       __float2int_rn(__uint_as_float(x.y) * kUnitsPerSpike),
+                       __float2int_rn(__uint_as_float(x.z) * kUnitsPerSpike),
+                       __float2int_rn(__uint_as_float(x.w) * kUnitsPerSpike));
+  }
+  float s4[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s4[i] = __shfl_sync(0xffffffffu, sc, c4 + i);
   __syncwarp();
-  if (n < p.N) {
-    const int nrows = p.T - row0 < 32 ? p.T - row0 : 32;
-    if (p.acc) {
-      int32_t* acc = p.acc + (int64_t)(row0 + sub) * p.N + n;
+  const int n = col0 + c4;
+  const int nrows = p.T - row0;
+  // rows are 4 N bytes apart, a multiple of 64: the bases decide
+  const bool vec = ((reinterpret_cast<uintptr_t>(p.acc) | reinterpret_cast<uintptr_t>(p.y)) & 15u) == 0;
 #pragma unroll
-      for (int r2 = 0; r2 < 16; ++r2)
-        if (2 * r2 + sub < nrows) acc[(int64_t)(2 * r2) * p.N] = val[r2];
-    }
-    if (p.y) {
-      float* y = p.y + (int64_t)(row0 + sub) * p.N + n;
-#pragma unroll
-      for (int r2 = 0; r2 < 16; ++r2)
-        if (2 * r2 + sub < nrows) y[(int64_t)(2 * r2) * p.N] = scale_out(sc, val[r2]);
+  for (int i = 0; i < 4; ++i) {
+    const int r = r8 + 8 * i;
+    if (r >= nrows || n >= p.N) continue;      // (n >= N for all columns of the block or none)
+    const int64_t off = (int64_t)(row0 + r) * p.N + n;
+    const float4 yv = make_float4(scale_out(s4[0], val[i].x), scale_out(s4[1], val[i].y),
+                                  scale_out(s4[2], val[i].z), scale_out(s4[3], val[i].w));
+    if (vec) {
+      if (p.acc) *reinterpret_cast<int4*>(p.acc + off) = val[i];
+      if (p.y) *reinterpret_cast<float4*>(p.y + off) = yv;
+    } else {
+      if (p.acc) {
+        p.acc[off] = val[i].x;
+        p.acc[off + 1] = val[i].y;
+        p.acc[off + 2] = val[i].z;
+        p.acc[off + 3] = val[i].w;
+      }
+      if (p.y) {
+        p.y[off] = yv.x;
+        p.y[off + 1] = yv.y;
+        p.y[off + 2] = yv.z;
+        p.y[off + 3] = yv.w;
+      }
     }
   }
+  __syncwarp();
 }
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
@@ -337,7 +318,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
       // works alone: no barrier joins the epilogue warps, so a warp that gives up
       // on a timed-out wait cannot strand the others.
       const int q = warp & 3;
-      uint32_t* tr = s_tr + (size_t)(warp - 2) * 32 * TR_STRIDE;
+      uint32_t* tr = s_tr + (size_t)(warp - 2) * 32 * TR16_STRIDE;
       int ab = 0;
       uint32_t aph = 0;
       for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
@@ -350,14 +331,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         }
         tc_fence_after();
         const int row0 = mb * BM + q * 32;
-        for (int c = 0; c < BN; c += 32) {
-          uint32_t v[32];
-          tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + c), v);
+        for (int c = 0; c < BN; c += 16) {
+          uint32_t v[16];
+          tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + c), v);
           if (a.p.fault == kFaultAbort) {    // test fault: the output stays unwritten
             if (lane == 0) atomicExch(a.p.err, kErrInjected);
             continue;
           }
-          store_chunk(a.p, tr, v, row0, nb * BN + c, column_scale(a.p, nb * BN + c + lane));
+          store_block16(a.p, tr, v, row0, nb * BN + c, column_scale(a.p, nb * BN + c + (lane & 15)));
         }
         tc_fence_before();
         __syncwarp();
