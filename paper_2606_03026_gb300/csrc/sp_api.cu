@@ -654,7 +654,7 @@ sp_status spike_proj_group_create(sp_group_t* group, const sp_plan_t* plans, int
   for (int j = 0; j < count; ++j) all_gemm = all_gemm && (plans[j]->flags & SP_PLAN_GEMM);
   if (all_gemm &&
       ((st = dev_alloc_zero(&g->gpart, (size_t)kGemmGroupSlots * kGemmPartialElems, s)) != SP_OK ||
-       (st = dev_alloc_zero(&g->gflags, (size_t)kGemmGroupSlots * 8, s)) != SP_OK)) {
+       (st = dev_alloc_zero(&g->gflags, (size_t)kGemmGroupFlags, s)) != SP_OK)) {
     group_free(g);
     return st;
   }
@@ -903,7 +903,7 @@ sp_status spike_proj_group_status(sp_group_t g, sp_stream_t stream) {
   SP_CUDA(cudaMemsetAsync(g->ws, 0, g->ws_elems * sizeof(int32_t), s));
   SP_CUDA(cudaMemsetAsync(g->tickets, 0, g->n_tickets * sizeof(uint32_t), s));
   if (g->gflags)
-    SP_CUDA(cudaMemsetAsync(g->gflags, 0, (size_t)kGemmGroupSlots * 8 * sizeof(uint32_t), s));
+    SP_CUDA(cudaMemsetAsync(g->gflags, 0, (size_t)kGemmGroupFlags * sizeof(uint32_t), s));
   SP_CUDA(cudaStreamSynchronize(s));
   return SP_EKERNEL;
 }

@@ -225,7 +225,22 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   // The set-up above overlaps the previous kernel of the stream (programmatic
-  // dependent launch); every global access below comes after it has finished.
+  // dependent launch), and so do the weight boxes of the first ring: the
+  // planes are plan-owned and written once, when the plan is made.  Every
+  // other global access comes after the previous kernel has finished.
+  int pre = 0;                              // ring slots whose weights are on their way
+  if (threadIdx.x == 0 && blockIdx.x < a.units) {
+    int tile, mb, nb, kb0, kb1;
+    unit_coords(a, blockIdx.x, tile, mb, nb, kb0, kb1);
+    pre = min(STAGES, kb1 - kb0);
+    for (int i = 0; i < pre; ++i) {
+      mbar_arrive_expect_tx(&full[i], STAGE_BYTES);
+      // test stall fault: CTA 0's first fill is never issued, so its MMA
+      // warp's bounded wait runs out
+      if (!(a.p.fault == kFaultStall && blockIdx.x == 0 && i == 0))
+        tma_load_2d(sB + (size_t)i * B_BYTES, &mapB, &full[i], (kb0 + i) * 2 * BK, nb * BN);
+    }
+  }
   pdl_launch_dependents();
   pdl_wait();
 
@@ -239,18 +254,21 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         int tile, mb, nb, kb0, kb1;
         unit_coords(a, u, tile, mb, nb, kb0, kb1);
         for (int kb = kb0; kb < kb1; ++kb) {
+          if (issued < pre) {               // the spikes of a slot that has its weights
+            if (!(a.p.fault == kFaultStall && blockIdx.x == 0 && issued == 0))
+              tma_load_2d(sA + (size_t)stage * A_BYTES, &mapA, &full[stage], kb * BK, mb * BM);
+            ++issued;
+            if (++stage == STAGES) { stage = 0; ph ^= 1u; }
+            continue;
+          }
           if (!mbar_wait(&empty[stage], ph ^ 1u, lim)) {
             *s_abort = 1;
             atomicExch(a.p.err, kErrMbarTimeout);
             break;
           }
           mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
-          // test stall fault: CTA 0's first fill is never issued, so its
-          // MMA warp's bounded wait runs out
-          if (!(a.p.fault == kFaultStall && blockIdx.x == 0 && issued == 0)) {
-            tma_load_2d(sA + (size_t)stage * A_BYTES, &mapA, &full[stage], kb * BK, mb * BM);
-            tma_load_2d(sB + (size_t)stage * B_BYTES, &mapB, &full[stage], kb * 2 * BK, nb * BN);
-          }
+          tma_load_2d(sA + (size_t)stage * A_BYTES, &mapA, &full[stage], kb * BK, mb * BM);
+          tma_load_2d(sB + (size_t)stage * B_BYTES, &mapB, &full[stage], kb * 2 * BK, nb * BN);
           ++issued;
           if (++stage == STAGES) { stage = 0; ph ^= 1u; }
         }
@@ -505,23 +523,23 @@ struct GroupUnit {
   int j;                  // member
   int mb, nb;             // this CTA's row tile and the channel tile
   int kb0, kb1;           // K blocks [kb0, kb1)
-  int role;               // 0 whole K, 1 owner of a split unit, 2 helper
-  int slot;               // helper: its partial slot; owner: its first helper's
+  int S, s;               // K range s of S (S = 1: whole K)
+  int slot;               // S > 1: the partial slot of range 0 (range i: + i)
 };
 
 template <int CL>
 __device__ __forceinline__ GroupUnit group_unit(const GemmGroupArgs& g, int v, int rank) {
   GroupUnit r;
-  int u = v, s = 0, S = 1;
-  r.role = 0;
+  int u = v;
+  r.s = 0;
+  r.S = 1;
   r.slot = 0;
   if (v >= g.whole) {
-    S = g.tail_s;
-    const int t = (v - g.whole) / S;
-    s = v - g.whole - t * S;
+    r.S = g.tail_s;
+    const int t = (v - g.whole) / r.S;
+    r.s = v - g.whole - t * r.S;
     u = g.whole + t;
-    r.role = s == 0 ? 1 : 2;
-    r.slot = t * (S - 1) + (s == 0 ? 0 : s - 1);
+    r.slot = t * r.S;
   }
   r.j = member_of(g, u);
   const GemmMember& M = g.m[r.j];
@@ -529,8 +547,8 @@ __device__ __forceinline__ GroupUnit group_unit(const GemmGroupArgs& g, int v, i
   const int mg = unit / M.tiles_n;
   r.nb = unit - mg * M.tiles_n;
   r.mb = mg * CL + rank;
-  r.kb0 = s * M.nkb / S;
-  r.kb1 = (s + 1) * M.nkb / S;
+  r.kb0 = r.s * M.nkb / r.S;
+  r.kb1 = (r.s + 1) * M.nkb / r.S;
   return r;
 }
 
@@ -593,27 +611,56 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
   else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
+  const uint32_t full_cl = kPair ? cluster_addr(full, 0) : 0u;   // even CTA's full[0]
+  // The weight boxes of the first ring before the dependency wait (the planes
+  // are plan-owned and written once, when the plan is made).
+  GroupUnit first = {};
+  int pre = 0;                              // ring slots whose weights are on their way
+  if (threadIdx.x == 0 && cluster < g.total) {
+    first = group_unit<CL>(g, cluster, rank);
+    const GemmMember& M = g.m[first.j];
+    tma_prefetch_desc(&M.b);
+    tma_prefetch_desc(&M.a);
+    pre = min(ST, first.kb1 - first.kb0);
+    for (int i = 0; i < pre; ++i) {
+      uint8_t* dB = sB + (size_t)i * C::kBStage;
+      const int x = (first.kb0 + i) * 2 * BK, y = first.nb * BN + rank * (BN / CL);
+      if (leader) mbar_arrive_expect_tx(&full[i], C::kStageTx);
+      if (kPair) tma_load_2d_pair(dB, &M.b, full_cl + (uint32_t)i * 8u, x, y);
+      else tma_load_2d(dB, &M.b, &full[i], x, y);
+    }
+  }
   pdl_launch_dependents();
   pdl_wait();
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
     if (lane == 0) {
-      const uint32_t full_cl = kPair ? cluster_addr(full, 0) : 0u;   // even CTA's full[0]
       int stage = 0;
       uint32_t ph = 0;
       int issued = 0;
-      int last = -1;
-      for (int v = cluster; v < g.total && !*s_abort; v += nclusters) {
-        const GroupUnit U = group_unit<CL>(g, v, rank);
+      GroupUnit U = first, next = first;
+      for (int v = cluster; v < g.total && !*s_abort; v += nclusters, U = next) {
         const GemmMember& M = g.m[U.j];
-        if (U.j != last) {
-          tma_prefetch_desc(&M.a);
-          tma_prefetch_desc(&M.b);
-          last = U.j;
-        }
         const int mb = U.mb, nb = U.nb;
+        const int ahead = min(U.kb0 + 3, U.kb1 - 1);
         for (int kb = U.kb0; kb < U.kb1; ++kb) {
+          if (kb == ahead && v + nclusters < g.total) {
+            // the next unit and its descriptors, while this one's blocks
+            // are in flight: fetched at its first block they left the MMA
+            // idle for a microsecond or two per unit
+            next = group_unit<CL>(g, v + nclusters, rank);
+            tma_prefetch_desc(&g.m[next.j].a);
+            tma_prefetch_desc(&g.m[next.j].b);
+          }
+          if (issued < pre) {               // the spikes of a slot that has its weights
+            uint8_t* dA = sA + (size_t)stage * A_BYTES;
+            if (kPair) tma_load_2d_pair(dA, &M.a, full_cl + (uint32_t)stage * 8u, kb * BK, mb * BM);
+            else tma_load_2d(dA, &M.a, &full[stage], kb * BK, mb * BM);
+            ++issued;
+            if (++stage == ST) { stage = 0; ph ^= 1u; }
+            continue;
+          }
           if (!mbar_wait(&empty[stage], ph ^ 1u)) {
             *s_abort = 1;
             atomicExch(g.err, kErrMbarTimeout);
@@ -652,8 +699,10 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
       uint32_t ph = 0;
       int ab = 0;
       uint32_t aph = 0;
-      for (int v = cluster; v < g.total && !*s_abort; v += nclusters) {
-        const GroupUnit U = group_unit<CL>(g, v, rank);
+      GroupUnit U = {}, next = {};
+      if (cluster < g.total) U = group_unit<CL>(g, cluster, rank);
+      for (int v = cluster; v < g.total && !*s_abort; v += nclusters, U = next) {
+        const int ahead = min(U.kb0 + 3, U.kb1 - 1);
         if (!mbar_wait(&tempty[ab], aph ^ 1u)) {
           *s_abort = 1;
           atomicExch(g.err, kErrMbarTimeout);
@@ -684,6 +733,7 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
           }
           if (kPair) mma_commit_pair(&empty[stage], 3);
           else mma_commit(&empty[stage]);
+          if (kb == ahead && v + nclusters < g.total) next = group_unit<CL>(g, v + nclusters, rank);
           if (++stage == ST) { stage = 0; ph ^= 1u; }
         }
         if (!ok) {
@@ -724,13 +774,21 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
           tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + half * 16);
       // this warp's 32 x 16 block of chunk c inside a 128 x 256 partial tile
       const size_t pofs = (size_t)(q * 32 + lane) + (size_t)half * 16 * 128;
-      if (U.role == 2) {
-        // helper: the partial of this CTA's rows to its slot, then this
-        // warp's flag (every lane's stores ordered before it)
-        float* dst = g.part + (size_t)(U.slot * CL + rank) * (BM * BN) + pofs;
+      const int S = U.S;
+      // this warp's flags: range i's partial is ready for range k at (i, k)
+      const auto flag = [&](int i, int k) {
+        return g.flags + ((size_t)((U.slot + i) * CL + rank) * 8 + (warp - 2)) * kGemmGroupMaxTail + k;
+      };
+      bool ok = true;
+      if (S > 1) {
+        // the chunks of the other ranges (chunk c belongs to range c mod S)
+        // to this range's slot, then their flags (every lane's stores ordered
+        // before them)
+        float* dst = g.part + (size_t)((U.slot + U.s) * CL + rank) * (BM * BN) + pofs;
         if (live) {
 #pragma unroll 1
           for (int c = 0; c < CPT; ++c) {
+            if (c % S == U.s) continue;
             uint32_t v[16];
             tmem_ld16(trow + (uint32_t)(c * 32), v);
 #pragma unroll
@@ -740,50 +798,45 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
         }
         __threadfence();
         __syncwarp();
-        if (lane == 0) st_release(g.flags + (size_t)(U.slot * CL + rank) * 8 + (warp - 2), 1u);
-      } else {
-        const int helpers = U.role == 1 ? g.tail_s - 1 : 0;
-        bool ok = true;
-        for (int h = 0; h < helpers && ok; ++h) {
-          // owner: wait (bounded) for the helper's warp that wrote this block
-          const uint32_t* f = g.flags + (size_t)((U.slot + h) * CL + rank) * 8 + (warp - 2);
+        if (lane < S && lane != U.s) {
+          st_release(flag(U.s, lane), 1u);
+          // and wait (bounded) for theirs
           const long long t0 = clock64();
-          while (ld_acquire(f) == 0u) {
+          while (ld_acquire(flag(lane, U.s)) == 0u) {
             if (clock64() - t0 > kWaitLimitCycles) {
               ok = false;
               break;
             }
           }
         }
-        __syncwarp();
-        if (!ok) {
-          *s_abort = 1;
-          if (lane == 0) atomicExch(g.err, kErrFlagTimeout);
-        } else if (live) {
-#pragma unroll 1
-          for (int c = 0; c < CPT; ++c) {
-            const int col0 = U.nb * BN + c * 32 + half * 16;
-            uint32_t v[16];
-            tmem_ld16(trow + (uint32_t)(c * 32), v);
-            for (int h = 0; h < helpers; ++h) {
-              const float* src = g.part + (size_t)((U.slot + h) * CL + rank) * (BM * BN) + pofs +
-                                 (size_t)c * 32 * 128;
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                v[i] = __float_as_uint(__uint_as_float(v[i]) + __ldcg(src + (size_t)i * 128));
-            }
-            if (M.p.fault == kFaultAbort) {   // test fault: the output stays unwritten
-              if (lane == 0) atomicExch(g.err, kErrInjected);
-              continue;
-            }
-            store_block16(M.p, tr, v, row0, col0, column_scale(M.p, col0 + (lane & 15)));
-          }
-        }
-        __syncwarp();
-        if (lane == 0)
-          for (int h = 0; h < helpers; ++h)
-            g.flags[(size_t)((U.slot + h) * CL + rank) * 8 + (warp - 2)] = 0u;   // for the next launch
+        ok = __all_sync(0xffffffffu, ok);
       }
+      if (!ok) {
+        *s_abort = 1;
+        if (lane == 0) atomicExch(g.err, kErrFlagTimeout);
+      } else if (live) {
+#pragma unroll 1
+        for (int c = U.s; c < CPT; c += S) {
+          const int col0 = U.nb * BN + c * 32 + half * 16;
+          uint32_t v[16];
+          tmem_ld16(trow + (uint32_t)(c * 32), v);
+          for (int h = 0; h < S; ++h) {
+            if (h == U.s) continue;
+            const float* src = g.part + (size_t)((U.slot + h) * CL + rank) * (BM * BN) + pofs +
+                               (size_t)c * 32 * 128;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              v[i] = __float_as_uint(__uint_as_float(v[i]) + __ldcg(src + (size_t)i * 128));
+          }
+          if (M.p.fault == kFaultAbort) {   // test fault: the output stays unwritten
+            if (lane == 0) atomicExch(g.err, kErrInjected);
+            continue;
+          }
+          store_block16(M.p, tr, v, row0, col0, column_scale(M.p, col0 + (lane & 15)));
+        }
+      }
+      __syncwarp();
+      if (lane < S && lane != U.s) *flag(lane, U.s) = 0u;   // for the next launch
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -1122,11 +1175,11 @@ cudaError_t launch_group_cl(const GemmGroupArgs& a, cudaStream_t s) {
   const int r = a.units % clusters;
   if (a.part && a.flags && r > 0) {
     int S = clusters / r;
-    if (S > 6) S = 6;
+    if (S > kGemmGroupMaxTail) S = kGemmGroupMaxTail;
     int min_nkb = 1 << 30;
     for (int j = 0; j < a.count; ++j)
       if (a.m[j].unit_end > a.units - r && a.m[j].nkb < min_nkb) min_nkb = a.m[j].nkb;
-    while (S > 1 && (min_nkb < 4 * S || r * (S - 1) * CL > kGemmGroupSlots)) --S;
+    while (S > 1 && (min_nkb < 4 * S || r * S * CL > kGemmGroupSlots)) --S;
     if (S > 1) {
       b.whole = a.units - r;
       b.tail_s = S;
