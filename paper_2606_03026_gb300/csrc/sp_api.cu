@@ -333,6 +333,7 @@ sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld,
     SP_CUDA(launch_spikes_to_01(spikes, fmt, ld, T, p->K, p->Kp, p->Xs, count, s));
   }
   GemmParams g;
+  g.count = in_place ? SpikeCount{} : count;
   g.scale = p->scale;
   g.acc = acc;
   g.y = y;
@@ -390,7 +391,7 @@ sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
     // the count cannot change the choice: the GEMM is enqueued at once, the
     // count comes with it (spike_proj_last_dispatch waits for it), and the
     // host does not.  173 byte rows of 1990 columns: 31.9 us a call with the
-    // count, its copy and the synchronisation ahead of the GEMM, 14.0
+    // count, its copy and the synchronisation ahead of the GEMM, 11.6
     // without.  A stream being captured takes the other way and is refused
     // by its synchronisation.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
@@ -760,6 +761,7 @@ sp_status spike_proj_group_prefill(sp_group_t g, const void* const* X, sp_fmt fm
     M.p.part = nullptr;
     M.p.part_units = 0;
     M.p.fault = g->fault;
+    M.p.count = SpikeCount{};
     M.tiles_n = tn[j];
     M.nkb = p->Kp / 64;
     M.unit_begin = (int32_t)units;

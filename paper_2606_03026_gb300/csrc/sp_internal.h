@@ -131,6 +131,17 @@ struct UnionParams {
 };
 constexpr int kUnionMaxRows = 256;      // rows per union launch
 
+// Where a count of active spikes (sum over the rows of |A_t|) goes.  The
+// counting kernel's blocks add into dev[0]; then either the last of them (by
+// tickets in dev[1]) or the GEMM that follows on the stream publishes it:
+// host[0] = count, then host[1] = seq (page-locked memory, visible without a
+// copy), dev left zero for the next call.
+struct SpikeCount {
+  int32_t* dev;           // two words, zero between calls; null: no count
+  int32_t* host;
+  int32_t seq;
+};
+
 // Tensor-core (tcgen05) prefill GEMM operands.
 struct GemmParams {
   const float* scale;
@@ -141,6 +152,7 @@ struct GemmParams {
   float* part;            // split-K partials, part_units x (128 x 256) fp32
   int32_t part_units;
   int32_t fault;          // Fault armed for this launch
+  SpikeCount count;       // to publish (count.dev set), added up by the staging pass before
 };
 
 // One continuous-input projection as the dense kernel sees it (row-major
@@ -222,20 +234,11 @@ cudaError_t launch_probe_gather(const uint8_t* base, const uint32_t* offsets16, 
 cudaError_t launch_gather(const GatherParams1& p, cudaStream_t s);
 cudaError_t launch_gather(const GatherParamsG& p, cudaStream_t s);
 cudaError_t launch_union(const UnionParams& p, cudaStream_t s);
-// Where a kernel that counts active spikes (sum over the rows of |A_t|) leaves
-// the count: the grid's blocks add into dev[0] and take tickets from dev[1];
-// the last one writes host[0] = count, then host[1] = seq (page-locked memory,
-// visible without a copy), and leaves dev zero for the next call.
-struct SpikeCount {
-  int32_t* dev;           // two words, zero between launches; null: no count
-  int32_t* host;
-  int32_t seq;
-};
-// Counts active spikes.
+// Counts active spikes and publishes the count.
 cudaError_t launch_density(const void* spikes, int fmt, int64_t ld, int B, int K,
                            const SpikeCount& count, cudaStream_t s);
-// Spike rows in any format -> bytes 0 / 1 [T][Kp] (zero past K), counted on the
-// way when count.dev is set.
+// Spike rows in any format -> bytes 0 / 1 [T][Kp] (zero past K), added up in
+// count.dev[0] on the way when that is set (the GEMM publishes it).
 cudaError_t launch_spikes_to_01(const void* spikes, int fmt, int64_t ld, int T, int K, int Kp,
                                 uint8_t* Xs, const SpikeCount& count, cudaStream_t s);
 

@@ -55,10 +55,20 @@ __device__ __forceinline__ const void* spike_row(const void* base, int fmt, int6
              : static_cast<const void*>(reinterpret_cast<const uint8_t*>(base) + row * ld);
 }
 
-// Adds the calling thread's share of a launch's spike count and, in the last
-// block to arrive, publishes the total (SpikeCount).  Every thread of the
-// grid calls it once; blockDim.x is a multiple of 32, at most 1024.
-__device__ __forceinline__ void count_spikes(int mine, const SpikeCount& c) {
+// Publishes the count in c.dev[0] and clears it (one thread, after every
+// block's addition).
+__device__ __forceinline__ void publish_count(const SpikeCount& c) {
+  volatile int32_t* host = c.host;
+  host[0] = atomicExch(c.dev, 0);
+  c.dev[1] = 0;
+  __threadfence_system();
+  host[1] = c.seq;
+}
+
+// Adds the calling thread's share to the count; `publish`: the last block to
+// arrive publishes it.  Every thread of the grid calls it once; blockDim.x is a
+// multiple of 32, at most 1024.
+__device__ __forceinline__ void count_spikes(int mine, const SpikeCount& c, bool publish) {
   __shared__ int s_sum[32];
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
@@ -68,14 +78,11 @@ __device__ __forceinline__ void count_spikes(int mine, const SpikeCount& c) {
   int sum = 0;
   for (int w = 0; w < (int)blockDim.x / 32; ++w) sum += s_sum[w];
   if (sum) atomicAdd(c.dev, sum);
+  if (!publish) return;
   __threadfence();
   if (atomicAdd(c.dev + 1, 1) != (int)gridDim.x - 1) return;
   __threadfence();
-  volatile int32_t* host = c.host;
-  host[0] = atomicExch(c.dev, 0);
-  c.dev[1] = 0;
-  __threadfence_system();
-  host[1] = c.seq;
+  publish_count(c);
 }
 
 // Warp-cooperative compaction of nw <= 32 words into ascending column

@@ -17,6 +17,7 @@
 //      the tile back in 16-byte groups, 16 loads per thread in flight, writes
 //      acc and y = s * float(acc) for every row, and re-zeroes the workspace.
 //      Nothing waits on another CTA.
+#include "sp_ptx.cuh"
 #include "sp_spikes.cuh"
 
 namespace sp {
@@ -209,6 +210,8 @@ union_kernel(const __grid_constant__ UnionParams p) {
 // Density probe: one thread per (row, 32-column word), grid-stride.
 __global__ void density_kernel(const void* spikes, int fmt, int64_t ld, int B, int K,
                                SpikeCount count) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int nw = ceil_div(K, 32);
   const int64_t total_words = (int64_t)nw * B;
   int total = 0;
@@ -218,7 +221,7 @@ __global__ void density_kernel(const void* spikes, int fmt, int64_t ld, int B, i
     const int w = (int)(i - (int64_t)t * nw);
     total += __popc(spike_word(spike_row(spikes, fmt, t, ld), fmt, K, 32 * w));
   }
-  count_spikes(total, count);
+  count_spikes(total, count, true);
 }
 
 int g_union_grid = 0;
@@ -255,8 +258,7 @@ cudaError_t launch_density(const void* spikes, int fmt, int64_t ld, int B, int K
   int64_t grid = (words + threads - 1) / threads;
   if (grid > 2048) grid = 2048;
   if (grid < 1) grid = 1;
-  density_kernel<<<(int)grid, threads, 0, s>>>(spikes, fmt, ld, B, K, count);
-  return cudaGetLastError();
+  return launch_pdl(density_kernel, dim3((unsigned)grid), dim3(threads), 0, s, spikes, fmt, ld, B, K, count);
 }
 
 }  // namespace sp
