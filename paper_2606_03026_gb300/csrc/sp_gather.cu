@@ -369,19 +369,20 @@ gather_kernel(const __grid_constant__ GatherParamsT<NP> p) {
 // tiles of its cluster are doing.  (Ending with a release / acquire cluster
 // barrier instead cost 0.5 us per 22-block decode step.)
 constexpr int kClusterLoads = 9;                   // column loads per lane in registers (64 registers)
-// and in shared memory: 8 for a group (4 CTAs per SM), 16 for a single
-// projection's clusters of 12 or 16 (fewer CTAs, each with more columns)
-template <int CL> constexpr int cluster_slots() { return CL > 8 ? 16 : 8; }
-template <int CL>
-using ClusterSmem = UnitSmem<kGatherClusterWarps, kGatherClusterMaxCK, cluster_slots<CL>()>;
+// and in shared memory (S): 8 for a group of projections (4 CTAs per SM), 16
+// for a single projection's clusters of 12 or 16 (fewer CTAs, each with more
+// columns) and for the rows of a batch (rates up to 0.2: a warp's share of a
+// chunk of 1024 columns then still loads in one round)
+template <int S>
+using ClusterSmem = UnitSmem<kGatherClusterWarps, kGatherClusterMaxCK, S>;
 
 // kLif: the fused spike producer (a separate instantiation, so that the plain
 // decode carries none of its code)
-template <int NP, bool kLif, int CL>
+template <int NP, bool kLif, int CL, int S>
 __global__ void __launch_bounds__(kGatherClusterThreads, 4)
 gather_cluster_kernel(const __grid_constant__ GatherParamsT<NP> p) {
-  extern __shared__ __align__(16) uint8_t dyn_smem[];   // ClusterSmem<CL>, sized at launch
-  ClusterSmem<CL>& sm = *reinterpret_cast<ClusterSmem<CL>*>(dyn_smem);
+  extern __shared__ __align__(16) uint8_t dyn_smem[];   // ClusterSmem<S>, sized at launch
+  ClusterSmem<S>& sm = *reinterpret_cast<ClusterSmem<S>*>(dyn_smem);
   // [sender chunk][owned group]: kch * ceil(128 / kch) < 128 + kch entries
   __shared__ __align__(16) int4 s_recv[kGatherNT / 4 + CL];
   __shared__ uint32_t s_lif[kLif ? kGatherClusterMaxCK / 32 : 1];   // LIF mode: the chunk's spike words
@@ -450,7 +451,7 @@ gather_cluster_kernel(const __grid_constant__ GatherParamsT<NP> p) {
     }
     __syncthreads();
   }
-  unit_partial<kGatherClusterWarps, kGatherClusterMaxCK, kClusterLoads, cluster_slots<CL>()>(
+  unit_partial<kGatherClusterWarps, kGatherClusterMaxCK, kClusterLoads, S>(
       sm, P, kLif ? nullptr : spike_row(p.spikes, p.fmt, j, p.ld_spikes), p.fmt, n0, kc * P.ck,
       P.ck, kLif ? s_lif : nullptr);
   // the owner's scales, read now: their load overlaps the exchange instead
@@ -512,7 +513,7 @@ cudaError_t set_carveout(Kern kernel, std::atomic<uint64_t>& done) {
 }
 
 // Clusters of the cluster form that can be resident at once (per device).
-template <int NP, bool kLif, int CL>
+template <int NP, bool kLif, int CL, int S>
 int cluster_capacity() {
   static std::atomic<int> cap[64];
   int dev = 0;
@@ -527,10 +528,10 @@ int cluster_capacity() {
   attr.val.clusterDim.z = 1;
   cfg.gridDim = dim3(CL, 1, 1);
   cfg.blockDim = dim3(kGatherClusterThreads, 1, 1);
-  cfg.dynamicSmemBytes = sizeof(ClusterSmem<CL>);
+  cfg.dynamicSmemBytes = sizeof(ClusterSmem<S>);
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, gather_cluster_kernel<NP, kLif, CL>, &cfg) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveClusters(&n, gather_cluster_kernel<NP, kLif, CL, S>, &cfg) != cudaSuccess ||
       n < 1) {
     (void)cudaGetLastError();
     n = -1;
@@ -541,16 +542,54 @@ int cluster_capacity() {
 
 // Resident-cluster count of the kernel the launch will use (0 on failure).
 template <int NP>
-int capacity_for(bool lif, int CL) {
-  if (lif) return cluster_capacity<NP, true, 6>();
+int capacity_for(bool lif, int CL, int S) {
+  if (lif) return cluster_capacity<NP, true, 6, 8>();
   switch (CL) {
-    case 16: return cluster_capacity<NP, false, 16>();
-    case 12: return cluster_capacity<NP, false, 12>();
-    default: return cluster_capacity<NP, false, 6>();
+    case 16: return cluster_capacity<NP, false, 16, 16>();
+    case 12: return cluster_capacity<NP, false, 12, 16>();
+    default:
+      if constexpr (NP > 1)
+        if (S == 16) return cluster_capacity<NP, false, 6, 16>();
+      return cluster_capacity<NP, false, 6, 8>();
   }
 }
 
-// Fills the cluster-form fields of q and the cluster size *cl_out; false
+// The rows of a batch leave most SMs idle with clusters of 6, and at spike
+// rates up to 0.2 a warp's share of a chunk of 1024 columns takes two rounds
+// of loads with 8 shared-memory slots.  So a few rows (at most kSpreadMaxCtas
+// CTAs) take clusters of 12 with chunks of at least 384 columns, and more (at
+// most kRowsMaxCtas CTAs) clusters of 6 with 16 slots.  us a call at 1536 x 6144,
+// rates U(0.05, 0.2) / all 0.05, before and after: 2 rows 4.3 / 3.2 -> 3.6 /
+// 3.2, 4 rows 4.9 / 3.4 -> 4.6 / 3.35, 8 rows 6.0 / 3.8 -> 5.65 / 3.6, 12 rows
+// 7.9 / 4.9 -> 6.3 / 3.9.  Past the lines the other side is faster: 8 rows in
+// clusters of 12 take 5.2 but 4.3 at 0.05, 16 rows with 16 slots 7.3 against
+// 7.2.  The projections of a decode step keep clusters of 6 with 8 slots: at a
+// rate of 0.1 one round suffices (2 blocks: 3.8, in clusters of 16 4.05).
+constexpr int kSpreadMaxCtas = 120;
+constexpr int kRowsMaxCtas = 228;
+
+// Sets the chunking of a batch's rows for clusters of 12; false when they take
+// clusters of 6.
+template <int NP>
+bool rows_spread(GatherParamsT<NP>& q) {
+  const GatherProblem& P = q.prob[0];        // the rows are alike
+  int kch = 12;
+  while (kch > 1 && (12 % kch != 0 || ceil_div(ceil_div(P.K, kch), 32) * 32 < 384)) --kch;
+  if (ceil_div(ceil_div(P.K, kch), 32) * 32 > kGatherClusterMaxCK) return false;
+  const int tpc = 12 / kch, ntiles = gather_ntiles(P.N);
+  const int ncl = ceil_div(ntiles, tpc);
+  if (4 * (ncl * tpc - ntiles) > ncl * tpc) return false;   // more than a quarter idle
+  if (q.nprob * ncl * 12 > kSpreadMaxCtas || q.nprob * ncl > capacity_for<NP>(false, 12, 16)) return false;
+  for (int j = 0; j < q.nprob; ++j) {
+    q.prob[j].kch = kch;
+    q.prob[j].tpc = tpc;
+    q.prob[j].ncl = ncl;
+  }
+  return true;
+}
+
+// Fills the cluster-form fields of q, the cluster size *cl_out and the
+// shared-memory slots *s_out; false
 // when the launch does not fit the cluster form (several tokens, a chunk
 // count above the cluster size, or more clusters than can be resident at
 // once).  A group of projections takes clusters of 6 and the fewest chunks
@@ -562,9 +601,14 @@ int capacity_for(bool lif, int CL) {
 // work, all resident together); more take a (clusters x CL, problems) grid
 // in which the problems with fewer clusters leave idle CTAs.
 template <int NP>
-bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out) {
+bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out, int* s_out) {
   if (q.B != 1) return false;
   int CL = 6;
+  // the rows of a batch: problems that are alike and share one weight matrix
+  // (a caller's group may hold a plan twice, or plans over parts of one matrix)
+  bool rows = NP > 1 && q.nprob > 1 && !q.lif_I;
+  for (int j = 1; rows && j < q.nprob; ++j)
+    rows = q.prob[j].W == q.prob[0].W && q.prob[j].N == q.prob[0].N && q.prob[j].K == q.prob[0].K;
   if (q.nprob == 1 && !q.lif_I) {
     GatherProblem& P = q.prob[0];
     const int ntiles = gather_ntiles(P.N);
@@ -591,28 +635,34 @@ bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out) {
     P.tpc = CL / P.kch;
     P.ncl = ceil_div(ntiles, P.tpc);
   } else {
-    for (int j = 0; j < q.nprob; ++j) {
-      GatherProblem& P = q.prob[j];
-      // the fewest chunks (a divisor of the cluster size) of at most 1024 columns
-      int kch = 0;
-      for (int d = 1; d <= CL; ++d)
-        if (CL % d == 0 && ceil_div(P.K, d) <= kGatherClusterMaxCK) {
-          kch = d;
-          break;
-        }
-      if (kch == 0) return false;
-      P.kch = kch;
-      P.ck = ceil_div(ceil_div(P.K, kch), 32) * 32;
-      P.tpc = CL / kch;
-      P.ncl = ceil_div(gather_ntiles(P.N), P.tpc);
+    if (rows && rows_spread(q)) {
+      CL = 12;
+    } else {
+      for (int j = 0; j < q.nprob; ++j) {
+        GatherProblem& P = q.prob[j];
+        // the fewest chunks (a divisor of the cluster size) of at most 1024 columns
+        int kch = 0;
+        for (int d = 1; d <= CL; ++d)
+          if (CL % d == 0 && ceil_div(P.K, d) <= kGatherClusterMaxCK) {
+            kch = d;
+            break;
+          }
+        if (kch == 0) return false;
+        P.kch = kch;
+        P.tpc = CL / kch;
+        P.ncl = ceil_div(gather_ntiles(P.N), P.tpc);
+      }
     }
+    for (int j = 0; j < q.nprob; ++j) q.prob[j].ck = ceil_div(ceil_div(q.prob[j].K, q.prob[j].kch), 32) * 32;
   }
   int total = 0, widest = 0;
   for (int j = 0; j < q.nprob; ++j) {
     total += q.prob[j].ncl;
     if (q.prob[j].ncl > widest) widest = q.prob[j].ncl;
   }
-  if (total > capacity_for<NP>(q.lif_I != nullptr, CL)) return false;
+  int S = CL > 8 ? 16 : 8;
+  if (rows && CL == 6 && total * CL <= kRowsMaxCtas && total <= capacity_for<NP>(false, 6, 16)) S = 16;
+  if (total > capacity_for<NP>(q.lif_I != nullptr, CL, S)) return false;
   q.ncl_list = 0;
   if (total <= kGatherMaxClusterList && widest <= 0xff) {
     int c = 0;
@@ -626,6 +676,7 @@ bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out) {
     *grid_y = q.nprob;
   }
   *cl_out = CL;
+  *s_out = S;
   return true;
 }
 
@@ -653,21 +704,24 @@ cudaError_t cluster_attrs(Kern kernel, int CL, size_t smem, std::atomic<uint64_t
 
 template <int NP>
 cudaError_t launch_gather_t(const GatherParamsT<NP>& p, cudaStream_t s) {
-  static std::atomic<uint64_t> carve_t{0}, carve_c{0}, carve_l{0}, carve_12{0}, carve_16{0};
+  static std::atomic<uint64_t> carve_t{0}, carve_c{0}, carve_l{0}, carve_6{0}, carve_12{0}, carve_16{0};
   if (p.units_total <= 0 || p.B <= 0 || p.max_units <= 0) return cudaSuccess;
   // the attributes first: the resident-cluster counts depend on the carveout
-  cudaError_t e = p.lif_I
-                      ? cluster_attrs(gather_cluster_kernel<NP, true, 6>, 6, sizeof(ClusterSmem<6>), carve_l)
-                      : cluster_attrs(gather_cluster_kernel<NP, false, 6>, 6, sizeof(ClusterSmem<6>), carve_c);
-  if (e == cudaSuccess && !p.lif_I && p.nprob == 1) {
-    e = cluster_attrs(gather_cluster_kernel<NP, false, 12>, 12, sizeof(ClusterSmem<12>), carve_12);
-    if (e == cudaSuccess)
-      e = cluster_attrs(gather_cluster_kernel<NP, false, 16>, 16, sizeof(ClusterSmem<16>), carve_16);
+  cudaError_t e =
+      p.lif_I ? cluster_attrs(gather_cluster_kernel<NP, true, 6, 8>, 6, sizeof(ClusterSmem<8>), carve_l)
+              : cluster_attrs(gather_cluster_kernel<NP, false, 6, 8>, 6, sizeof(ClusterSmem<8>), carve_c);
+  if (e == cudaSuccess && !p.lif_I) {
+    e = cluster_attrs(gather_cluster_kernel<NP, false, 12, 16>, 12, sizeof(ClusterSmem<16>), carve_12);
+    if (e == cudaSuccess && p.nprob == 1)
+      e = cluster_attrs(gather_cluster_kernel<NP, false, 16, 16>, 16, sizeof(ClusterSmem<16>), carve_16);
+    if constexpr (NP > 1)
+      if (e == cudaSuccess)
+        e = cluster_attrs(gather_cluster_kernel<NP, false, 6, 16>, 6, sizeof(ClusterSmem<16>), carve_6);
   }
   if (e != cudaSuccess) return e;
   GatherParamsT<NP> q = p;
-  int gx = 0, gy = 0, CL = 6;
-  const bool cluster = cluster_form(q, &gx, &gy, &CL);
+  int gx = 0, gy = 0, CL = 6, S = 8;
+  const bool cluster = cluster_form(q, &gx, &gy, &CL, &S);
   if (p.lif_I && !cluster) return cudaErrorNotSupported;   // the fused producer needs the cluster form
   if (cluster) {
     cudaLaunchConfig_t cfg = {};
@@ -683,20 +737,15 @@ cudaError_t launch_gather_t(const GatherParamsT<NP>& p, cudaStream_t s) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (p.lif_I) {
-      cfg.dynamicSmemBytes = sizeof(ClusterSmem<6>);
-      return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, true, 6>, q);
-    }
+    cfg.dynamicSmemBytes = S == 16 ? sizeof(ClusterSmem<16>) : sizeof(ClusterSmem<8>);
+    if (p.lif_I) return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, true, 6, 8>, q);
     switch (CL) {
-      case 16:
-        cfg.dynamicSmemBytes = sizeof(ClusterSmem<16>);
-        return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 16>, q);
-      case 12:
-        cfg.dynamicSmemBytes = sizeof(ClusterSmem<12>);
-        return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 12>, q);
+      case 16: return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 16, 16>, q);
+      case 12: return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 12, 16>, q);
       default:
-        cfg.dynamicSmemBytes = sizeof(ClusterSmem<6>);
-        return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 6>, q);
+        if constexpr (NP > 1)
+          if (S == 16) return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 6, 16>, q);
+        return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 6, 8>, q);
     }
   }
   e = set_carveout(gather_kernel<NP>, carve_t);

@@ -295,3 +295,24 @@ def test_auto_counts_without_waiting(fmt, shift):
         assert_parity(acc, y, want_acc, want_y, f"auto {fmt} shift {shift} p {p}")
         plan.batched(x, fmt, T, ld, acc, y, "gather")
         assert plan.last_dispatch() == ("gemm", int(X.astype(np.int64).sum()))
+
+
+@pytest.mark.parametrize("N,K", [(1536, 6144), (1536, 1536), (512, 4000), (2064, 3000), (16, 300), (1040, 255),
+                                 (48, 12000), (528, 16384)])
+def test_batched_gather_cluster_shapes(N, K):
+    """The per-token gather over the cluster layouts a batch may take (clusters
+    of 16, 12 and 6, one to sixteen chunks, idle tile slots, and the ticket form
+    past them): every row equals the single decode and the oracle, at rates
+    with one and with several rounds of column loads."""
+    Qc, s, _ = synth.random_case(92, N, K)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=64)
+    rng = synth.rng_for(7302, N, K)
+    for B, p, fmt in ((2, 0.1, "bits"), (3, 1.0, "u8"), (5, 0.3, "bool8"), (8, 0.2, "bits"), (13, 0.5, "bits"),
+                      (24, 0.15, "u8"), (40, 0.05, "bits")):
+        X = synth.bernoulli(rng, (B, K), p)
+        X[B // 2] = 0
+        want_acc, want_y = oracle.project(Qc, s, N, K, X, "u8", ldq=Qc.shape[1])
+        rows = to_dev(synth.pack_bits(X)) if fmt == "bits" else to_dev(X)
+        acc, y = run_batched(plan, rows, fmt, B, rows.shape[1], N, "gather")
+        assert_parity(acc, y, want_acc, want_y, f"B={B} p={p} {fmt}")
+    assert plan.status() == sp.SP_OK

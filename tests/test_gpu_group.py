@@ -222,3 +222,32 @@ def test_large_mixed_group():
             assert (acc[j, N:] == 5).all(), "wrote past the member's N"
     assert group.status() == sp.SP_OK
     group.close()
+
+
+@pytest.mark.parametrize("order", [(0, 0), (0, 1, 0), (0, 2, 0), (1, 1, 1, 1), (0, 3, 0), (2, 0, 2, 1, 2)])
+def test_group_of_plans_that_share_weights(order):
+    """Groups that hold a plan more than once, with other plans between, or
+    plans over parts of the same matrix (fewer outputs, fewer columns): only
+    members that are all alike run as the rows of a batch do."""
+    Q, s, _ = synth.random_case(61, 1536, 6144)
+    Q2, s2, _ = synth.random_case(62, 512, 4000)
+    Wd, sd = to_dev(Q), to_dev(s)
+    members = [(Q, s, 1536, 6144, Wd, sd), (Q2, s2, 512, 4000, to_dev(Q2), to_dev(s2)),
+               (Q, s, 1040, 6144, Wd, sd), (Q, s, 1536, 500, Wd, sd)]
+    plans = {i: sp.Plan(m[4], m[5], m[2], m[3], ldw=m[0].shape[1]) for i, m in enumerate(members)}
+    group = sp.Group([plans[i] for i in order])
+    for p in (0.1, 1.0):
+        X = synth.bernoulli(synth.rng_for(7303, len(order)), (len(order), 6144), p)
+        bits = to_dev(synth.pack_bits(X))
+        acc = torch.full((len(order), 1536), -7, dtype=torch.int32, device=DEV)
+        y = torch.full((len(order), 1536), -7.0, device=DEV)
+        group.decode(bits, "bits", bits.shape[1], acc, y, 1536)
+        torch.cuda.synchronize()
+        for j, i in enumerate(order):
+            q, sc, N, K = members[i][:4]
+            want_acc, want_y = oracle.project(q, sc, N, K, X[j:j + 1, :K], "u8", ldq=q.shape[1])
+            assert_parity(acc[j:j + 1, :N].contiguous(), y[j:j + 1, :N].contiguous(), want_acc, want_y,
+                          f"order {order} member {j} p {p}")
+            assert torch.all(acc[j, N:] == -7)
+    assert group.status() == sp.SP_OK
+    group.close()
