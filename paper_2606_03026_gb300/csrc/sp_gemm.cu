@@ -53,6 +53,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "sp_gemm.h"
 #include "sp_ptx.cuh"
 #include "sp_spikes.cuh"
@@ -1059,15 +1061,25 @@ cudaError_t init_sms() {
 }
 
 // K splits for a T x N output: split only when the tiles alone leave SMs
-// idle, and only as far as every cluster stays resident in a single wave.
+// idle, and only as far as every cluster stays resident in a single wave.  A
+// range keeps at least 3 K blocks, or 2 where the launch is small (at most
+// kSplitSmallCtas CTAs) and that brings the 32-column chunks a CTA finishes
+// from more than 2 to fewer, or to 1: there the output of a CTA, not its K
+// loop, is the longest part.  us a call with at least 4 blocks / by this rule:
+// 100 x 1536 x 1536 9.15 / 8.1 (S = 6 / 8), 100 x 2048 x 768 8.8 / 8.0 (3 / 4),
+// 173 x 512 x 600 9.5 / 8.2 (2 / 5), 173 x 1024 x 1024 8.3 / 7.9 (4 / 8).  Past it
+// the exchange costs more than it saves: 100 x 2048 x 768 at S = 6 8.6, 512 x
+// 1024 x 1024 (128 CTAs) at S = 8 9.4 against 8.7 at 4.
+constexpr int kSplitSmallCtas = 64;
 int pick_splits(int T, int N, int Kp, int part_units) {
   const int tiles = ceil_div(T, BM) * ceil_div(N, BN);
   const int nkb = Kp / BK;
   int S = 1;
   if (tiles < g_num_sms) {
-    S = g_num_sms / tiles;
-    if (S > 8) S = 8;
-    if (S > nkb / 4) S = nkb / 4;
+    const int most = std::min(8, g_num_sms / tiles);
+    S = std::min(most, nkb / 3);
+    const int fine = std::min(most, nkb / 2);
+    if (tiles * fine <= kSplitSmallCtas && (S < 4 || fine == 8)) S = fine;
     if (S < 1) S = 1;
     while (S > 1) {
       const int kbps = ceil_div(nkb, S);

@@ -316,3 +316,20 @@ def test_batched_gather_cluster_shapes(N, K):
         acc, y = run_batched(plan, rows, fmt, B, rows.shape[1], N, "gather")
         assert_parity(acc, y, want_acc, want_y, f"B={B} p={p} {fmt}")
     assert plan.status() == sp.SP_OK
+
+
+@pytest.mark.parametrize("N,K", [(512, 600), (512, 130), (1024, 1024), (1536, 1536), (2048, 768), (1040, 1990),
+                                 (256, 64), (528, 448), (1536, 3000)])
+def test_gemm_split_shapes(N, K):
+    """The 128-row GEMM over the K splits it may take (1 to 8 ranges, of 1 to many
+    K blocks), at row counts around its tiles."""
+    Qc, s, _ = synth.random_case(93, N, K)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=512, gemm=True)
+    rng = synth.rng_for(7304, N, K)
+    for T in (65, 100, 128, 129, 173, 300, 512):
+        X = synth.bernoulli(rng, (T, K), 0.2)
+        want_acc, want_y = oracle.project(Qc, s, N, K, X, "u8", ldq=Qc.shape[1])
+        rows = to_dev(X)
+        acc, y = run_batched(plan, rows, "u8", T, K, N, "gemm")
+        assert_parity(acc, y, want_acc, want_y, f"T={T}")
+    assert plan.status() == sp.SP_OK
