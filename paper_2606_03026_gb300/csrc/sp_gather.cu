@@ -497,27 +497,11 @@ gather_cluster_kernel(const __grid_constant__ GatherParamsT<NP> p) {
   }
 }
 
-// Asks for the largest shared-memory carveout once per device and kernel, so
-// that every resident CTA's shared memory fits beside L1.
-template <typename Kern>
-cudaError_t set_carveout(Kern kernel, std::atomic<uint64_t>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
-  if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           (int)cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_relaxed);
-  return e;
-}
-
 // Clusters of the cluster form that can be resident at once (per device).
 template <int NP, bool kLif, int CL, int S>
-int cluster_capacity() {
+int cluster_capacity(int dev) {
   static std::atomic<int> cap[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
+  if (dev >= 64) return 0;
   int n = cap[dev].load(std::memory_order_relaxed);
   if (n != 0) return n;
   cudaLaunchConfig_t cfg = {};
@@ -542,15 +526,15 @@ int cluster_capacity() {
 
 // Resident-cluster count of the kernel the launch will use (0 on failure).
 template <int NP>
-int capacity_for(bool lif, int CL, int S) {
-  if (lif) return cluster_capacity<NP, true, 6, 8>();
+int capacity_for(int dev, bool lif, int CL, int S) {
+  if (lif) return cluster_capacity<NP, true, 6, 8>(dev);
   switch (CL) {
-    case 16: return cluster_capacity<NP, false, 16, 16>();
-    case 12: return cluster_capacity<NP, false, 12, 16>();
+    case 16: return cluster_capacity<NP, false, 16, 16>(dev);
+    case 12: return cluster_capacity<NP, false, 12, 16>(dev);
     default:
       if constexpr (NP > 1)
-        if (S == 16) return cluster_capacity<NP, false, 6, 16>();
-      return cluster_capacity<NP, false, 6, 8>();
+        if (S == 16) return cluster_capacity<NP, false, 6, 16>(dev);
+      return cluster_capacity<NP, false, 6, 8>(dev);
   }
 }
 
@@ -571,7 +555,7 @@ constexpr int kRowsMaxCtas = 228;
 // Sets the chunking of a batch's rows for clusters of 12; false when they take
 // clusters of 6.
 template <int NP>
-bool rows_spread(GatherParamsT<NP>& q) {
+bool rows_spread(GatherParamsT<NP>& q, int dev) {
   const GatherProblem& P = q.prob[0];        // the rows are alike
   int kch = 12;
   while (kch > 1 && (12 % kch != 0 || ceil_div(ceil_div(P.K, kch), 32) * 32 < 384)) --kch;
@@ -579,7 +563,7 @@ bool rows_spread(GatherParamsT<NP>& q) {
   const int tpc = 12 / kch, ntiles = gather_ntiles(P.N);
   const int ncl = ceil_div(ntiles, tpc);
   if (4 * (ncl * tpc - ntiles) > ncl * tpc) return false;   // more than a quarter idle
-  if (q.nprob * ncl * 12 > kSpreadMaxCtas || q.nprob * ncl > capacity_for<NP>(false, 12, 16)) return false;
+  if (q.nprob * ncl * 12 > kSpreadMaxCtas || q.nprob * ncl > capacity_for<NP>(dev, false, 12, 16)) return false;
   for (int j = 0; j < q.nprob; ++j) {
     q.prob[j].kch = kch;
     q.prob[j].tpc = tpc;
@@ -601,7 +585,7 @@ bool rows_spread(GatherParamsT<NP>& q) {
 // work, all resident together); more take a (clusters x CL, problems) grid
 // in which the problems with fewer clusters leave idle CTAs.
 template <int NP>
-bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out, int* s_out) {
+bool cluster_form(GatherParamsT<NP>& q, int dev, int* grid_x, int* grid_y, int* cl_out, int* s_out) {
   if (q.B != 1) return false;
   int CL = 6;
   // the rows of a batch: problems that are alike and share one weight matrix
@@ -635,7 +619,7 @@ bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out, i
     P.tpc = CL / P.kch;
     P.ncl = ceil_div(ntiles, P.tpc);
   } else {
-    if (rows && rows_spread(q)) {
+    if (rows && rows_spread(q, dev)) {
       CL = 12;
     } else {
       for (int j = 0; j < q.nprob; ++j) {
@@ -661,10 +645,10 @@ bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out, i
     if (q.prob[j].ncl > widest) widest = q.prob[j].ncl;
   }
   int S = CL > 8 ? 16 : 8;
-  if (rows && CL == 6 && total * CL <= kRowsMaxCtas && total <= capacity_for<NP>(false, 6, 16)) S = 16;
-  if (total > capacity_for<NP>(q.lif_I != nullptr, CL, S)) return false;
+  if (rows && CL == 6 && total * CL <= kRowsMaxCtas && total <= capacity_for<NP>(dev, false, 6, 16)) S = 16;
+  if (total > capacity_for<NP>(dev, q.lif_I != nullptr, CL, S)) return false;
   q.ncl_list = 0;
-  if (total <= kGatherMaxClusterList && widest <= 0xff) {
+  if (NP > 1 && total <= kGatherMaxClusterList && widest <= 0xff) {
     int c = 0;
     for (int j = 0; j < q.nprob; ++j)
       for (int cl = 0; cl < q.prob[j].ncl; ++cl) q.cl_list[c++] = (uint16_t)((j << 8) | cl);
@@ -680,20 +664,17 @@ bool cluster_form(GatherParamsT<NP>& q, int* grid_x, int* grid_y, int* cl_out, i
   return true;
 }
 
-// Sets the one-time attributes of a cluster-form kernel, once per device: the
+// Sets the one-time attributes of a gather kernel, once per device: the
 // largest shared-memory carveout (the resident-cluster count depends on it),
 // for clusters above 8 CTAs the non-portable cluster size, and the dynamic
 // shared memory above 48 KB.  (Each is a driver call of about a microsecond:
 // set on every launch they made a single decode's host time the bound.)
 template <typename Kern>
-cudaError_t cluster_attrs(Kern kernel, int CL, size_t smem, std::atomic<uint64_t>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
+cudaError_t cluster_attrs(Kern kernel, int dev, int CL, size_t smem, std::atomic<uint64_t>& done) {
   const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
   if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           (int)cudaSharedmemCarveoutMaxShared);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                       (int)cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess && CL > 8)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && smem > 48 * 1024)
@@ -706,22 +687,24 @@ template <int NP>
 cudaError_t launch_gather_t(const GatherParamsT<NP>& p, cudaStream_t s) {
   static std::atomic<uint64_t> carve_t{0}, carve_c{0}, carve_l{0}, carve_6{0}, carve_12{0}, carve_16{0};
   if (p.units_total <= 0 || p.B <= 0 || p.max_units <= 0) return cudaSuccess;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   // the attributes first: the resident-cluster counts depend on the carveout
-  cudaError_t e =
-      p.lif_I ? cluster_attrs(gather_cluster_kernel<NP, true, 6, 8>, 6, sizeof(ClusterSmem<8>), carve_l)
-              : cluster_attrs(gather_cluster_kernel<NP, false, 6, 8>, 6, sizeof(ClusterSmem<8>), carve_c);
+  e = p.lif_I ? cluster_attrs(gather_cluster_kernel<NP, true, 6, 8>, dev, 6, sizeof(ClusterSmem<8>), carve_l)
+              : cluster_attrs(gather_cluster_kernel<NP, false, 6, 8>, dev, 6, sizeof(ClusterSmem<8>), carve_c);
   if (e == cudaSuccess && !p.lif_I) {
-    e = cluster_attrs(gather_cluster_kernel<NP, false, 12, 16>, 12, sizeof(ClusterSmem<16>), carve_12);
+    e = cluster_attrs(gather_cluster_kernel<NP, false, 12, 16>, dev, 12, sizeof(ClusterSmem<16>), carve_12);
     if (e == cudaSuccess && p.nprob == 1)
-      e = cluster_attrs(gather_cluster_kernel<NP, false, 16, 16>, 16, sizeof(ClusterSmem<16>), carve_16);
+      e = cluster_attrs(gather_cluster_kernel<NP, false, 16, 16>, dev, 16, sizeof(ClusterSmem<16>), carve_16);
     if constexpr (NP > 1)
       if (e == cudaSuccess)
-        e = cluster_attrs(gather_cluster_kernel<NP, false, 6, 16>, 6, sizeof(ClusterSmem<16>), carve_6);
+        e = cluster_attrs(gather_cluster_kernel<NP, false, 6, 16>, dev, 6, sizeof(ClusterSmem<16>), carve_6);
   }
   if (e != cudaSuccess) return e;
   GatherParamsT<NP> q = p;
   int gx = 0, gy = 0, CL = 6, S = 8;
-  const bool cluster = cluster_form(q, &gx, &gy, &CL, &S);
+  const bool cluster = cluster_form(q, dev, &gx, &gy, &CL, &S);
   if (p.lif_I && !cluster) return cudaErrorNotSupported;   // the fused producer needs the cluster form
   if (cluster) {
     cudaLaunchConfig_t cfg = {};
@@ -748,7 +731,7 @@ cudaError_t launch_gather_t(const GatherParamsT<NP>& p, cudaStream_t s) {
         return cudaLaunchKernelEx(&cfg, gather_cluster_kernel<NP, false, 6, 8>, q);
     }
   }
-  e = set_carveout(gather_kernel<NP>, carve_t);
+  e = cluster_attrs(gather_kernel<NP>, dev, 1, 0, carve_t);
   if (e != cudaSuccess) return e;
   if ((int64_t)p.max_units * p.B > 0x7fffffffll) return cudaErrorInvalidConfiguration;
   // one CTA per unit; the hardware keeps every unit of a decode step resident

@@ -89,9 +89,11 @@ struct GatherParamsT {
   uint32_t* tickets;      // problem j token t tile n: ticket_begin_j*B + t*ntile_j + n
   int* err;
   // cluster form: cluster c of a 1-D grid is cluster (cl_list[c] & 0xff) of
-  // problem (cl_list[c] >> 8); ncl_list == 0: grid (clusters x 6, problems)
+  // problem (cl_list[c] >> 8); ncl_list == 0: grid (clusters x CL, problems),
+  // the only form of a single problem (whose parameters stay small: the launch
+  // copies them)
   int32_t ncl_list;
-  uint16_t cl_list[kGatherMaxClusterList];
+  uint16_t cl_list[NP > 1 ? kGatherMaxClusterList : 1];
   // fused spike producer (cluster form only): when lif_I is set, problem j's
   // spike row is made inside the kernel by one LIF step of row j of
   // (lif_vin, lif_I); the new state goes to lif_vout (and the spike words to
