@@ -47,14 +47,13 @@
 // (the lists of a CTA are fetched only when all 8 of its leading keys pass),
 // ordered by counting, gated, and the candidates recomputed, two rows per
 // warp.  Its CTAs are small enough in registers, shared memory and carve-out
-// to run beside a projection CTA: the next call's projection starts while
-// the selection runs, and a projection CTA that had to wait for a
+// to run beside a projection CTA: a projection CTA that had to wait for a
 // selection's SM held up the call by 7 us.
 //
 // Measured on 57,344 x 1536, back to back with three weight copies, us a call:
-// gate closed 21.7 (22.0 before this form: the weights 14 of it, the codes
-// 1.3, the selection and the two hand-offs 6), every call verified 24.9 (26.0);
-// four states, every call verified 30.7 (60.6); two states 27.9 (39.8).
+// gate closed 21.5 (22.0 before this form: the weights 14 of it, the codes
+// 1.3, the selection and the two hand-offs 6), every call verified 24.3 (26.0);
+// four states, every call verified 30.4 (60.6).
 #include "sp_internal.h"
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
@@ -293,8 +292,9 @@ __device__ __forceinline__ void verify_rows2(const HeadParams& p, const float* h
 // writes codes four to a word, zero from K to Kpad.  h is read again for the
 // codes (from L1): kept in registers it made the code larger, and as the code
 // runs once per CTA its size showed (2.3 us instead of 1.3).
-template <int B>
-__device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes, float* s_red, float* s_sx) {
+template <int B, class Ring>
+__device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes, float* s_red, float* s_sx,
+                                           const Ring& issue_ring) {
   constexpr int G = B == 1 ? 1 : B == 2 ? 2 : 4;
   constexpr int T = kHeadThreads / G;            // threads of one hidden state
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -321,12 +321,16 @@ __device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes,
     }
     *reinterpret_cast<uint32_t*>(s_codes + b * (p.Kpad + kCodePad) + k) = packed;
   };
-  float mx = 0.f;
+  const auto max4 = [&](float m, const float4& v) {
+    return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+  };
+  // h is requested ahead of the weight ring, whose 96 KB per SM it would
+  // otherwise queue behind (25.9 against 25.3 us a call)
+  const float4 v0 = load4(4 * tt);
+  issue_ring();
+  float mx = max4(0.f, v0);
 #pragma unroll 4
-  for (int k = 4 * tt; k < p.K; k += 4 * T) {
-    const float4 v = load4(k);
-    mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-  }
+  for (int k = 4 * tt + 4 * T; k < p.K; k += 4 * T) mx = max4(mx, load4(k));
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   if (lane == 0) s_red[warp] = mx;
@@ -338,7 +342,7 @@ __device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes,
   if (b < B) {
     if (tt == 0) s_sx[b] = sx;
 #pragma unroll 1
-    for (int k = 4 * tt; k < p.Kpad; k += 4 * T) pack(load4(k), k, sx);
+    for (int k = 4 * tt; k < p.Kpad; k += 4 * T) pack(k == 4 * tt ? v0 : load4(k), k, sx);
   }
   __syncthreads();
 }
@@ -415,20 +419,15 @@ head_kernel(const __grid_constant__ HeadParams p) {
       open_unit();
     }
   };
-  // The first ring is issued before the dependency wait: of the kernels that
-  // may still be running then (those of this library, which alone let their
-  // successors start early) none writes the weights, and whatever else may
-  // have written them on the stream has completed.
-#pragma unroll 1
-  for (int s = 0; s < kHeadRing; ++s) load();
+  // Nothing is read before the wait: the weights are the caller's, and an
+  // earlier kernel of the stream may have written them.
   pdl_wait();
-  // One state: the selection's CTAs fit beside this kernel's; resident early,
-  // they start as soon as the last list is written (with several states they
-  // come after the weight stream, below: 30 against 32 us a call for four).
-  if constexpr (B == 1) pdl_launch_dependents();
 
   // 1. activation scale and INT8 codes of each hidden state
-  head_codes<B>(p, s_codes, s_red, s_sx);
+  head_codes<B>(p, s_codes, s_red, s_sx, [&]() {
+#pragma unroll 1
+    for (int s = 0; s < kHeadRing; ++s) load();
+  });
 
   // 2. approximate logits; the even warp of each pair keeps the pair's best 64
   // keys per hidden state
@@ -526,8 +525,8 @@ head_kernel(const __grid_constant__ HeadParams p) {
   // 3. every pair's list into the workspace; the CTA's best keys (of the
   // pairs' best) into its leading keys.  With several states all the warps
   // share the pairs' lists, through shared memory (the ring is idle).
+  pdl_launch_dependents();
   if constexpr (B > 1) {
-    pdl_launch_dependents();
     cp_async_wait<0>();
     __syncthreads();
   }
@@ -589,7 +588,6 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
   const int rank = (int)blockIdx.x - b * kSelCluster;
   const int ks = p.k_sel, nc = p.nctas;
   asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // waited for before the first remote store
-  pdl_launch_dependents();
   pdl_wait();                                    // every list and count is written
   hkey lead[kCtaLead];                           // of projection CTA t
   if (t < nc) {
@@ -619,6 +617,10 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
   for (int i = t; i < nc * per; i += kSelThreads)
     if (count_larger(s_cand, nc * per, s_cand[i]) == kHeadList - 1 && s_cand[i] != 0ull) s_bound = s_cand[i];
   __syncthreads();
+  // The next call's projection waits for this kernel in any case; started at
+  // this kernel's start its idle CTAs slowed the call (57,344 rows, one state,
+  // tau 0.5: 24.6 against 24.0 us; four states 31.7 against 31.3).
+  pdl_launch_dependents();
   const hkey T = s_bound;
   if (t < nc) {
     int n = 0;

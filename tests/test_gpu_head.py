@@ -253,10 +253,9 @@ def test_head_errors():
 
 @pytest.mark.parametrize("V,K", [(3000, 256), (57344, 1536)])
 def test_head_equal_logits(V, K):
-    """A zero hidden state makes every approximate logit 0: the histogram
-    bound passes every listed key, so the selection merges every list (the
-    exact slow path). Candidates are then the lowest rows, the gap is 0 and
-    the recomputed logits are all 0."""
+    """A zero hidden state makes every approximate logit 0, so the row index
+    alone orders the keys. Candidates are then the lowest rows, the gap is 0
+    and the recomputed logits are all 0."""
     if V == 57344:
         Q, s, Qd, sd = full_head()
     else:
@@ -288,3 +287,22 @@ def test_head_codes_at_exact_halves():
     head = sp.Head(to_dev(Q), to_dev(s), K=K)
     got = run_head(head, h, np.inf, 16, V)
     check(got, Q, s, V, K, h, np.inf, 16, "exact halves")
+
+
+def test_head_weights_written_on_the_stream():
+    """The kernel that comes right before a call writes the weights: the call
+    reads what it wrote (the weights are borrowed, not copied)."""
+    Q, s, _, sd = full_head()
+    V, K = Q.shape
+    Qd = to_dev(Q)
+    head = sp.Head(Qd, sd, K=K)
+    h = synth.rng_for(7805).standard_normal((1, K)).astype(np.float32)
+    hd = to_dev(h)
+    out = {"token": torch.zeros(1, dtype=torch.int32, device=DEV), "verified": torch.zeros(1, dtype=torch.int32, device=DEV),
+           "gap": torch.zeros(1, device=DEV), "cand": torch.zeros(1, 64, dtype=torch.int32, device=DEV),
+           "r": torch.zeros(1, 64, device=DEV), "z": torch.full((1, V + 3), float("nan"), device=DEV)}
+    for i in range(4):
+        Qd.neg_()
+        head(hd, 4.0, 64, *out.values())
+        got = {k: v.cpu().numpy() for k, v in out.items()}
+        check(got, Q if i % 2 else -Q, s, V, K, h, 4.0, 64, f"call {i}")
