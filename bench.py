@@ -1146,12 +1146,12 @@ def bench_dense(torch, sp, synth, dev, stream, peaks, peak_kind, world, blocks=2
            "B": 1, "problems_per_launch": len(probs[1]), "bytes_per_step": nbytes,
            "ms_per_step": ms, "projected_tokens_per_s": 1e3 / ms,
            "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
-                        "frac": gbs / hbm, "traffic": measured_traffic("dense_kernel", "sp_dense.cu"),
-                        "kernel": "dense_kernel<1> (66 projections, one launch)",
+                        "frac": gbs / hbm, "traffic": measured_traffic("dense_mma_kernel", "sp_dense.cu"),
+                        "kernel": "dense_mma_kernel<1> (66 projections, one launch)",
                         "peak_kind": peak_kind},
            "B_sweep": sweep,
-           "note": "B = 2-4 reuse each converted weight for B FMAs at 2 CTAs per SM; they run "
-                   "below both the HBM rate and the FP32 issue rate (latency-bound)"}
+           "note": "tensor-core form: the rows of B are columns of the same MMA, so B = 2-4 read "
+                   "and convert the weights once and stay HBM-bound"}
     if with_oracle:
         W, s = srcs["up"]
         N, K = W.shape

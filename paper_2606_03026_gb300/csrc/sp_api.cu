@@ -358,16 +358,15 @@ sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld,
 //   GEMM, T <= 64 ~ 3.4 us + 0.33 us per K block of a CTA's K range
 //                   (ceil(Kp / 64 / S), S = the cluster size) + 0.045 us per row
 //   GEMM, T > 64  ~ max(11.3 us + 2 B N K ops / 1.4 PFLOP/s, 8.5 us + 0.55 us per 1024 of K)
-// (the GEMM only for SP_PLAN_GEMM plans).  Measured at 1536 x 6144: gather
-// 4.2 / 6.7 / 9.0 / 11.6 / 16.5 us at B = 1 / 8 / 16 / 32 / 64 in the ticket
-// form, and 6.0 / 7.6 / 9.3 us at B = 8 / 16 / 32 with the rows run as a
-// group (the fixed term fitted to the latter: 4.2 us before), small-T GEMM
-// 7.2 / 7.2 / 7.3 / 8.0 / 9.2 us, the 128-row GEMM 12.1 us at B = 65 .. 128
-// (17.5 us at K = 16384); at 1536 x 1536 the gather (rows as a group) wins
-// up to B = 6 (3.6 against 4.5 us at B = 4) and the small-T GEMM from B = 8.  The union fetch is never chosen automatically: it
-// was slower than the per-token gather at every batch size measured (its
-// adds are ALU-bound, and the 126 MB L2 serves the per-token re-reads of a
-// 9.4 MB weight matrix).
+// (the GEMM only for SP_PLAN_GEMM plans).  The constants were fitted before
+// the kernels' latest speed-ups (both sides 0.2 to 1.3 us faster); measured
+// since, 1536 x 6144: gather (rows as a group) 3.6 / 4.6
+// / 5.6 / 6.4 us at B = 2 / 4 / 8 / 12, small-T GEMM 7.05 us at B = 16 and 8.5
+// at 64 (gather 16.2), the 128-row GEMM 10.9 us at B = 100; 1536 x 1536: the
+// gather up to B = 6, the small-T GEMM from B = 8 (5.7 us at 64).  The union
+// fetch is never chosen automatically: it was slower than the per-token
+// gather at every batch size measured (its adds are ALU-bound, and the 126 MB
+// L2 serves the per-token re-reads of a 9.4 MB weight matrix).
 sp_kernel choose(const sp_plan_s* p, int B, int32_t total) {
   if (!(p->flags & SP_PLAN_GEMM)) return SP_GATHER;
   const double gather_us = 3.9 + 0.08 * (B - 1) + (double)total * p->N / 6.7e6;

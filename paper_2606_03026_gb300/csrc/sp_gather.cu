@@ -18,8 +18,9 @@
 //      shared memory with cp.async) and adds them into biased 16-bit lanes
 //      (at most 256 columns per warp, so the lanes cannot overflow),
 //   3. the warps' partials meet in shared memory.
-// Cluster form (one token per problem, K <= 6 x 1024: batch-1 decode and
-// grouped decode steps): 256-thread CTAs, chunks of up to 1024 columns, and
+// Cluster form (one token per problem: batch-1 decode up to K = 16 x 1024,
+// grouped decode steps up to 6 x 1024, and the rows of a batch as a group of
+// problems that share W): 256-thread CTAs, chunks of up to 1024 columns, and
 // the chunk CTAs of a tile in one thread-block cluster that reduces its
 // partials through distributed shared memory (no workspace, no atomics).
 // Ticket form (any batch and K): 128-thread CTAs, 512-column chunks; acc / y
@@ -573,10 +574,9 @@ bool rows_spread(GatherParamsT<NP>& q, int dev) {
 }
 
 // Fills the cluster-form fields of q, the cluster size *cl_out and the
-// shared-memory slots *s_out; false
-// when the launch does not fit the cluster form (several tokens, a chunk
-// count above the cluster size, or more clusters than can be resident at
-// once).  A group of projections takes clusters of 6 and the fewest chunks
+// shared-memory slots *s_out; false when the launch does not fit the cluster
+// form (several tokens, a chunk count above the cluster size, or more clusters
+// than can be resident at once).  A group of projections takes clusters of 6 and the fewest chunks
 // of at most 1024 columns.  A single projection (which alone would leave
 // most SMs idle) takes the cluster size and chunking with the most working
 // CTAs among clusters of 16, 12 and 6, chunks of 256 to 1024 columns and at
