@@ -36,9 +36,9 @@ struct sp_plan_s {
   size_t n_tickets = 0;
   int* err = nullptr;             // device error word
   int32_t* d_counts = nullptr;    // spike count in progress and its tickets (SpikeCount)
-  int32_t* h_counts = nullptr;    // page-locked: the last count, the sequence number it is of
-  int32_t count_seq = 0;          // counts asked for
-  bool count_pending = false;     // last_active is still to be read from h_counts
+  uint64_t* h_count = nullptr;    // page-locked: the last count and the sequence number it is of (SpikeCount)
+  uint32_t count_seq = 0;         // counts asked for
+  bool count_pending = false;     // last_active is still to be read from h_count
   // tensor-core path
   uint8_t* Wq = nullptr;          // [N][2 Kp] e4m3 weight planes (16 h, l)
   uint8_t* Xs = nullptr;          // [xs_rows][Kp] 0/1 spike staging
@@ -143,7 +143,7 @@ void plan_free(sp_plan_s* p) {
   cudaFree(p->tickets);
   cudaFree(p->err);
   cudaFree(p->d_counts);
-  if (p->h_counts) cudaFreeHost(p->h_counts);
+  if (p->h_count) cudaFreeHost(p->h_count);
   cudaFree(p->Wq);
   cudaFree(p->Xs);
   cudaFree(p->part);
@@ -379,12 +379,18 @@ sp_kernel choose(const sp_plan_s* p, int B, int32_t total) {
   return gemm_us < gather_us ? SP_GEMM : SP_GATHER;
 }
 
+// The count of the plan's last SP_AUTO call, -1 while it is not published.
+int32_t published_count(const sp_plan_s* p) {
+  const uint64_t word = __atomic_load_n(p->h_count, __ATOMIC_ACQUIRE);
+  return (uint32_t)(word >> 32) == p->count_seq ? (int32_t)(uint32_t)word : -1;
+}
+
 sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld, int32_t* acc,
                     float* y, sp_kernel strategy, cudaStream_t s) {
   SpikeCount count = {};
   if (strategy == SP_AUTO) {
     count.dev = p->d_counts;
-    count.host = p->h_counts;
+    count.host = p->h_count;
     count.seq = ++p->count_seq;
     // Where the GEMM is modelled faster than a gather of no column at all,
     // the count cannot change the choice: the GEMM is enqueued at once, the
@@ -405,9 +411,9 @@ sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
     }
     SP_CUDA(launch_density(spikes, fmt, ld, B, p->K, count, s));
     SP_CUDA(cudaStreamSynchronize(s));
-    strategy = choose(p, B, p->h_counts[0]);
+    p->last_active = published_count(p);
+    strategy = choose(p, B, p->last_active);
     p->last_kernel = strategy;
-    p->last_active = p->h_counts[0];
     p->count_pending = false;
     count = SpikeCount{};
   }
@@ -494,12 +500,12 @@ sp_status spike_proj_plan(sp_plan_t* plan, const int8_t* W, int64_t ldw, const f
     plan_free(p);
     return st;
   }
-  cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&p->h_counts), 2 * sizeof(int32_t));
+  cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&p->h_count), sizeof(uint64_t));
   if (e != cudaSuccess) {
     plan_free(p);
     return cuda_fail(e);
   }
-  p->h_counts[0] = p->h_counts[1] = 0;
+  *p->h_count = 0;
   if (flags & SP_PLAN_GEMM) {
     p->Kp = gemm_k_pad(K);
     p->xs_rows = ceil_div(max_batch, 128) * 128;
@@ -571,9 +577,12 @@ sp_status spike_proj_last_dispatch(sp_plan_t plan, sp_kernel* chosen, int32_t* a
   if (!plan) return SP_EINVAL;
   if (plan->count_pending) {
     // the counting kernel of the last SP_AUTO call may still be running
-    const volatile int32_t* host = plan->h_counts;
-    if (host[1] != plan->count_seq) SP_CUDA(cudaDeviceSynchronize());
-    plan->last_active = host[0];
+    int32_t count = published_count(plan);
+    if (count < 0) {
+      SP_CUDA(cudaDeviceSynchronize());
+      count = published_count(plan);
+    }
+    plan->last_active = count;
     plan->count_pending = false;
   }
   if (chosen) *chosen = plan->last_kernel;

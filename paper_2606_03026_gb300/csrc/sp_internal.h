@@ -135,13 +135,14 @@ constexpr int kUnionMaxRows = 256;      // rows per union launch
 
 // Where a count of active spikes (sum over the rows of |A_t|) goes.  The
 // counting kernel's blocks add into dev[0]; then either the last of them (by
-// tickets in dev[1]) or the GEMM that follows on the stream publishes it:
-// host[0] = count, then host[1] = seq (page-locked memory, visible without a
-// copy), dev left zero for the next call.
+// tickets in dev[1]) or the GEMM that follows on the stream publishes it in
+// *host (page-locked memory, visible without a copy), dev left zero for the
+// next call.  Count and sequence number travel in one 64-bit word: as two words
+// an Arm host may read the new number and the old count.
 struct SpikeCount {
   int32_t* dev;           // two words, zero between calls; null: no count
-  int32_t* host;
-  int32_t seq;
+  uint64_t* host;         // seq << 32 | count
+  uint32_t seq;
 };
 
 // Tensor-core (tcgen05) prefill GEMM operands.

@@ -58,11 +58,9 @@ __device__ __forceinline__ const void* spike_row(const void* base, int fmt, int6
 // Publishes the count in c.dev[0] and clears it (one thread, after every
 // block's addition).
 __device__ __forceinline__ void publish_count(const SpikeCount& c) {
-  volatile int32_t* host = c.host;
-  host[0] = atomicExch(c.dev, 0);
+  const uint32_t count = (uint32_t)atomicExch(c.dev, 0);
   c.dev[1] = 0;
-  __threadfence_system();
-  host[1] = c.seq;
+  *static_cast<volatile uint64_t*>(c.host) = (uint64_t)c.seq << 32 | count;
 }
 
 // Adds the calling thread's share to the count; `publish`: the last block to

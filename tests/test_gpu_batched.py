@@ -333,3 +333,23 @@ def test_gemm_split_shapes(N, K):
         acc, y = run_batched(plan, rows, "u8", T, K, N, "gemm")
         assert_parity(acc, y, want_acc, want_y, f"T={T}")
     assert plan.status() == sp.SP_OK
+
+
+def test_auto_count_is_of_the_call_before():
+    """The count read right after an SP_AUTO call that did not wait for it is
+    that call's, never the one before (the host may find the sequence number
+    of a call in place while it still holds an earlier count, if the two are
+    read apart)."""
+    N, K, T = 512, 512, 128
+    Qc, s, _ = synth.random_case(94, N, K)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=T, gemm=True)
+    rng = synth.rng_for(7305)
+    X = [synth.bernoulli(rng, (T, K), p) for p in (0.05, 0.6, 0.0, 0.3)]
+    want = [("gemm", int(x.astype(np.int64).sum())) for x in X]
+    rows = [to_dev(x) for x in X]
+    y = torch.empty(T, N, dtype=torch.float32, device=DEV)
+    for i in range(4000):
+        plan.batched(rows[i % 4], "u8", T, K, None, y, "auto")
+        if i % 3:                                # several calls in flight before the question, or none
+            assert plan.last_dispatch() == want[i % 4], f"call {i}"
+    plan.close()
