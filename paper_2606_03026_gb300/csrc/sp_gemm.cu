@@ -821,6 +821,9 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
           }
         }
         ok = __all_sync(0xffffffffu, ok);
+        // each lane has acquired one range's flag and all lanes read every
+        // range's partials: a vote orders no memory, this barrier does
+        __syncwarp();
       }
       if (!ok) {
         *s_abort = 1;

@@ -188,6 +188,50 @@ def test_tail_split_shapes(T, shapes):
     group.close()
 
 
+@pytest.mark.parametrize("T,units,K", [
+    (256, 30, 640), (256, 24, 1000), (256, 18, 1100), (256, 15, 1280), (256, 5, 1600),   # CTA pairs: 2 to 6 ranges
+    (256, 76 + 25, 1030), (250, 12, 520),             # a whole round first; ranges of few K blocks
+    (128, 60, 512), (70, 40, 777), (128, 7, 1536),    # single CTAs: 2, 3 and 6 ranges
+])
+def test_tail_split_ranges(T, units, K):
+    """The tail of a grouped launch cut into 2 to 6 K ranges (by the number of
+    units of its last round on a 152-SM device), for CTA pairs and single
+    CTAs: launches that follow one another without a wait, on alternating
+    inputs, all equal to the oracle's rows."""
+    shapes, left = [], units
+    while left:
+        tn = min(left, 11 if left > 22 else 4)
+        shapes.append((256 * tn - (16 if left > tn else 112), K, 256 * tn))
+        left -= tn
+    members = make_members(shapes, T, seed=units)
+    group = sp.Group([m[-1] for m in members])
+    ldx = (K + 15) // 16 * 16
+    inputs = []
+    for i in range(2):
+        X = [synth.bernoulli(synth.rng_for(7400 + i, units, j), (T, K), 0.2) for j in range(len(members))]
+        xs = [torch.zeros(T, ldx, dtype=torch.bool, device=DEV) for _ in members]
+        for x, r in zip(X, xs):
+            r[:, :K] = to_dev(x).bool()
+        rows = np.unique([0, 31, 63, T // 2, T - 1])
+        wants = [oracle.project(m[0], m[1], m[3], K, x[rows], "u8", ldq=m[5]) for m, x in zip(members, X)]
+        inputs.append((xs, rows, wants))
+    outs = []
+    for i in range(8):
+        accs = [torch.full((T, m[3]), -7, dtype=torch.int32, device=DEV) for m in members]
+        ys = [torch.full((T, m[3]), -7.0, dtype=torch.float32, device=DEV) for m in members]
+        group.prefill(inputs[i % 2][0], "bool8", T, ldx, accs, ys)
+        outs.append((accs, ys))
+    torch.cuda.synchronize()
+    for i, (accs, ys) in enumerate(outs):
+        _, rows, wants = inputs[i % 2]
+        for j, (wa, wy) in enumerate(wants):
+            assert_parity(accs[j][rows], ys[j][rows], wa, wy, f"launch {i} member {j}")
+            if i >= 2:
+                assert torch.equal(accs[j], outs[i - 2][0][j]), f"launch {i} member {j} differs from {i - 2}"
+    assert group.status() == sp.SP_OK
+    group.close()
+
+
 def test_group_prefill_errors():
     members = make_members(RAGGED[:2], 8, seed=9)
     plain = sp.Plan(to_dev(members[0][0]), to_dev(members[0][1]), members[0][3], members[0][4],
