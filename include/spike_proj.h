@@ -510,8 +510,13 @@ sp_status spike_proj_head(sp_head_t head, const float *h, int64_t ldh, int32_t B
  *                   CTA never stores its partial sums into the owners'
  *                   shared memory, and the owners' waits (bounded by about
  *                   2 ms) run out: the kernel raises the error word and those
- *                   owners leave their outputs unwritten.  Other kernels
- *                   ignore it (it is still disarmed by their launch).
+ *                   owners leave their outputs unwritten.  A grouped
+ *                   prefill runs on a single thread-block cluster, so that no
+ *                   K range of its split tail finds another one's partial sums
+ *                   in time: the ranges hand their output over to the one that
+ *                   comes last, and the results are exact, with no error.
+ *                   Other kernels ignore it (it is still disarmed by their
+ *                   launch).
  * No fault traps, faults the GPU or spins without bound.  spike_proj_plan_status
  * / spike_proj_group_status then return SP_EKERNEL, clear the error word and
  * re-zero the workspace, and the next call is exact again.

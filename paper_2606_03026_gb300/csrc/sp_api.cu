@@ -81,7 +81,7 @@ struct sp_group_s {
   sp_plan_s* plans[kMaxProblems] = {};
   GemmGroupArgs* gemm = nullptr;
   float* gpart = nullptr;         // tail-split partials (groups of SP_PLAN_GEMM plans)
-  uint32_t* gflags = nullptr;     // their flags, zero between launches
+  uint32_t* garrivals = nullptr;  // their arrival counters, zero between launches
   int32_t fault = 0;              // test fault armed for the next launch (sp_fault)
   const void* rows_ptr[kMaxProblems] = {};
   int64_t rows_ld[kMaxProblems] = {};
@@ -154,7 +154,7 @@ void group_free(sp_group_s* g) {
   if (!g) return;
   delete g->gemm;
   cudaFree(g->gpart);
-  cudaFree(g->gflags);
+  cudaFree(g->garrivals);
   cudaFree(g->ws);
   cudaFree(g->tickets);
   cudaFree(g->err);
@@ -663,7 +663,7 @@ sp_status spike_proj_group_create(sp_group_t* group, const sp_plan_t* plans, int
   for (int j = 0; j < count; ++j) all_gemm = all_gemm && (plans[j]->flags & SP_PLAN_GEMM);
   if (all_gemm &&
       ((st = dev_alloc_zero(&g->gpart, (size_t)kGemmGroupSlots * kGemmPartialElems, s)) != SP_OK ||
-       (st = dev_alloc_zero(&g->gflags, (size_t)kGemmGroupFlags, s)) != SP_OK)) {
+       (st = dev_alloc_zero(&g->garrivals, (size_t)kGemmGroupArrivals, s)) != SP_OK)) {
     group_free(g);
     return st;
   }
@@ -729,7 +729,7 @@ sp_status spike_proj_group_prefill(sp_group_t g, const void* const* X, sp_fmt fm
   a.count = g->count;
   a.err = g->err;
   a.part = g->gpart;
-  a.flags = g->gflags;
+  a.arrivals = g->garrivals;
   int64_t units = 0;
   // CTA pairs (2-SM MMA over 256 rows) when the members' row tiles pair up
   // with little padding
@@ -912,8 +912,8 @@ sp_status spike_proj_group_status(sp_group_t g, sp_stream_t stream) {
   SP_CUDA(cudaMemsetAsync(g->err, 0, sizeof(int), s));
   SP_CUDA(cudaMemsetAsync(g->ws, 0, g->ws_elems * sizeof(int32_t), s));
   SP_CUDA(cudaMemsetAsync(g->tickets, 0, g->n_tickets * sizeof(uint32_t), s));
-  if (g->gflags)
-    SP_CUDA(cudaMemsetAsync(g->gflags, 0, (size_t)kGemmGroupFlags * sizeof(uint32_t), s));
+  if (g->garrivals)
+    SP_CUDA(cudaMemsetAsync(g->garrivals, 0, (size_t)kGemmGroupArrivals * sizeof(uint32_t), s));
   SP_CUDA(cudaStreamSynchronize(s));
   return SP_EKERNEL;
 }

@@ -535,6 +535,7 @@ struct GroupUnit {
   int mb, nb;             // this CTA's row tile and the channel tile
   int kb0, kb1;           // K blocks [kb0, kb1)
   int S, s;               // K range s of S (S = 1: whole K)
+  int t;                  // S > 1: which of the split units
   int slot;               // S > 1: the partial slot of range 0 (range i: + i)
 };
 
@@ -544,13 +545,13 @@ __device__ __forceinline__ GroupUnit group_unit(const GemmGroupArgs& g, int v, i
   int u = v;
   r.s = 0;
   r.S = 1;
-  r.slot = 0;
+  r.t = r.slot = 0;
   if (v >= g.whole) {
     r.S = g.tail_s;
-    const int t = (v - g.whole) / r.S;
-    r.s = v - g.whole - t * r.S;
-    u = g.whole + t;
-    r.slot = t * r.S;
+    r.t = (v - g.whole) / r.S;
+    r.s = v - g.whole - r.t * r.S;
+    u = g.whole + r.t;
+    r.slot = r.t * r.S;
   }
   r.j = member_of(g, u);
   const GemmMember& M = g.m[r.j];
@@ -568,8 +569,11 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+// *p += 1; returns the count before.
+__device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t* p) {
+  uint32_t v;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
 template <int CL>
@@ -786,71 +790,68 @@ gemm_group_kernel(const __grid_constant__ GemmGroupArgs g) {
       // this warp's 32 x 16 block of chunk c inside a 128 x 256 partial tile
       const size_t pofs = (size_t)(q * 32 + lane) + (size_t)half * 16 * 128;
       const int S = U.S;
-      // this warp's flags: range i's partial is ready for range k at (i, k)
-      const auto flag = [&](int i, int k) {
-        return g.flags + ((size_t)((U.slot + i) * CL + rank) * 8 + (warp - 2)) * kGemmGroupMaxTail + k;
-      };
-      bool ok = true;
-      if (S > 1) {
-        // the chunks of the other ranges (chunk c belongs to range c mod S)
-        // to this range's slot, then their flags (every lane's stores ordered
-        // before them)
+      // this warp's arrival counters of the unit's chunks, and the chunks that
+      // it is to finish
+      uint32_t* arrivals = g.arrivals + ((size_t)(U.t * CL + rank) * 8 + (warp - 2)) * CPT;
+      uint32_t finish = live ? (1u << CPT) - 1u : 0u;
+      if (S > 1 && live) {
+        uint32_t own = 0u;                     // chunk c belongs to range c mod S
+        for (int c = U.s; c < CPT; c += S) own |= 1u << c;
         float* dst = g.part + (size_t)((U.slot + U.s) * CL + rank) * (BM * BN) + pofs;
-        if (live) {
+        // chunks into this range's slot, and the arrival at them (every lane's
+        // stores ordered before it); the chunks all others have arrived at
+        const auto hand_over = [&](uint32_t chunks) {
 #pragma unroll 1
-          for (int c = 0; c < CPT; ++c) {
-            if (c % S == U.s) continue;
+          for (uint32_t left = chunks; left; left &= left - 1u) {
+            const int c = __ffs((int)left) - 1;
             uint32_t v[16];
             tmem_ld16(trow + (uint32_t)(c * 32), v);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
               __stcg(dst + (size_t)(c * 32 + i) * 128, __uint_as_float(v[i]));
           }
-        }
-        __threadfence();
-        __syncwarp();
-        if (lane < S && lane != U.s) {
-          st_release(flag(U.s, lane), 1u);
-          // and wait (bounded) for theirs
+          __threadfence();
+          __syncwarp();
+          const bool last = lane < CPT && (chunks >> lane & 1u) &&
+                            arrive_acq_rel(arrivals + lane) == (uint32_t)(S - 1);
+          return __ballot_sync(0xffffffffu, last);
+        };
+        finish = hand_over(~own & ((1u << CPT) - 1u));
+        bool complete = false;
+        if (lane < CPT && (own >> lane & 1u)) {
           const long long t0 = clock64();
-          while (ld_acquire(flag(lane, U.s)) == 0u) {
-            if (clock64() - t0 > kWaitLimitCycles) {
-              ok = false;
-              break;
-            }
-          }
+          do {
+            complete = ld_acquire(arrivals + lane) == (uint32_t)(S - 1);
+          } while (!complete && clock64() - t0 < kGemmGroupGrace);
         }
-        ok = __all_sync(0xffffffffu, ok);
-        // each lane has acquired one range's flag and all lanes read every
-        // range's partials: a vote orders no memory, this barrier does
+        const uint32_t ready = __ballot_sync(0xffffffffu, complete);
+        finish |= ready;
+        if (own & ~ready) finish |= hand_over(own & ~ready);
+        // the acquires above are of single lanes, the partials below are read
+        // by all: a ballot orders no memory, this barrier does
         __syncwarp();
       }
-      if (!ok) {
-        *s_abort = 1;
-        if (lane == 0) atomicExch(g.err, kErrFlagTimeout);
-      } else if (live) {
 #pragma unroll 1
-        for (int c = U.s; c < CPT; c += S) {
-          const int col0 = U.nb * BN + c * 32 + half * 16;
-          uint32_t v[16];
-          tmem_ld16(trow + (uint32_t)(c * 32), v);
-          for (int h = 0; h < S; ++h) {
-            if (h == U.s) continue;
-            const float* src = g.part + (size_t)((U.slot + h) * CL + rank) * (BM * BN) + pofs +
-                               (size_t)c * 32 * 128;
+      for (uint32_t left = finish; left; left &= left - 1u) {
+        const int c = __ffs((int)left) - 1;
+        const int col0 = U.nb * BN + c * 32 + half * 16;
+        uint32_t v[16];
+        tmem_ld16(trow + (uint32_t)(c * 32), v);
+        for (int h = 0; h < S; ++h) {
+          if (h == U.s) continue;
+          const float* src = g.part + (size_t)((U.slot + h) * CL + rank) * (BM * BN) + pofs +
+                             (size_t)c * 32 * 128;
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              v[i] = __float_as_uint(__uint_as_float(v[i]) + __ldcg(src + (size_t)i * 128));
-          }
-          if (M.p.fault == kFaultAbort) {   // test fault: the output stays unwritten
-            if (lane == 0) atomicExch(g.err, kErrInjected);
-            continue;
-          }
-          store_block16(M.p, tr, v, row0, col0, column_scale(M.p, col0 + (lane & 15)));
+          for (int i = 0; i < 16; ++i)
+            v[i] = __float_as_uint(__uint_as_float(v[i]) + __ldcg(src + (size_t)i * 128));
         }
+        if (M.p.fault == kFaultAbort) {   // test fault: the output stays unwritten
+          if (lane == 0) atomicExch(g.err, kErrInjected);
+          continue;
+        }
+        store_block16(M.p, tr, v, row0, col0, column_scale(M.p, col0 + (lane & 15)));
       }
-      __syncwarp();
-      if (lane < S && lane != U.s) *flag(lane, U.s) = 0u;   // for the next launch
+      if (S > 1 && lane < CPT && (finish >> lane & 1u)) arrivals[lane] = 0u;   // for the next launch
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -1197,7 +1198,7 @@ cudaError_t launch_group_cl(const GemmGroupArgs& a, cudaStream_t s) {
   b.whole = a.units;
   b.tail_s = 1;
   const int r = a.units % clusters;
-  if (a.part && a.flags && r > 0) {
+  if (a.part && a.arrivals && r > 0) {
     int S = clusters / r;
     if (S > kGemmGroupMaxTail) S = kGemmGroupMaxTail;
     int min_nkb = 1 << 30;
@@ -1211,6 +1212,9 @@ cudaError_t launch_group_cl(const GemmGroupArgs& a, cudaStream_t s) {
   }
   b.total = b.whole + (a.units - b.whole) * b.tail_s;
   if (clusters > b.total) clusters = b.total;
+  // test stall fault: one cluster runs every unit, so that the K ranges of the
+  // tail run one after another and hand their chunks over
+  if (a.m[0].p.fault == kFaultStall) clusters = 1;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

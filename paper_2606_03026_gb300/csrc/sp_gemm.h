@@ -90,12 +90,18 @@ struct GemmMember {
 // Tail split: when the units do not fill the last round of the persistent
 // grid, each of the last r units is cut into S ranges of its K blocks (S =
 // min(clusters / r, kGemmGroupMaxTail)), so the last round runs r S sub-units
-// on as many clusters.  Range s finishes the 32-column chunks c with c mod S ==
-// s of the output: it writes its fp32 partials of the other chunks to part
-// (per CTA one 128 x 256 tile), raises a flag per warp for every other range,
-// waits (bounded) for theirs, adds, writes and clears.  (With one range
-// finishing the whole tile, its output and the partials it read were the last
-// 18 us of a 137 us launch.)  The launcher fills whole / tail_s / total.
+// on as many clusters.  Range s owns the 32-column chunks c with c mod S == s
+// of the output: each of its epilogue warps writes its fp32 partials of the
+// other chunks to part (per CTA one 128 x 256 tile), counts its arrival at each
+// of them, and finishes the own chunks that all others have arrived at (adds,
+// writes, clears the counter).  An own chunk that is still short of arrivals
+// after kGemmGroupGrace cycles is handed over: the range stores it like the
+// others and leaves, and whichever range arrives last finishes it.  So no
+// range depends on another one's running (the clusters of a launch need not
+// be resident together: a kernel of another stream may hold SMs), and the
+// ranges share the output where they run together.  (With one range finishing
+// the whole tile, its output and the partials it read were the last 18 us of a
+// 137 us launch.)  The launcher fills whole / tail_s / total.
 struct GemmGroupArgs {
   GemmMember m[kGemmMaxMembers];
   int32_t count;          // members
@@ -103,17 +109,20 @@ struct GemmGroupArgs {
   int32_t cl;             // CTAs per unit (1, or 2 for the CTA-pair MMA)
   int* err;               // device error word
   float* part;            // tail-split partials, kGemmGroupSlots x 128 x 256 fp32 (or null)
-  uint32_t* flags;        // kGemmGroupFlags words, zero between launches
+  uint32_t* arrivals;     // kGemmGroupArrivals words, zero between launches
   int32_t whole;          // units run over their whole K (the first ones)
   int32_t tail_s;         // K ranges per tail unit (1: no split)
   int32_t total;          // whole + (units - whole) * tail_s
 };
 // Partial tiles (128 x 256 fp32, one per CTA of a sub-unit) that the tail
-// split may need: at most one per SM; the most K ranges; and the flags, one per
-// slot, epilogue warp and reading range.
+// split may need: at most one per SM; the most K ranges; the arrival counters,
+// one per CTA of a split unit (at least two slots each), epilogue warp and
+// chunk; and how long a range keeps its chunks (about 50 us: ranges of one
+// round end within a few of each other).
 constexpr int kGemmGroupSlots = 160;
 constexpr int kGemmGroupMaxTail = 6;
-constexpr int kGemmGroupFlags = kGemmGroupSlots * 8 * kGemmGroupMaxTail;
+constexpr int kGemmGroupArrivals = kGemmGroupSlots / 2 * 8 * 8;
+constexpr long long kGemmGroupGrace = 100000;
 // CTAs per unit for a grouped launch whose members have these tile counts:
 // 2 unless pairing row tiles adds more than 1/8 of idle (row-padding) tiles.
 int gemm_group_cluster(const int* tiles_m, const int* tiles_n, int count);

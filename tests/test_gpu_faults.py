@@ -142,8 +142,8 @@ def test_small_gemm_stall(down):
 def test_group_abort():
     """A decode step's group (ticket-free cluster form) at 3 and 22 blocks
     (the latter with more CTAs than SMs), aborted and stalled, and the
-    grouped prefill (tail split: owners and helpers exchange partials behind
-    flags)."""
+    grouped prefill (tail split: K ranges exchange partials behind arrival
+    counters)."""
     weights = synth.decode_step_weights(0, blocks=3)
     plans = [sp.Plan(to_dev(Q), to_dev(s), N, K, max_batch=256, gemm=True)
              for (Q, s, N, K) in weights]
@@ -202,8 +202,8 @@ def test_group_abort():
         return torch.stack(accs), torch.stack(ys)
 
     check_recovery(group, prefill, wantp_acc, wantp_y, "group prefill")
-    # the grouped prefill does not wait on other CTAs' copies: it ignores a
-    # stall, which its launch still disarms
+    # no CTA of the grouped prefill depends on another one's running: under a
+    # stall its K ranges run one after another and the results stay exact
     group.inject_fault(sp.SP_FAULT_STALL)
     acc, y = prefill()
     torch.cuda.synchronize()

@@ -168,9 +168,10 @@ def test_prefill_mixed_decoder_group():
 ])
 def test_tail_split_shapes(T, shapes):
     """Groups whose tiles leave the persistent grid's last round partly idle:
-    the tail units run as K ranges on several clusters, the owner adding the
-    helpers' fp32 partials.  Every output against the oracle, twice (the
-    partials' flags are cleared for the next launch)."""
+    the tail units run as K ranges on several clusters, each range finishing
+    its share of the unit's chunks from all ranges' fp32 partials.  Every
+    output against the oracle, twice (the arrival counters are cleared for
+    the next launch)."""
     members = make_members(shapes, T, seed=len(shapes))
     group = sp.Group([m[-1] for m in members])
     ldx = max(m[4] for m in members)
@@ -229,6 +230,40 @@ def test_tail_split_ranges(T, units, K):
             if i >= 2:
                 assert torch.equal(accs[j], outs[i - 2][0][j]), f"launch {i} member {j} differs from {i - 2}"
     assert group.status() == sp.SP_OK
+    group.close()
+
+
+@pytest.mark.parametrize("T,shapes", [
+    (256, [(1536, 700, 1536)] * 5),                   # pairs, 30 units: 2 ranges
+    (256, [(1200, 1000, 1216), (1024, 1100, 1024), (1536, 1536, 1536)]),   # pairs, 15 units: 4 ranges
+    (256, [(2560, 640, 2560)] * 10),                  # a whole round, then 24 units in 3 ranges
+    (130, [(496, 1600, 512)] * 3),                    # pairs with a row tile of two rows
+    (100, [(1536, 2000, 1536), (1536, 2048, 1536)]),  # single CTAs, 12 units: 6 ranges
+])
+def test_tail_ranges_one_after_another(T, shapes):
+    """No K range of the tail waits for another one to run: with the whole
+    launch on one cluster the ranges of a unit follow each other, every one
+    but the last hands all of its chunks over, and the results are exact."""
+    members = make_members(shapes, T, seed=len(shapes) + 50)
+    group = sp.Group([m[-1] for m in members])
+    ldx = (max(m[4] for m in members) + 15) // 16 * 16
+    xs_dev = []
+    for m in members:
+        r = np.zeros((T, ldx), np.uint8)
+        r[:, : m[4]] = m[2]
+        xs_dev.append(to_dev(r).bool())
+    rows = np.unique([0, 31, T // 2, T - 2, T - 1])
+    wants = [oracle.project(Q, s, N, K, x[rows], "u8", ldq=ldq) for (Q, s, x, N, K, ldq, _) in members]
+    first = None
+    for rep in range(4):                              # serial, side by side, serial, side by side
+        if rep % 2 == 0:
+            group.inject_fault(sp.SP_FAULT_STALL)
+        accs, ys = run_group(group, members, xs_dev, "bool8", T, ldx)
+        for j, (wa, wy) in enumerate(wants):
+            assert_parity(accs[j][rows], ys[j][rows], wa, wy, f"member {j} rep {rep}")
+        first = first or accs
+        assert all(torch.equal(a, b) for a, b in zip(accs, first)), f"rep {rep}"
+        assert group.status() == sp.SP_OK
     group.close()
 
 
