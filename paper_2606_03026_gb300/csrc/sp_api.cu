@@ -13,6 +13,18 @@
 
 using namespace sp;
 
+cudaError_t sp::current_device(int* dev, int* sms) {
+  static PerDevice count;
+  cudaError_t e = cudaGetDevice(dev);
+  if (e != cudaSuccess) return e;
+  *sms = count.get(*dev, [&]() {
+    int n = 0;
+    e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, *dev);
+    return e == cudaSuccess ? n : 0;
+  });
+  return e;
+}
+
 // Scratch of spike_proj_decode_noalloc, one copy per device in static device
 // memory: the split-K workspace of one spike row at the largest N and one
 // ticket per 512-channel output tile.  Zero when the module loads; every

@@ -488,26 +488,24 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
   }
 }
 
-int g_dense_sms = 0;
-
-// Resident CTAs of dense_kernel<B> per SM (0 before the first query).
+// Resident CTAs of dense_kernel<B> per SM.
 template <int B>
-int dense_ctas_per_sm() {
-  static int n = 0;
-  if (n == 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dense_kernel<B>, kDenseThreads, 0) !=
-                    cudaSuccess) {
-    (void)cudaGetLastError();
-    n = 1;
-  }
-  return n > 0 ? n : 1;
+int dense_ctas_per_sm(int dev) {
+  static PerDevice ctas;
+  return ctas.get(dev, []() {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dense_kernel<B>, kDenseThreads, 0) != cudaSuccess)
+      (void)cudaGetLastError();
+    return n > 0 ? n : 1;
+  });
 }
 
 template <int B>
-cudaError_t launch_dense_t(const DenseParams& p, cudaStream_t s) {
+cudaError_t launch_dense_t(const DenseParams& p, int dev, int sms, cudaStream_t s) {
   // one wave of resident CTAs (never more than the units need): every unit a
   // warp takes from the grid-stride sequence starts without waiting for a CTA
   const int warps_per_cta = kDenseThreads / 32;
-  int grid = g_dense_sms * dense_ctas_per_sm<B>();
+  int grid = sms * dense_ctas_per_sm<B>(dev);
   const int need = (p.units + warps_per_cta - 1) / warps_per_cta;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
@@ -515,15 +513,14 @@ cudaError_t launch_dense_t(const DenseParams& p, cudaStream_t s) {
 }
 
 template <int B>
-cudaError_t launch_dense_mma(const DenseMmaParams& p, cudaStream_t s) {
-  static bool attr_done = false;
-  if (!attr_done) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        dense_mma_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMmaRingBytes + kMmaTableBytes);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
-  return launch_pdl(dense_mma_kernel<B>, dim3(g_dense_sms), dim3(kMmaThreads),
+cudaError_t launch_dense_mma(const DenseMmaParams& p, int dev, int sms, cudaStream_t s) {
+  static PerDevice attr;
+  const cudaError_t e = attr.once(dev, []() {
+    return cudaFuncSetAttribute(dense_mma_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kMmaRingBytes + kMmaTableBytes);
+  });
+  if (e != cudaSuccess) return e;
+  return launch_pdl(dense_mma_kernel<B>, dim3(sms), dim3(kMmaThreads),
                     (size_t)(kMmaRingBytes + p.table_bytes),
                     s, p);
 }
@@ -531,13 +528,9 @@ cudaError_t launch_dense_mma(const DenseMmaParams& p, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream_t s) {
-  if (g_dense_sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&g_dense_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  int dev = 0, sms = 0;
+  const cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
   // The tensor-core form where an activation table fits in shared memory and
   // the weights outweigh its start (it holds a whole SM, so it cannot start
   // beside the previous kernel).  us per call, FMAs / tensor cores: one row,
@@ -569,10 +562,10 @@ cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream
     }
     p.cost = cost;
     switch (B) {
-      case 1: return launch_dense_mma<1>(p, s);
-      case 2: return launch_dense_mma<2>(p, s);
-      case 3: return launch_dense_mma<3>(p, s);
-      default: return launch_dense_mma<4>(p, s);
+      case 1: return launch_dense_mma<1>(p, dev, sms, s);
+      case 2: return launch_dense_mma<2>(p, dev, sms, s);
+      case 3: return launch_dense_mma<3>(p, dev, sms, s);
+      default: return launch_dense_mma<4>(p, dev, sms, s);
     }
   }
   DenseParams p;
@@ -587,10 +580,10 @@ cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream
   for (int j = count; j < kDenseMaxProblems; ++j) p.unit_end[j] = units;
   p.units = units;
   switch (B) {
-    case 1: return launch_dense_t<1>(p, s);
-    case 2: return launch_dense_t<2>(p, s);
-    case 3: return launch_dense_t<3>(p, s);
-    default: return launch_dense_t<4>(p, s);
+    case 1: return launch_dense_t<1>(p, dev, sms, s);
+    case 2: return launch_dense_t<2>(p, dev, sms, s);
+    case 3: return launch_dense_t<3>(p, dev, sms, s);
+    default: return launch_dense_t<4>(p, dev, sms, s);
   }
 }
 

@@ -984,9 +984,6 @@ __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, in
   if (count.dev) count_spikes(active, count, false);
 }
 
-int g_num_sms = 0;
-bool g_attr_set = false;
-
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -1017,9 +1014,9 @@ bool encode_u8_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t o
 }
 
 // Largest number of clusters of `size` CTAs that can be resident at once.
-int max_active_clusters(int size) {
-  static int cache[9] = {0};
-  if (cache[size] == 0) {
+int max_active_clusters(int dev, int size) {
+  static PerDevice cache[9];
+  return cache[size].get(dev, [&]() {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1036,32 +1033,21 @@ int max_active_clusters(int size) {
       (void)cudaGetLastError();
       n = -1;
     }
-    cache[size] = n;
-  }
-  return cache[size];
+    return n;
+  });
 }
 
-cudaError_t set_gemm_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kGemmSmem);
+// The current device, its number of SMs, and gemm_kernel's attributes on it.
+cudaError_t gemm_init(int* dev, int* sms) {
+  static PerDevice attr;
+  const cudaError_t e = current_device(dev, sms);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 0);
-  if (e != cudaSuccess) return e;
-  done = true;
-  return cudaSuccess;
-}
-
-cudaError_t init_sms() {
-  if (g_attr_set) return cudaSuccess;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  g_attr_set = true;
-  return cudaSuccess;
+  return attr.once(*dev, []() {
+    const cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kGemmSmem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 0);
+  });
 }
 
 // K splits for a T x N output: split only when the tiles alone leave SMs
@@ -1075,12 +1061,12 @@ cudaError_t init_sms() {
 // the exchange costs more than it saves: 100 x 2048 x 768 at S = 6 8.6, 512 x
 // 1024 x 1024 (128 CTAs) at S = 8 9.4 against 8.7 at 4.
 constexpr int kSplitSmallCtas = 64;
-int pick_splits(int T, int N, int Kp, int part_units) {
+int pick_splits(int dev, int sms, int T, int N, int Kp, int part_units) {
   const int tiles = ceil_div(T, BM) * ceil_div(N, BN);
   const int nkb = Kp / BK;
   int S = 1;
-  if (tiles < g_num_sms) {
-    const int most = std::min(8, g_num_sms / tiles);
+  if (tiles < sms) {
+    const int most = std::min(8, sms / tiles);
     S = std::min(most, nkb / 3);
     const int fine = std::min(most, nkb / 2);
     if (tiles * fine <= kSplitSmallCtas && (S < 4 || fine == 8)) S = fine;
@@ -1088,7 +1074,7 @@ int pick_splits(int T, int N, int Kp, int part_units) {
     while (S > 1) {
       const int kbps = ceil_div(nkb, S);
       const int exact = ceil_div(nkb, kbps);            // splits with work
-      if (exact == S && max_active_clusters(S) >= tiles && tiles * S <= part_units) break;
+      if (exact == S && max_active_clusters(dev, S) >= tiles && tiles * S <= part_units) break;
       --S;
     }
   }
@@ -1150,9 +1136,9 @@ namespace {
 // Largest number of clusters of `cl` CTAs of gemm_group_kernel<cl> that can be
 // resident at once (-1 when the occupancy query fails).
 template <int CL>
-int group_active_clusters() {
-  static int n = 0;
-  if (n == 0) {
+int group_active_clusters(int dev) {
+  static PerDevice clusters;
+  return clusters.get(dev, []() {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1169,24 +1155,21 @@ int group_active_clusters() {
       (void)cudaGetLastError();
       c = -1;
     }
-    n = c;
-  }
-  return n;
+    return c;
+  });
 }
 
 template <int CL>
-cudaError_t launch_group_cl(const GemmGroupArgs& a, cudaStream_t s) {
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_group_kernel<CL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)GroupCfg<CL>::kSmem);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
-  int clusters = g_num_sms / CL;
+cudaError_t launch_group_cl(const GemmGroupArgs& a, int dev, int sms, cudaStream_t s) {
+  static PerDevice attr_set;
+  const cudaError_t e = attr_set.once(dev, []() {
+    return cudaFuncSetAttribute(gemm_group_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)GroupCfg<CL>::kSmem);
+  });
+  if (e != cudaSuccess) return e;
+  int clusters = sms / CL;
   if (CL > 1) {
-    const int resident = group_active_clusters<CL>();
+    const int resident = group_active_clusters<CL>(dev);
     if (resident < 1) return cudaErrorInvalidConfiguration;
     if (clusters > resident) clusters = resident;
   }
@@ -1244,26 +1227,27 @@ int gemm_group_cluster(const int* tiles_m, const int* tiles_n, int count) {
 }
 
 cudaError_t launch_gemm_group(const GemmGroupArgs& a, cudaStream_t s) {
-  cudaError_t e = init_sms();
+  int dev = 0, sms = 0;
+  const cudaError_t e = current_device(&dev, &sms);
   if (e != cudaSuccess) return e;
   if (a.units < 1) return cudaSuccess;
   switch (a.cl) {
-    case 1: return launch_group_cl<1>(a, s);
-    case 2: return launch_group_cl<2>(a, s);
+    case 1: return launch_group_cl<1>(a, dev, sms, s);
+    case 2: return launch_group_cl<2>(a, dev, sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 int gemm_splits(int T, int N, int Kp, int part_units) {
-  if (init_sms() != cudaSuccess || set_gemm_attrs() != cudaSuccess) return 1;
-  return pick_splits(T, N, Kp, part_units);
+  int dev = 0, sms = 0;
+  if (gemm_init(&dev, &sms) != cudaSuccess) return 1;
+  return pick_splits(dev, sms, T, N, Kp, part_units);
 }
 
 cudaError_t launch_gemm(const CUtensorMap& mapA, const CUtensorMap& mapB, int S, int T, int N,
                         int Kp, const GemmParams& p, cudaStream_t s) {
-  cudaError_t e = init_sms();
-  if (e != cudaSuccess) return e;
-  e = set_gemm_attrs();
+  int dev = 0, sms = 0;
+  const cudaError_t e = gemm_init(&dev, &sms);
   if (e != cudaSuccess) return e;
   GemmArgs a;
   a.p = p;
@@ -1274,7 +1258,7 @@ cudaError_t launch_gemm(const CUtensorMap& mapA, const CUtensorMap& mapB, int S,
   a.splits = S;
   a.units = a.tiles_m * a.tiles_n * S;
   if (S == 1) {
-    const int grid = a.units < g_num_sms ? a.units : g_num_sms;
+    const int grid = a.units < sms ? a.units : sms;
     return launch_pdl(gemm_kernel, dim3(grid), dim3(kGemmThreads), kGemmSmem, s, mapA, mapB, a);
   }
   cudaLaunchConfig_t cfg = {};

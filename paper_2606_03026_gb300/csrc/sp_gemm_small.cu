@@ -530,13 +530,11 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
   }
 }
 
-int g_sms = 0;
-
 // Largest number of clusters of `size` CTAs of gemm_small_kernel that can be
 // resident at once (-1 when the occupancy query fails).
-int small_active_clusters(int size) {
-  static int cache[kGemmSmallMaxS + 1] = {0};
-  if (cache[size] == 0) {
+int small_active_clusters(int dev, int size) {
+  static PerDevice cache[kGemmSmallMaxS + 1];
+  return cache[size].get(dev, [&]() {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -553,43 +551,40 @@ int small_active_clusters(int size) {
       (void)cudaGetLastError();
       n = -1;
     }
-    cache[size] = n;
-  }
-  return cache[size];
+    return n;
+  });
 }
 
-cudaError_t small_init() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmSmem);
+// The current device, its number of SMs, and the kernel's attribute on it.
+cudaError_t small_init(int* dev, int* sms) {
+  static PerDevice attr;
+  const cudaError_t e = current_device(dev, sms);
   if (e != cudaSuccess) return e;
-  done = true;
-  return cudaSuccess;
+  return attr.once(*dev, []() {
+    return cudaFuncSetAttribute(gemm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmSmem);
+  });
 }
 
 }  // namespace
 
 int gemm_small_splits(int T, int N, int Kp) {
-  if (T < 1 || T > kGemmSmallMaxT || small_init() != cudaSuccess) return 0;
+  int dev = 0, sms = 0;
+  if (T < 1 || T > kGemmSmallMaxT || small_init(&dev, &sms) != cudaSuccess) return 0;
   const int tiles = ceil_div(N, kSmM);
   const int nkb = Kp / kSmBK;
   // the most K ranges that keep every CTA's spike slice in shared memory,
   // every cluster resident at once and no SM holding two CTAs
   for (int S = kGemmSmallMaxS; S >= 1; S /= 2) {
-    if (S > nkb || ceil_div(nkb, S) > kGemmSmallMaxKB || tiles * S > g_sms) continue;
-    if (S > 1 && small_active_clusters(S) < tiles) continue;
+    if (S > nkb || ceil_div(nkb, S) > kGemmSmallMaxKB || tiles * S > sms) continue;
+    if (S > 1 && small_active_clusters(dev, S) < tiles) continue;
     return S;
   }
   return 0;
 }
 
 cudaError_t launch_gemm_small(const CUtensorMap& mapW, const GemmSmallArgs& a, cudaStream_t s) {
-  cudaError_t e = small_init();
+  int dev = 0, sms = 0;
+  const cudaError_t e = small_init(&dev, &sms);
   if (e != cudaSuccess) return e;
   if (a.S < 1 || a.S > kGemmSmallMaxS || (a.S & (a.S - 1)) != 0 || a.T < 1 || a.T > kGemmSmallMaxT || a.TN % 16 != 0 ||
       a.TN < a.T || a.TN > kGemmSmallMaxT || a.nkb < a.S || ceil_div(a.nkb, a.S) > kGemmSmallMaxKB)

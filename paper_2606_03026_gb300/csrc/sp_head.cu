@@ -734,34 +734,25 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
   if (p.cand && t < ks) p.cand[(int64_t)b * ks + t] = key_row(s_best[t]);
 }
 
-int g_head_sms = 0;
-
-template <typename Kern>
-cudaError_t raise_smem(Kern kernel, size_t bytes, size_t& set_bytes) {
-  if (bytes <= set_bytes) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) set_bytes = bytes;
-  return e;
-}
-
 template <int B>
-cudaError_t launch_head_t(HeadParams p, cudaStream_t s) {
+cudaError_t launch_head_t(HeadParams p, int dev, int sms, cudaStream_t s) {
   // The largest shared-memory carve-out for the selection too: with a smaller
   // one its SM could not take a projection CTA beside it (the next call's,
   // which starts while the selection runs), and the late CTA held up the call.
-  static bool carve_done = false;
-  if (!carve_done) {
-    const cudaError_t e = cudaFuncSetAttribute(head_select_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                               (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    carve_done = true;
-  }
-  static size_t set_proj = 0;    // per instance: head_kernel<B> is a kernel of its own
-  const size_t smem = kHeadRingBytes + (size_t)B * (p.Kpad + kCodePad);
-  cudaError_t e = raise_smem(head_kernel<B>, smem, set_proj);
+  static PerDevice carve, ring;  // per instance: head_kernel<B> is a kernel of its own
+  cudaError_t e = carve.once(dev, []() {
+    return cudaFuncSetAttribute(head_select_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                (int)cudaSharedmemCarveoutMaxShared);
+  });
   if (e != cudaSuccess) return e;
+  e = ring.once(dev, []() {
+    return cudaFuncSetAttribute(head_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kHeadRingBytes + (size_t)B * (SPIKE_PROJ_HEAD_MAX_K + kCodePad)));
+  });
+  if (e != cudaSuccess) return e;
+  const size_t smem = kHeadRingBytes + (size_t)B * (p.Kpad + kCodePad);
   // one wave, one CTA per SM
-  int grid = g_head_sms;
+  int grid = sms;
   if (grid > p.units) grid = p.units;
   if (grid > kHeadMaxGrid) grid = kHeadMaxGrid;
   p.nctas = grid;
@@ -788,13 +779,9 @@ cudaError_t launch_head_t(HeadParams p, cudaStream_t s) {
 size_t head_workspace_bytes() { return kListBytes + kLeadBytes; }
 
 cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
-  if (g_head_sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&g_head_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  int dev = 0, sms = 0;
+  const cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
   HeadParams p;
   p.W = a.W;
   p.ldw = a.ldw;
@@ -819,10 +806,10 @@ cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
   p.lead = reinterpret_cast<hkey*>(static_cast<unsigned char*>(a.ws) + kListBytes);
   p.nctas = 0;
   switch (a.B) {
-    case 1: return launch_head_t<1>(p, s);
-    case 2: return launch_head_t<2>(p, s);
-    case 3: return launch_head_t<3>(p, s);
-    default: return launch_head_t<4>(p, s);
+    case 1: return launch_head_t<1>(p, dev, sms, s);
+    case 2: return launch_head_t<2>(p, dev, sms, s);
+    case 3: return launch_head_t<3>(p, dev, sms, s);
+    default: return launch_head_t<4>(p, dev, sms, s);
   }
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "spike_proj.h"
 
 namespace sp {
@@ -206,6 +208,36 @@ struct HeadArgs {
 };
 size_t head_workspace_bytes();
 cudaError_t launch_head(const HeadArgs& a, cudaStream_t s);
+
+// What a launcher keeps of a device (an attribute it has set on a kernel, an
+// occupancy, a number of SMs) holds for that device alone, and several host
+// threads may make the first calls: one atomic value per device, 0 = not yet
+// asked for.  Devices past kMaxDevices are asked every time.
+constexpr int kMaxDevices = 64;
+struct PerDevice {
+  std::atomic<int> value[kMaxDevices] = {};
+  // the device's value, from query() (not 0) the first time
+  template <typename Query>
+  int get(int dev, Query query) {
+    int n = dev < kMaxDevices ? value[dev].load(std::memory_order_relaxed) : 0;
+    if (n == 0) {
+      n = query();
+      if (dev < kMaxDevices) value[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
+  }
+  // set() until it has succeeded once on the device
+  template <typename Set>
+  cudaError_t once(int dev, Set set) {
+    if (dev < kMaxDevices && value[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    const cudaError_t e = set();
+    if (e == cudaSuccess && dev < kMaxDevices) value[dev].store(1, std::memory_order_relaxed);
+    return e;
+  }
+};
+
+// The current device and its number of SMs.
+cudaError_t current_device(int* dev, int* sms);
 
 // Launches `kernel` with programmatic stream serialization: its blocks may
 // become resident while the previous kernel of the stream is still running

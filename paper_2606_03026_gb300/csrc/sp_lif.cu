@@ -156,16 +156,10 @@ lif_kernel_v4(const __grid_constant__ LifParams p) {
   }
 }
 
-int g_lif_sms = 0;
-
 cudaError_t launch_lif_params(const LifParams& p, cudaStream_t s) {
-  if (g_lif_sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&g_lif_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  int dev = 0, sms = 0;
+  const cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
   // the vector form for large states only: at decode sizes (a few hundred
   // thousand neurons) its small grid made the following decode launch start
   // later (producer + decode step 16.2 against 14.7 us with the scalar form)
@@ -175,7 +169,7 @@ cudaError_t launch_lif_params(const LifParams& p, cudaStream_t s) {
   const int64_t total_warps =
       vec ? ((int64_t)p.rows * ((p.K + 127) / 128) + 1) / 2 : (int64_t)p.rows * ((p.K + 31) / 32);
   const int64_t need = (total_warps + kLifThreads / 32 - 1) / (kLifThreads / 32);
-  int64_t grid = (int64_t)g_lif_sms * 8;
+  int64_t grid = (int64_t)sms * 8;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   if (vec) return launch_pdl(lif_kernel_v4, dim3((unsigned)grid), dim3(kLifThreads), 0, s, p);

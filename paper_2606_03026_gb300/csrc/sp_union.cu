@@ -224,29 +224,27 @@ __global__ void density_kernel(const void* spikes, int fmt, int64_t ld, int B, i
   count_spikes(total, count, true);
 }
 
-int g_union_grid = 0;
-
 }  // namespace
 
 cudaError_t launch_union(const UnionParams& p, cudaStream_t s) {
   if (p.B <= 0) return cudaSuccess;
   if (p.B > kUnionMaxRows) return cudaErrorInvalidValue;
-  if (g_union_grid == 0) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(union_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kUnionSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, union_kernel, kUnionThreads,
-                                                      kUnionSmem);
-    if (e != cudaSuccess) return e;
-    g_union_grid = sms * (per_sm > 0 ? per_sm : 1);
-  }
+  static PerDevice attr, ctas;               // resident CTAs per SM
+  int dev = 0, sms = 0;
+  cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  e = attr.once(dev, []() {
+    return cudaFuncSetAttribute(union_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUnionSmem);
+  });
+  if (e != cudaSuccess) return e;
+  const int per_sm = ctas.get(dev, [&]() {
+    int n = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, union_kernel, kUnionThreads, kUnionSmem);
+    return e != cudaSuccess ? 0 : n > 0 ? n : 1;
+  });
+  if (e != cudaSuccess) return e;
   const int units = ceil_div(p.N, kUnionNT) * ceil_div(p.K, kUnionCK);
-  const int grid = units < g_union_grid ? units : g_union_grid;
+  const int grid = units < sms * per_sm ? units : sms * per_sm;
   union_kernel<<<grid, kUnionThreads, kUnionSmem, s>>>(p);
   return cudaGetLastError();
 }

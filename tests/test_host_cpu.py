@@ -1,0 +1,87 @@
+"""The library's host side (launch choice, attributes, error paths) on fake
+devices: its objects linked to a stand-in of the CUDA runtime that checks
+launches and runs no kernel (fake_cudart.cpp).  No GPU."""
+import ctypes
+import subprocess
+from pathlib import Path
+
+import pytest
+
+from paper_2606_03026_gb300 import _build, spikeproj as sp
+
+HERE = Path(__file__).resolve().parent
+FAKE = 1 << 30                                # addresses that no host code reads
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    _build.build()
+    out = tmp_path_factory.mktemp("fake") / "libspikeproj_fake.so"
+    cuda = Path(_build.nvcc()).resolve().parent.parent / "include"
+    objs = [_build.OUT / (src.stem + ".o") for src in _build.sources()]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-pthread", "-Wl,-Bsymbolic", f"-I{cuda}",
+                    f"-I{_build.INCLUDE}", f"-I{_build.CSRC}", str(HERE / "fake_cudart.cpp"), *map(str, objs),
+                    "-o", str(out)], check=True)
+    lib = ctypes.CDLL(str(out))
+    for name, (args, res) in sp._SIGNATURES.items():
+        fn = getattr(lib, name)
+        fn.argtypes, fn.restype = args, res
+    return lib
+
+
+@pytest.fixture(autouse=True)
+def reset(lib):
+    lib.fake_fail(b"")
+    lib.fake_counts(0, 0)
+    lib.fake_device(0)
+    lib.fake_launches(), lib.fake_syncs(), lib.fake_stream_syncs()
+
+
+def make_plan(lib, N=1536, K=6144, rows=512):
+    h = ctypes.c_void_p()
+    assert lib.spike_proj_plan(ctypes.byref(h), FAKE, N, FAKE, N, K, rows, sp.SP_PLAN_GEMM, None) == sp.SP_OK
+    return h
+
+
+def dense(lib, shapes, B):
+    table = (sp.SpDense * len(shapes))()
+    for j, (N, K) in enumerate(shapes):
+        ld = (K + 15) // 16 * 16
+        table[j] = sp.SpDense(FAKE, ld, FAKE, FAKE, ld, FAKE, N, N, K)
+    return lib.spike_proj_dense(ctypes.addressof(table), len(shapes), B, None)
+
+
+@pytest.mark.parametrize("first", [0, 1])
+def test_every_call_on_either_device(lib, first):
+    """What a launch needs of a device (attributes, occupancy, SM count) is
+    set on each device a call is made on, not on the first one alone."""
+    for dev in (first, 1 - first, first):
+        lib.fake_device(dev)
+        for B in range(1, sp.SPIKE_PROJ_DENSE_MAX_B + 1):
+            assert dense(lib, [(4608, 6144 if B <= 2 else 3072)] * 3, B) == sp.SP_OK, f"dense B={B} on {dev}"
+            assert dense(lib, [(64, 256)], B) == sp.SP_OK
+        for V, K in ((57344, 1536), (3000, 8192)):
+            head = ctypes.c_void_p()
+            assert lib.spike_proj_head_create(ctypes.byref(head), FAKE, K, FAKE, V, K, None) == sp.SP_OK
+            for B in range(1, 5):
+                assert lib.spike_proj_head(head, FAKE, K, B, 0.5, 64, FAKE, None, None, None, None, None, 0,
+                                           None) == sp.SP_OK, f"head B={B} K={K} on {dev}"
+            assert lib.spike_proj_head_destroy(head) == sp.SP_OK
+        plans = [make_plan(lib) for _ in range(2)]
+        for T in (1, 5, 16, 64, 100, 512):
+            for strategy in ("gather", "gemm", "union"):
+                assert lib.spike_proj_batched(plans[0], FAKE, sp.SP_SPIKES_U8, T, 6144, FAKE, FAKE,
+                                              sp.KERNELS[strategy], None) == sp.SP_OK, f"{strategy} T={T} on {dev}"
+        assert lib.spike_proj_decode(plans[0], FAKE, sp.SP_SPIKES_U8, FAKE, FAKE, None) == sp.SP_OK
+        assert lib.spike_proj_lif(FAKE, FAKE, 4096, 8, 4096, 0.9, 1.0, FAKE, 128, None) == sp.SP_OK
+        group = ctypes.c_void_p()
+        two = (ctypes.c_void_p * 2)(*plans)
+        rows = (ctypes.c_void_p * 2)(FAKE, FAKE)
+        assert lib.spike_proj_group_create(ctypes.byref(group), two, 2, None) == sp.SP_OK
+        assert lib.spike_proj_group_decode(group, FAKE, sp.SP_SPIKES_U8, 6144, FAKE, FAKE, 1536, None) == sp.SP_OK
+        for T in (100, 256):                  # single CTAs and CTA pairs
+            assert lib.spike_proj_group_prefill(group, rows, sp.SP_SPIKES_BOOL8, T, 6144, rows, rows,
+                                                None) == sp.SP_OK, f"group prefill T={T} on {dev}"
+        assert lib.spike_proj_group_destroy(group) == sp.SP_OK
+        for p in plans:
+            assert lib.spike_proj_plan_destroy(p) == sp.SP_OK
