@@ -418,6 +418,9 @@ sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
       if (st == SP_OK) {
         p->last_kernel = SP_GEMM;
         p->count_pending = true;
+      } else {
+        // the staging pass may have added its count, which no GEMM takes now
+        (void)cudaMemsetAsync(p->d_counts, 0, 2 * sizeof(int32_t), s);
       }
       return st;
     }
@@ -612,6 +615,7 @@ sp_status spike_proj_plan_status(sp_plan_t plan, sp_stream_t stream) {
   SP_CUDA(cudaMemsetAsync(plan->err, 0, sizeof(int), s));
   SP_CUDA(cudaMemsetAsync(plan->ws, 0, (size_t)plan->max_batch * plan->N * sizeof(int32_t), s));
   SP_CUDA(cudaMemsetAsync(plan->tickets, 0, plan->n_tickets * sizeof(uint32_t), s));
+  SP_CUDA(cudaMemsetAsync(plan->d_counts, 0, 2 * sizeof(int32_t), s));
   SP_CUDA(cudaStreamSynchronize(s));
   return SP_EKERNEL;
 }

@@ -43,6 +43,17 @@ def make_plan(lib, N=1536, K=6144, rows=512):
     return h
 
 
+def auto(lib, plan, T=173, K=6144):
+    """SP_AUTO on byte rows where the GEMM is picked whatever the count."""
+    return lib.spike_proj_batched(plan, FAKE, sp.SP_SPIKES_U8, T, K, FAKE, FAKE, sp.SP_AUTO, None)
+
+
+def last_dispatch(lib, plan):
+    chosen, count = ctypes.c_int(), ctypes.c_int32()
+    assert lib.spike_proj_last_dispatch(plan, ctypes.byref(chosen), ctypes.byref(count)) == sp.SP_OK
+    return chosen.value, count.value
+
+
 def dense(lib, shapes, B):
     table = (sp.SpDense * len(shapes))()
     for j, (N, K) in enumerate(shapes):
@@ -85,3 +96,18 @@ def test_every_call_on_either_device(lib, first):
         assert lib.spike_proj_group_destroy(group) == sp.SP_OK
         for p in plans:
             assert lib.spike_proj_plan_destroy(p) == sp.SP_OK
+
+
+def test_count_after_a_failed_launch(lib):
+    """A GEMM that cannot be launched after the pass that counts the spikes
+    has been: the next call's count is its own."""
+    plan = make_plan(lib)
+    lib.fake_counts(100, 0)
+    lib.fake_fail(b"gemm_kernel")
+    for _ in range(2):
+        assert auto(lib, plan) == sp.SP_ECUDA
+    lib.fake_fail(b"")
+    lib.fake_counts(70, 0)
+    assert auto(lib, plan) == sp.SP_OK
+    assert last_dispatch(lib, plan) == (sp.SP_GEMM, 70)
+    assert lib.spike_proj_plan_destroy(plan) == sp.SP_OK
