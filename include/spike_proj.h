@@ -207,8 +207,10 @@ sp_status spike_proj_prefill(sp_plan_t plan, const uint8_t *X, int32_t T,
 
 /* Strategy and total active count (sum over rows of |A|) of the last
  * batched / prefill call with SP_AUTO on this plan; the count is -1 when the
- * last call did not measure it.  Synchronises the device if the kernel that
- * counts has not finished. */
+ * last call did not measure it.  If the kernel that counts has still to run,
+ * the call waits for the count on the host, without a CUDA call (other streams
+ * and a capture on one are left alone); it synchronises the plan's device only
+ * when the count has not come after two seconds. */
 sp_status spike_proj_last_dispatch(sp_plan_t plan, sp_kernel *chosen,
                                    int32_t *active_count);
 

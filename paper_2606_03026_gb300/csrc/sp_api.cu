@@ -4,9 +4,11 @@
 #include <atomic>
 #include <cstdlib>
 #include <algorithm>
+#include <chrono>
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <thread>
 
 #include "sp_gemm.h"
 #include "sp_internal.h"
@@ -50,7 +52,8 @@ struct sp_plan_s {
   int32_t* d_counts = nullptr;    // spike count in progress and its tickets (SpikeCount)
   uint64_t* h_count = nullptr;    // page-locked: the last count and the sequence number it is of (SpikeCount)
   uint32_t count_seq = 0;         // counts asked for
-  bool count_pending = false;     // last_active is still to be read from h_count
+  bool count_pending = false;     // last_active is still to be read from h_count,
+  uint32_t pending_seq = 0;       // under this sequence number
   // tensor-core path
   uint8_t* Wq = nullptr;          // [N][2 Kp] e4m3 weight planes (16 h, l)
   uint8_t* Xs = nullptr;          // [xs_rows][Kp] 0/1 spike staging
@@ -391,11 +394,15 @@ sp_kernel choose(const sp_plan_s* p, int B, int32_t total) {
   return gemm_us < gather_us ? SP_GEMM : SP_GATHER;
 }
 
-// The count of the plan's last SP_AUTO call, -1 while it is not published.
-int32_t published_count(const sp_plan_s* p) {
+// The plan's count of sequence number seq, -1 while it is not published.
+int32_t published_count(const sp_plan_s* p, uint32_t seq) {
   const uint64_t word = __atomic_load_n(p->h_count, __ATOMIC_ACQUIRE);
-  return (uint32_t)(word >> 32) == p->count_seq ? (int32_t)(uint32_t)word : -1;
+  return (uint32_t)(word >> 32) == seq ? (int32_t)(uint32_t)word : -1;
 }
+
+// How long spike_proj_last_dispatch waits for a count before it turns to the
+// device (the kernels ahead of it on its stream take microseconds each).
+constexpr std::chrono::seconds kCountWait{2};
 
 sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld, int32_t* acc,
                     float* y, sp_kernel strategy, cudaStream_t s) {
@@ -418,6 +425,7 @@ sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
       if (st == SP_OK) {
         p->last_kernel = SP_GEMM;
         p->count_pending = true;
+        p->pending_seq = count.seq;
       } else {
         // the staging pass may have added its count, which no GEMM takes now
         (void)cudaMemsetAsync(p->d_counts, 0, 2 * sizeof(int32_t), s);
@@ -426,7 +434,7 @@ sp_status run_multi(sp_plan_s* p, const void* spikes, int fmt, int B, int64_t ld
     }
     SP_CUDA(launch_density(spikes, fmt, ld, B, p->K, count, s));
     SP_CUDA(cudaStreamSynchronize(s));
-    p->last_active = published_count(p);
+    p->last_active = published_count(p, count.seq);
     strategy = choose(p, B, p->last_active);
     p->last_kernel = strategy;
     p->count_pending = false;
@@ -591,11 +599,24 @@ sp_status spike_proj_prefill(sp_plan_t plan, const uint8_t* X, int32_t T, int64_
 sp_status spike_proj_last_dispatch(sp_plan_t plan, sp_kernel* chosen, int32_t* active_count) {
   if (!plan) return SP_EINVAL;
   if (plan->count_pending) {
-    // the counting kernel of the last SP_AUTO call may still be running
-    int32_t count = published_count(plan);
+    // The GEMM of the last SP_AUTO call may still be to run: its count is
+    // waited for without a CUDA call, which would stall other streams, or
+    // break a capture on one.  Past kCountWait (the stream is far behind, or
+    // the device has failed) the plan's device is synchronised after all.
+    const auto t0 = std::chrono::steady_clock::now();
+    int32_t count = published_count(plan, plan->pending_seq);
+    while (count < 0 && std::chrono::steady_clock::now() - t0 < kCountWait) {
+      std::this_thread::yield();
+      count = published_count(plan, plan->pending_seq);
+    }
     if (count < 0) {
-      SP_CUDA(cudaDeviceSynchronize());
-      count = published_count(plan);
+      int dev = 0;
+      SP_CUDA(cudaGetDevice(&dev));
+      if (dev != plan->device) SP_CUDA(cudaSetDevice(plan->device));
+      const cudaError_t e = cudaDeviceSynchronize();
+      if (dev != plan->device) SP_CUDA(cudaSetDevice(dev));
+      SP_CUDA(e);
+      count = published_count(plan, plan->pending_seq);
     }
     plan->last_active = count;
     plan->count_pending = false;

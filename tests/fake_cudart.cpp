@@ -29,7 +29,7 @@ struct State {
   std::string fail;                                            // launches of kernels with this in the name fail
   int active = 0;                                              // spikes that a counting kernel finds
   int publish_ms = 0;                                          // delay of a publication (< 0: it never comes)
-  int launches = 0, syncs = 0, stream_syncs = 0;
+  int launches = 0, synced = -1;                               // synced: the device last synchronised
   size_t pushed_smem = 0;                                      // of a <<<...>>> launch
   std::vector<std::thread> pending;
 };
@@ -94,8 +94,7 @@ void fake_counts(int active, int publish_ms) {
 }
 void fake_device(int device) { state().device = device; }
 int fake_launches() { return std::exchange(state().launches, 0); }
-int fake_syncs() { return std::exchange(state().syncs, 0); }
-int fake_stream_syncs() { return std::exchange(state().stream_syncs, 0); }
+int fake_synced() { return std::exchange(state().synced, -1); }
 
 // ---- the runtime ------------------------------------------------------------
 void** __cudaRegisterFatBinary(void*) { return reinterpret_cast<void**>(&state()); }
@@ -151,12 +150,11 @@ cudaError_t cudaDeviceGetAttribute(int* value, cudaDeviceAttr attr, int) {
 }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() {
-  ++state().syncs;
+  state().synced = state().device;
   finish_pending();
   return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t) {
-  ++state().stream_syncs;
   finish_pending();
   return cudaSuccess;
 }

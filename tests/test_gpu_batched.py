@@ -353,3 +353,34 @@ def test_auto_count_is_of_the_call_before():
         if i % 3:                                # several calls in flight before the question, or none
             assert plan.last_dispatch() == want[i % 4], f"call {i}"
     plan.close()
+
+
+def test_last_dispatch_beside_a_capture():
+    """Asking for a count that is still to come leaves a capture on another
+    stream alone."""
+    N, K, T = 512, 512, 128
+    Qc, s, _ = synth.random_case(95, N, K)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=T, gemm=True)
+    X = synth.bernoulli(synth.rng_for(7306), (T, K), 0.2)
+    xd = to_dev(X)
+    y = torch.empty(T, N, dtype=torch.float32, device=DEV)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    out = torch.ones(8, device=DEV)
+    with torch.cuda.stream(a):
+        plan.batched(xd, "u8", T, K, None, y, "auto")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(b):
+        graph.capture_begin()
+        out.add_(1)
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(20_000_000)                # about 10 ms: the count comes after the question
+        plan.batched(xd, "u8", T, K, None, y, "auto")
+        assert plan.last_dispatch() == ("gemm", int(X.astype(np.int64).sum()))
+    with torch.cuda.stream(b):
+        out.mul_(3)
+        graph.capture_end()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert torch.all(out == 6)
+    plan.close()

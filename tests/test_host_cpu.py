@@ -34,7 +34,7 @@ def reset(lib):
     lib.fake_fail(b"")
     lib.fake_counts(0, 0)
     lib.fake_device(0)
-    lib.fake_launches(), lib.fake_syncs(), lib.fake_stream_syncs()
+    lib.fake_launches(), lib.fake_synced()
 
 
 def make_plan(lib, N=1536, K=6144, rows=512):
@@ -110,4 +110,37 @@ def test_count_after_a_failed_launch(lib):
     lib.fake_counts(70, 0)
     assert auto(lib, plan) == sp.SP_OK
     assert last_dispatch(lib, plan) == (sp.SP_GEMM, 70)
+    assert lib.spike_proj_plan_destroy(plan) == sp.SP_OK
+
+
+def test_last_dispatch_waits_without_the_device(lib):
+    """The count of a call that did not wait for it is waited for on the host:
+    no synchronisation, which would stall other streams and break a capture
+    elsewhere.  A count that never comes is -1 and not an earlier call's, after
+    a synchronisation of the plan's own device."""
+    lib.fake_device(1)
+    plan = make_plan(lib)
+    lib.fake_device(0)
+    for active, ms in ((5, 0), (90, 60), (12, 5)):
+        lib.fake_counts(active, ms)
+        assert auto(lib, plan) == sp.SP_OK
+        assert last_dispatch(lib, plan) == (sp.SP_GEMM, active)
+        assert lib.fake_synced() == -1
+    lib.fake_counts(33, -1)
+    assert auto(lib, plan) == sp.SP_OK
+    assert last_dispatch(lib, plan) == (sp.SP_GEMM, -1)
+    assert lib.fake_synced() == 1
+    device = ctypes.c_int()
+    assert lib.cudaGetDevice(ctypes.byref(device)) == 0 and device.value == 0
+    assert lib.spike_proj_plan_destroy(plan) == sp.SP_OK
+
+
+def test_last_dispatch_after_a_failed_call(lib):
+    """A call that fails leaves the call before it the last one."""
+    plan = make_plan(lib)
+    lib.fake_counts(41, 30)
+    assert auto(lib, plan) == sp.SP_OK
+    lib.fake_fail(b"spikes_to_01")
+    assert auto(lib, plan) == sp.SP_ECUDA
+    assert last_dispatch(lib, plan) == (sp.SP_GEMM, 41)
     assert lib.spike_proj_plan_destroy(plan) == sp.SP_OK
