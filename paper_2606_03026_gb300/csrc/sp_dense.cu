@@ -20,10 +20,18 @@
 // exact part of the FP32 product and only the additions round.  Per warp: 16
 // weight rows as the MMA's M, the split activations of all B rows as its N
 // (columns 4 b + {0, 1, 2} = hi, mid, lo of row b), 64 weight columns per
-// chunk.  The chunk's MMAs start from zero and their sums are added to the
-// running FP32 sums of the lane, so the tensor core's own accumulation chain
-// is four MMAs long; at the end y = s * (hi + (mid + lo)).  Relative error
-// (2-norm, K = 1536, N(0, 1) activations) 8.2e-8, against 1.4e-7 with FMAs.
+// chunk.  Every MMA starts from zero, the sums of a chunk's four meet in pairs
+// and are added to the running FP32 sums of the lane; at the end
+// y = s * (hi + (mid + lo)).  How an MMA rounds its sum of 16 products is not
+// specified; on this device each product is cut to a multiple of 2^-24 of the
+// largest one's leading power of two and the sum to 24 bits.  So 16 products
+// lose at most 17 units u = 2^-24 of sum |W x|, the two additions of a chunk 2,
+// the running sum one per chunk and the three parts 2: depth 22 + ceil(K / 64).
+// (With the four MMAs of a chunk chained through their accumulator a large
+// product cost 63 others their last bits: 24.5 units measured at K = 64, 8.6 this way,
+// 10.7 with FMAs.  The additions are packed two to an instruction: for
+// four rows 1 to 2 us a call, nothing for one.)  Relative error (2-norm, K =
+// 1536, N(0, 1) activations) 8.2e-8, against 1.4e-7 with FMAs.
 // Bounds and layout:
 //   - with FP32 FMAs the kernel is bound by instructions and L1 (per weight a
 //     byte permute, an FADD and B FFMAs, and every lane re-reads the
@@ -179,22 +187,27 @@ constexpr int kMmaTile = 1024;
 constexpr int kMmaRingBytes = kMmaWarps * kMmaRing * kMmaRows * kMmaChunk;
 constexpr int kMmaTableBytes = 224 * 1024 - kMmaRingBytes;
 
-// d (+)= A B for one 16 x 16 x 8 step (kFirst: d is overwritten).
-template <bool kFirst>
+// d = A B for one 16 x 16 x 8 step.
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                          uint32_t a3, uint32_t b0, uint32_t b1) {
-  if (kFirst)
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-        "{%8, %9}, {%10, %10, %10, %10};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
-  else
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-        "{%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// Two FP32 values, added each by itself (round to nearest) in one instruction.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair(const float (&d)[4], int e) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(d[2 * e]), "f"(d[2 * e + 1]));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
 }
 
 __device__ __forceinline__ void cp_async16(uint4* dst, const int8_t* src) {
@@ -428,11 +441,9 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
       const DenseProblem& P = p.prob[j];
       const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kMmaRows;
       const int nch = (P.K + kMmaChunk - 1) / kMmaChunk;
-      float run[NT][4];
+      f32x2 run[NT][2];
 #pragma unroll
-      for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) run[n][e] = 0.f;
+      for (int n = 0; n < NT; ++n) run[n][0] = run[n][1] = 0ull;
       const uint4* tab = reinterpret_cast<const uint4*>(s_tab + base) + lane;
       for (int c0 = 0; c0 < nch; c0 += kMmaRing) {
 #pragma unroll
@@ -443,9 +454,10 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
             const uint32_t wa[4] = {w0.x, w0.y, w0.z, w0.w};
             const uint32_t wb[4] = {w1.x, w1.y, w1.z, w1.w};
             const uint4* tc = tab + (c0 + s) * NT * (kMmaTile / 16);
-            float part[NT][4];
+            f32x2 chunk[NT][2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
+              float part[2][NT][4];
               uint4 bf[NT];
 #pragma unroll
               for (int n = 0; n < NT; ++n) bf[n] = tc[n * (kMmaTile / 16) + 32 * h];
@@ -457,15 +469,18 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
 #pragma unroll
                 for (int n = 0; n < NT; ++n) {
                   const uint32_t b0 = m ? bf[n].z : bf[n].x, b1 = m ? bf[n].w : bf[n].y;
-                  if (h == 0 && m == 0) mma_bf16<true>(part[n], a0, a1, a2, a3, b0, b1);
-                  else mma_bf16<false>(part[n], a0, a1, a2, a3, b0, b1);
+                  mma_bf16(part[m][n], a0, a1, a2, a3, b0, b1);
                 }
               }
+#pragma unroll
+              for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  const f32x2 sum = add2(pair(part[0][n], e), pair(part[1][n], e));
+                  if (h == 0) chunk[n][e] = sum;
+                  else run[n][e] = add2(run[n][e], add2(chunk[n][e], sum));
+                }
             }
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) run[n][e] = __fadd_rn(run[n][e], part[n][e]);
           }
           load(s);
         }
@@ -476,8 +491,9 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
       for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          const float lo = __shfl_xor_sync(0xffffffffu, run[n][2 * e], 1);
-          const float sum = __fadd_rn(run[n][2 * e], __fadd_rn(run[n][2 * e + 1], lo));
+          const float a0 = __uint_as_float((uint32_t)run[n][e]), a1 = __uint_as_float((uint32_t)(run[n][e] >> 32));
+          const float lo = __shfl_xor_sync(0xffffffffu, a0, 1);
+          const float sum = __fadd_rn(a0, __fadd_rn(a1, lo));
           const int b = 2 * n + (t >> 1), row = row0 + g + 8 * e;
           if ((t & 1) == 0 && b < B && row < P.N)
             P.y[(int64_t)b * P.ldy + row] = __fmul_rn(__ldg(P.scale + row), sum);

@@ -261,3 +261,42 @@ def test_dense_errors():
     sp.spike_proj_dense([good], 1)
     torch.cuda.synchronize()
     assert torch.equal(y, torch.zeros_like(y))
+
+
+def tensor_bound(K, s, mag, want):
+    """The bound of the tensor-core form: depth 22 + ceil(K / 64)."""
+    d = 22 + (K + 63) // 64
+    gamma = d * U / (1 - d * U)
+    return np.abs(s) * gamma * mag + U * np.abs(want)
+
+
+@pytest.mark.parametrize("K,N", [(64, 30000), (512, 6400), (1536, 3072)])
+@pytest.mark.parametrize("B", [1, 2, 3, 4])
+def test_dense_tensor_form_one_large_product(B, K, N):
+    """One product that dwarfs the others of its sum, at every position of a
+    64-column chunk, the others of one sign and just below what an FP32 sum of
+    its size holds: every addition may lose all of one, which the bound allows
+    for.  (A sum of more products than the bound counts on would break it.)"""
+    N = N if B > 2 else N * 9600 // 2560 if B == 2 else N * 10
+    rng = synth.rng_for(714, K, B)
+    W = np.ones((N, K), np.int8)
+    W[16:] = rng.integers(1, 128, (N - 16, K))
+    W[:16, :] = 1
+    s = np.ones(N, np.float32)
+    Wd, sd = to_dev(W), to_dev(s)
+    rows = np.r_[0:16, rng.choice(np.arange(16, N), 48, replace=False)]
+    y = torch.empty(B, N, device=DEV)
+    for p0 in range(0, 64, B):
+        for small in (1.9921875 * 2.0 ** -25, 1.75 * 2.0 ** -24, 2.0 ** -21):
+            x = np.full((B, K), small, np.float32)
+            x[:, 1::2] *= np.float32(1 + 2.0 ** -14)          # parts below the leading one too
+            for b in range(B):
+                x[b, (p0 + b) % 64] = 1.0
+            xd = to_dev(x)
+            sp.spike_proj_dense([(Wd, K, sd, xd, K, y, N, N, K)], B)
+            got = y.cpu().numpy()[:, rows].astype(np.float64)
+            prod = x[:, None, :].astype(np.float64) * W[rows][None].astype(np.float64)
+            want = prod.sum(-1)
+            err = np.abs(got - want)
+            worst = (err / tensor_bound(K, 1.0, np.abs(prod).sum(-1), want)).max()
+            assert worst <= 1, f"K={K} B={B} position {p0} small {small}: {worst:.2f} of the bound"
