@@ -373,9 +373,14 @@ sp_status spike_proj_decode_noalloc(const int8_t *W, int64_t ldw,
  *     y[b*ldy + m] = s_m * sum_{k<K} float(W[m*ldw + k]) * x[b*ldx + k]
  *
  * computed in FP32: every product is exact (or, with FMAs, enters its
- * addition unrounded) and the sums round in FP32 in an order fixed by the
- * sizes of the call, so a result is identical on every run; one FP32 multiply
- * applies s_m.  |y - s_m * exact| <= |s_m| * gamma(d) * sum_k |W x| + u |y|
+ * addition unrounded) and the sums round in FP32 in a fixed order, so a result
+ * is identical on every run; one FP32 multiply applies s_m.  There are two
+ * forms of the sum, which may differ in the last bits.  Which one is taken
+ * depends on the sizes of the launch (its weight bytes, B and the widest K: the
+ * same projection alone and in a step may take different ones) and, for an
+ * activation row with a value that is not finite or outside 2^-100 .. 2^100, on
+ * that row; given the form, a row's result depends on nothing but the row, its
+ * weights and K.  |y - s_m * exact| <= |s_m| * gamma(d) * sum_k |W x| + u |y|
  * with u = 2^-24, gamma(d) = d u / (1 - d u) and
  *   - d = 16 * ceil(K / 512) + 5 for small launches and large K: lane l of a
  *     warp sums the 16-column chunks l, l + 32, ... with fmaf in ascending k,

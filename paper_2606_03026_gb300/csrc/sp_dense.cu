@@ -65,11 +65,13 @@
 // gives y: an FP32 sum of K products of depth at most 16 * ceil(K / 512) + 5.
 // Its small CTAs start while the previous kernel drains: 2.2 us a call at
 // 0.5 MB, where the tensor-core form, which fills its SM, takes 4.1.
-// dense_mma_kernel runs a problem with FMAs too when an activation is not
-// finite or outside 2^-100 .. 2^100 (its three parts would not be exact).
+// dense_mma_kernel runs an activation row with FMAs too when one of its values
+// is not finite or outside 2^-100 .. 2^100 (its three parts would not be exact).
 //
-// In both forms the order of every sum depends on the sizes alone, so the
-// result is the same on every run.
+// In both forms the order of a sum depends on K alone, so the result is the
+// same on every run, and a row's does not depend on the other rows of the call
+// or on the other problems of the launch, but through the choice of the form,
+// which goes by the sizes of the whole launch.
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
 #include "sp_spikes.cuh"
@@ -89,6 +91,8 @@ constexpr int kDenseThreads = 256;
 template <int B> struct DenseShape { static constexpr int batch = 1, min_ctas = 2; };
 template <> struct DenseShape<1> { static constexpr int batch = 1, min_ctas = 4; };
 
+template <int B> constexpr uint32_t kAllRows = (1u << B) - 1u;
+
 struct DenseParams {
   int32_t count, B;
   int32_t units;                       // total over problems
@@ -96,10 +100,10 @@ struct DenseParams {
   int32_t unit_end[kDenseMaxProblems]; // prefix sums of each problem's units
 };
 
-// y of rows row0 .. row0 + nrows - 1 (nrows <= 4) of P for the B activation
-// rows, by one warp with FP32 FMAs.
+// y of rows row0 .. row0 + nrows - 1 (nrows <= 4) of P for the activation rows
+// in `rows` (bit b: row b), by one warp with FP32 FMAs.
 template <int B>
-__device__ __forceinline__ void dense_rows(const DenseProblem& P, int row0, int nrows) {
+__device__ __forceinline__ void dense_rows(const DenseProblem& P, int row0, int nrows, uint32_t rows) {
   constexpr int kDenseBatch = DenseShape<B>::batch;
   const int lane = threadIdx.x & 31;
   const int nch = (P.K + 511) / 512;        // chunk rounds of the whole warp
@@ -156,7 +160,7 @@ __device__ __forceinline__ void dense_rows(const DenseProblem& P, int row0, int 
   for (int r = 0; r < kDenseRows; ++r)
 #pragma unroll
     for (int b = 0; b < B; ++b)
-      if (lane == r * B + b && r < nrows)
+      if (lane == r * B + b && r < nrows && (rows >> b & 1u))
         P.y[(int64_t)b * P.ldy + row0 + r] = __fmul_rn(__ldg(P.scale + row0 + r), acc[r][b]);
 }
 
@@ -171,7 +175,7 @@ dense_kernel(const __grid_constant__ DenseParams p) {
     while (u >= p.unit_end[j]) ++j;
     const DenseProblem& P = p.prob[j];
     const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kDenseRows;
-    dense_rows<B>(P, row0, min(kDenseRows, P.N - row0));
+    dense_rows<B>(P, row0, min(kDenseRows, P.N - row0), kAllRows<B>);
   }
 }
 
@@ -260,11 +264,11 @@ struct DenseMmaParams {
   int64_t cost_end[kDenseMaxProblems]; // prefix sums of each problem's chunks
 };
 
-// The rows of one unit of the tensor-core form with FP32 FMAs.
+// One unit of the tensor-core form with FP32 FMAs, for some activation rows.
 template <int B>
-__device__ __forceinline__ void dense_unit_fma(const DenseProblem& P, int row0) {
+__device__ __forceinline__ void dense_unit_fma(const DenseProblem& P, int row0, uint32_t rows) {
   for (int r = row0; r < row0 + kMmaRows && r < P.N; r += kDenseRows)
-    dense_rows<B>(P, r, min(kDenseRows, P.N - r));
+    dense_rows<B>(P, r, min(kDenseRows, P.N - r), rows);
 }
 
 template <int B>
@@ -273,7 +277,7 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
   constexpr int NT = (B + 1) / 2;      // 8-column MMA tiles: two activation rows each
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t* s_tab = smem + kMmaRingBytes;
-  __shared__ uint8_t s_fma[kDenseMaxProblems];   // problem j0 + i: an activation does not split exactly
+  __shared__ uint32_t s_fma[kDenseMaxProblems];  // problem j0 + i: activation rows that do not split exactly
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -329,7 +333,7 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
     auto open_unit = [&]() {
       while (lu < u1) {                  // the next unit of this warp that runs here
         while (lu >= p.unit_end[lj]) ++lj;
-        if (!any_fma || !s_fma[lj - j0]) break;
+        if (!any_fma || s_fma[lj - j0] != kAllRows<B>) break;
         lu += kMmaWarps;
       }
       lc = lch = 0;
@@ -373,13 +377,13 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
         const DenseProblem& P = p.prob[j];
         if (j > j0 && P.x == p.prob[j - 1].x && P.K == p.prob[j - 1].K && P.ldx == p.prob[j - 1].ldx) continue;
         const int nch = (P.K + kMmaChunk - 1) / kMmaChunk;
-        bool exact = true;
         for (int i = threadIdx.x; i < nch * 4 * B; i += kMmaThreads) {
           const int tt = i & 3, b = (i >> 2) % B, c = (i >> 2) / B;
           float x[16];
           load_x16(P.x + (int64_t)b * P.ldx, c * kMmaChunk + 16 * tt, P.K, x);
           uint4* dst = reinterpret_cast<uint4*>(s_tab + base + (c * NT + (b >> 1)) * kMmaTile) +
                        (b & 1) * 16 + tt;
+          bool exact = true;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             // MMAs 2 h and 2 h + 1 of the chunk: columns (0, 2), (1, 3) of each
@@ -396,18 +400,20 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
             for (int s = 0; s < 3; ++s)
               dst[32 * h + 4 * s] = make_uint4(o[0][s], o[1][s], o[2][s], o[3][s]);
           }
-        }
-        if (!exact) {
-          bad = 1;
-          s_fma[j - j0] = 1;
+          if (!exact) {
+            bad = 1;
+            atomicOr(&s_fma[j - j0], 1u << b);
+          }
         }
         base += nch * NT * kMmaTile;
       }
     }
     any_fma = __syncthreads_or(bad) != 0;
     if (any_fma) {
-      // rare: those problems (and the ones that share their activations) with
-      // FP32 FMAs; the loops below leave them out
+      // rare: those activation rows (of each problem that shares them) with
+      // FP32 FMAs; the loops below do not write them, and leave out a problem
+      // of none but such rows.  (A row's products stay in its own columns of
+      // the MMA: what they are does not reach the other rows.)
       if (threadIdx.x == 0)
         for (int j = j0 + 1; j < j1; ++j)
           if (p.prob[j].x == p.prob[j - 1].x && p.prob[j].K == p.prob[j - 1].K && p.prob[j].ldx == p.prob[j - 1].ldx)
@@ -416,7 +422,7 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
       for (int u = u0 + warp, j = j0; u < u1; u += kMmaWarps) {
         while (u >= p.unit_end[j]) ++j;
         const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kMmaRows;
-        if (s_fma[j - j0]) dense_unit_fma<B>(p.prob[j], row0);
+        if (s_fma[j - j0]) dense_unit_fma<B>(p.prob[j], row0, s_fma[j - j0]);
       }
       // the ring again, without them
       cp_async_wait<0>();
@@ -437,7 +443,8 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
         }
         ++j;
       }
-      if (any_fma && s_fma[j - j0]) continue;
+      const uint32_t skip = any_fma ? s_fma[j - j0] : 0u;
+      if (skip == kAllRows<B>) continue;
       const DenseProblem& P = p.prob[j];
       const int row0 = (u - (j ? p.unit_end[j - 1] : 0)) * kMmaRows;
       const int nch = (P.K + kMmaChunk - 1) / kMmaChunk;
@@ -495,7 +502,7 @@ dense_mma_kernel(const __grid_constant__ DenseMmaParams p) {
           const float lo = __shfl_xor_sync(0xffffffffu, a0, 1);
           const float sum = __fadd_rn(a0, __fadd_rn(a1, lo));
           const int b = 2 * n + (t >> 1), row = row0 + g + 8 * e;
-          if ((t & 1) == 0 && b < B && row < P.N)
+          if ((t & 1) == 0 && b < B && row < P.N && !(skip >> b & 1u))
             P.y[(int64_t)b * P.ldy + row] = __fmul_rn(__ldg(P.scale + row), sum);
         }
     }

@@ -300,3 +300,37 @@ def test_dense_tensor_form_one_large_product(B, K, N):
             err = np.abs(got - want)
             worst = (err / tensor_bound(K, 1.0, np.abs(prod).sum(-1), want)).max()
             assert worst <= 1, f"K={K} B={B} position {p0} small {small}: {worst:.2f} of the bound"
+
+
+@pytest.mark.parametrize("B", [2, 4])
+def test_dense_rows_do_not_meet(B):
+    """A row's bits depend on its own activations: another row that holds an
+    infinity, a NaN or a value that three bf16 parts cannot hold leaves it as
+    it is, and the row itself follows IEEE arithmetic."""
+    N0, K0 = BIG if B <= 2 else BIG4
+    W, x, s, ldw, ldx = case(400, N0, K0, B)
+    W2, x2, s2, ldw2, ldx2 = case(401, 333, 700, B)
+    Wd, sd, Wd2, sd2 = to_dev(W), to_dev(s), to_dev(W2), to_dev(s2)
+
+    def call(x, x2):
+        y, y2 = torch.full((B, N0), 7.0, device=DEV), torch.full((B, 333), 7.0, device=DEV)
+        sp.spike_proj_dense([(Wd, ldw, sd, to_dev(x), ldx, y, N0, N0, K0),
+                             (Wd2, ldw2, sd2, to_dev(x2), ldx2, y2, 333, 333, 700)], B)
+        return y.cpu().numpy(), y2.cpu().numpy()
+
+    base, base2 = call(x, x2)
+    for v in (float("inf"), float("nan"), 1e-40, 1e38):
+        for bad in range(B):
+            xv, xv2 = x.copy(), x2.copy()
+            xv[bad, 77], xv2[bad, 13] = v, v
+            got, got2 = call(xv, xv2)
+            for b in range(B):
+                if b != bad:
+                    assert np.array_equal(got[b], base[b]) and np.array_equal(got2[b], base2[b]), (v, bad, b)
+            with np.errstate(invalid="ignore", over="ignore"):
+                want = (xv2[bad, :700].astype(np.float64) * W2[:, :700]).sum(-1) * s2
+            if v != v:
+                assert np.isnan(got2[bad]).all()
+            elif abs(v) < 1:
+                mag = (np.abs(xv2[bad, :700]).astype(np.float64) * np.abs(W2[:, :700])).sum(-1)
+                assert np.all(np.abs(got2[bad] - want) <= tree_bound(700, s2.astype(np.float64), mag, want))
