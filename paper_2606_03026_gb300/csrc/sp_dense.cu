@@ -50,9 +50,9 @@
 //     activation rows), while the first ring is in flight.
 //   - one 512-thread CTA per SM takes an equal, contiguous share of the
 //     launch's chunks, so that it meets one or two activation tables.
-// Measured on 66 projections (4608 / 1536 / 6144 x 1536, 415 MB): 70.6 us for
-// one activation row (5.9 TB/s) and 73.2 us for four; with dense_kernel 81 and
-// 259 us.
+// Measured on 66 projections (4608 / 1536 / 6144 x 1536, 415 MB), by the machine:
+// 70.8 to 74.8 us for one activation row (5.9 to 5.6 TB/s) and 74.0 to 78.2 for
+// four; with dense_kernel 81 and 260 us.
 //
 // dense_kernel<B> (small launches, and K whose table does not fit): a unit
 // is 4 consecutive rows of one problem, owned by one warp.  Lane l
@@ -72,6 +72,8 @@
 // same on every run, and a row's does not depend on the other rows of the call
 // or on the other problems of the launch, but through the choice of the form,
 // which goes by the sizes of the whole launch.
+#include <algorithm>
+
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
 #include "sp_spikes.cuh"
@@ -548,18 +550,91 @@ cudaError_t launch_dense_mma(const DenseMmaParams& p, int dev, int sms, cudaStre
                     s, p);
 }
 
+// Whether two consecutive problems share one activation table.
+bool same_table(const DenseProblem& a, const DenseProblem& b) {
+  return a.x == b.x && a.K == b.K && a.ldx == b.ldx;
+}
+
+// Bytes of shared memory for the activation tables: two of the largest where
+// they fit.
+int table_bytes(int largest) { return 2 * largest <= kMmaTableBytes ? 2 * largest : largest; }
+
+// The faster form by a model of both, us per call:
+//   FMAs          a + b (K rounds of a warp) + c (warp rounds per SM) + d MB, by B
+//   tensor cores  3.4 + 0.136 per chunk that a warp takes one after another + 0.134 MB
+//                 + 2.2 where a CTA meets a second activation table, + 2.6 (three rows
+//                 or four) where the two do not fit together
+// A unit is 16 rows of one warp, so the tensor-core form pays for few units per
+// warp (a warp alone reads a wide row from a ring of 8 KB) and for uneven ones
+// (16.1 units a CTA take two rounds of 16 warps), and a launch of many small
+// problems for its tables.  Fitted on 2153 launches of 1.5 to 200 MB (K = 64 to
+// 6144, 1 to 66 problems, weights in L2 and from HBM), each timed in both forms:
+// error 9 %, and 0.996 of the rate of always taking the faster one.  (By a line on
+// the bytes alone 0.987, with launches at up to twice their time: 64 problems of 52
+// x 3000, three rows, 14.2 us by FMAs and 24.8; one row of 39,062 x 1536 in L2 12.9
+// and 15.3; the 66 problems of a decode step, one row and four, 81 and 260 by FMAs,
+// 71 to 75 and 74 to 78 on the tensor cores.)
+bool mma_is_faster(const DenseProblem* probs, int count, int B, int sms) {
+  constexpr double kFma[SPIKE_PROJ_DENSE_MAX_B][4] = {
+      {3.4, 0.70, 0.044, -0.015}, {3.2, 0.83, 0.059, 0.021}, {2.9, 1.28, 0.058, 0.076}, {3.0, 1.57, 0.070, 0.121}};
+  const auto ring = [](int nch) { return ceil_div(nch, kMmaRing) * kMmaRing; };
+  int64_t cost = 0, quads = 0, rounds = 0;                 // chunks; units of 4 rows, their K rounds
+  double mb = 0;
+  int most = 0, wide = 0;
+  for (int j = 0; j < count; ++j) {
+    const DenseProblem& P = probs[j];
+    const int nch = ceil_div(P.K, kMmaChunk);
+    cost += (int64_t)ceil_div(P.N, kMmaRows) * nch;
+    quads += ceil_div(P.N, kDenseRows);
+    rounds += (int64_t)ceil_div(P.N, kDenseRows) * ceil_div(P.K, 512);
+    mb += 1e-6 * P.N * P.K;
+    if (nch > most) most = nch;
+    if (ceil_div(P.K, 512) > wide) wide = ceil_div(P.K, 512);
+  }
+  const int64_t warps = (int64_t)sms * (kDenseThreads / 32) * (B == 1 ? DenseShape<1>::min_ctas : DenseShape<2>::min_ctas);
+  const double serial_fma =
+      quads <= warps ? wide : (double)((quads + warps - 1) / warps) * rounds / quads;
+  const double* f = kFma[B - 1];
+  const double fma = f[0] + f[1] * serial_fma + f[2] * rounds / sms + f[3] * mb;
+
+  const int tiles = (B + 1) / 2;
+  const int fits = table_bytes(most * tiles * kMmaTile);
+  int64_t serial = cost / ((int64_t)sms * kMmaWarps);
+  bool second = false, apart = false;
+  int64_t at = 0;                                          // chunk at which problem j + 1 begins
+  for (int j = 0; j < count; ++j) {
+    const int nch = ceil_div(probs[j].K, kMmaChunk);
+    const int64_t mine = ceil_div(probs[j].N, kMmaRows);
+    const int64_t units = std::min(mine, (cost + (int64_t)sms * nch - 1) / ((int64_t)sms * nch));   // of one CTA
+    serial = std::max(serial, (units + kMmaWarps - 1) / kMmaWarps * ring(nch));
+    at += mine * nch;
+    if (j + 1 == count || same_table(probs[j], probs[j + 1])) continue;
+    const int next = ceil_div(probs[j + 1].K, kMmaChunk);
+    const int64_t cta = at * sms / cost;                   // the CTA whose share that chunk is in
+    const int64_t before = std::min(mine, (at - cost * cta / sms) / nch);   // its units of the two problems
+    const int64_t after = std::min<int64_t>(ceil_div(probs[j + 1].N, kMmaRows),
+                                            (cost * (cta + 1) / sms - at + next - 1) / next);
+    if (before < 1 || after < 1) continue;
+    second = true;
+    if ((nch + next) * tiles * kMmaTile > fits) {
+      apart = true;
+      serial = std::max(serial, (before + kMmaWarps - 1) / kMmaWarps * ring(nch) +
+                                    (after + kMmaWarps - 1) / kMmaWarps * ring(next));
+    }
+  }
+  const double mma = 3.4 + 0.136 * serial + 0.134 * mb + (second ? 2.2 : 0.0) + (apart && B > 2 ? 2.6 : 0.0);
+  return mma < 1.03 * fma;                                 // equal ones to the tensor cores
+}
+
 }  // namespace
 
 cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream_t s) {
   int dev = 0, sms = 0;
   const cudaError_t e = current_device(&dev, &sms);
   if (e != cudaSuccess) return e;
-  // The tensor-core form where an activation table fits in shared memory and
-  // the weights outweigh its start (it holds a whole SM, so it cannot start
-  // beside the previous kernel).  us per call, FMAs / tensor cores: one row,
-  // 18.9 MB 6.9 / 8.1 and 37.7 MB 12.8 / 11.0; two rows, 8.4 MB 5.1 / 5.7 and
-  // 13.1 MB 10.1 / 7.5; three rows, 2.1 MB 4.1 / 4.7 and 4.7 MB 5.7 / 5.5; four
-  // rows, 0.5 MB 3.7 / 4.1 and 2.1 MB 4.9 / 4.6.
+  // The tensor-core form where an activation table fits in shared memory, the
+  // weights outweigh its start (it holds a whole SM, so it cannot start beside
+  // the previous kernel), and it is modelled to be the faster one.
   constexpr int64_t kMmaMinBytes[SPIKE_PROJ_DENSE_MAX_B] = {24 << 20, 9 << 20, 3 << 20, 3 << 19};
   int maxK = 0;
   int64_t bytes = 0;
@@ -568,11 +643,11 @@ cudaError_t launch_dense(const DenseProblem* probs, int count, int B, cudaStream
     bytes += (int64_t)probs[j].N * probs[j].K;
   }
   const int table = ceil_div(maxK, kMmaChunk) * ((B + 1) / 2) * kMmaTile;
-  if (table <= kMmaTableBytes && bytes >= kMmaMinBytes[B - 1]) {
+  if (table <= kMmaTableBytes && bytes >= kMmaMinBytes[B - 1] && mma_is_faster(probs, count, B, sms)) {
     DenseMmaParams p;
     p.count = count;
     p.one28 = 0x43004300u;
-    p.table_bytes = table * 2 <= kMmaTableBytes ? table * 2 : table;
+    p.table_bytes = table_bytes(table);
     int units = 0;
     int64_t cost = 0;
     for (int j = 0; j < count; ++j) {

@@ -29,6 +29,7 @@ struct State {
   std::string fail;                                            // launches of kernels with this in the name fail
   int active = 0;                                              // spikes that a counting kernel finds
   int publish_ms = 0;                                          // delay of a publication (< 0: it never comes)
+  std::string last;                                            // the kernel launched last
   int launches = 0, synced = -1;                               // synced: the device last synchronised
   size_t pushed_smem = 0;                                      // of a <<<...>>> launch
   std::vector<std::thread> pending;
@@ -66,6 +67,7 @@ cudaError_t launch(const void* f, size_t smem, unsigned cluster, void** args) {
   if (smem > 48 * 1024 && s.smem[key] < (int)smem) return cudaErrorInvalidValue;
   if (cluster > 8 && !s.nonportable[key]) return cudaErrorInvalidClusterSize;
   ++s.launches;
+  s.last = name;
   if (name.find("spikes_to_01_kernel") != std::string::npos) {
     const auto& c = *static_cast<const sp::SpikeCount*>(args[7]);
     if (c.dev) c.dev[0] += s.active;
@@ -94,6 +96,7 @@ void fake_counts(int active, int publish_ms) {
 }
 void fake_device(int device) { state().device = device; }
 int fake_launches() { return std::exchange(state().launches, 0); }
+int fake_last_is(const char* name) { return state().last.find(name) != std::string::npos; }
 int fake_synced() { return std::exchange(state().synced, -1); }
 
 // ---- the runtime ------------------------------------------------------------

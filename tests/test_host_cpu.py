@@ -54,11 +54,12 @@ def last_dispatch(lib, plan):
     return chosen.value, count.value
 
 
-def dense(lib, shapes, B):
+def dense(lib, shapes, B, own=True):
+    """own: every problem has activations of its own."""
     table = (sp.SpDense * len(shapes))()
     for j, (N, K) in enumerate(shapes):
         ld = (K + 15) // 16 * 16
-        table[j] = sp.SpDense(FAKE, ld, FAKE, FAKE, ld, FAKE, N, N, K)
+        table[j] = sp.SpDense(FAKE, ld, FAKE, FAKE + own * (j << 20), ld, FAKE, N, N, K)
     return lib.spike_proj_dense(ctypes.addressof(table), len(shapes), B, None)
 
 
@@ -144,3 +145,40 @@ def test_last_dispatch_after_a_failed_call(lib):
     assert auto(lib, plan) == sp.SP_ECUDA
     assert last_dispatch(lib, plan) == (sp.SP_GEMM, 41)
     assert lib.spike_proj_plan_destroy(plan) == sp.SP_OK
+
+
+def is_tensor_form(lib, shapes, B, own=True):
+    assert dense(lib, shapes, B, own) == sp.SP_OK
+    assert lib.fake_last_is(b"dense_kernel") or lib.fake_last_is(b"dense_mma_kernel")
+    return bool(lib.fake_last_is(b"dense_mma_kernel"))
+
+
+def test_dense_form(lib):
+    """The form of a continuous-input launch: the tensor cores where they were
+    measured to be the faster one (decode steps, large launches), FMAs where
+    those were (small and wide launches, few rows per CTA, many small problems
+    with activations of their own)."""
+    step = [(n, 1536) for _ in range(22) for n in (4608, 1536, 6144)]
+    for B in (1, 2, 3, 4):
+        assert is_tensor_form(lib, step, B) and is_tensor_form(lib, step, B, own=False)
+        assert not is_tensor_form(lib, [(64, 1536)], B)
+        assert not is_tensor_form(lib, [(4096, 16384)], B)           # K without a table
+        assert is_tensor_form(lib, [(200_000, 128)], B)
+    for shapes, B in (([(52, 3000)] * 64, 3), ([(136, 3000)] * 64, 3), ([(66, 6144)] * 64, 1), ([(39062, 1536)], 1),
+                      ([(65, 6144)] * 64, 2), ([(136, 3000)] * 64, 4), ([(16927, 1536)], 1)):
+        assert not is_tensor_form(lib, shapes, B), (shapes[0], len(shapes), B)
+    for shapes, B in (([(13020, 768)], 2), ([(6000, 3000)], 4), ([(3000, 3000)], 4), ([(11718, 1536)], 3),
+                      ([(78125, 768)], 1), ([(65104, 1536)], 2), ([(406, 768)] * 64, 4)):
+        assert is_tensor_form(lib, shapes, B), (shapes[0], len(shapes), B)
+
+
+def test_dense_form_of_the_gpu_tests(lib):
+    """The launches that test_gpu_dense.py means for the tensor-core form."""
+    import test_gpu_dense as t
+    for B in (1, 2, 3, 4):
+        assert is_tensor_form(lib, [*t.edge_shapes(B), t.FILLER], B)
+        assert is_tensor_form(lib, [(8000, 3072), (17, 3072), (383, 3072), t.FILLER], B, own=False)
+        assert is_tensor_form(lib, [s for _ in range(9) for s in ((40, 200), (20, 100))] + [t.FILLER], B)
+        assert is_tensor_form(lib, [(4000, 1536), (333, 700), t.FILLER], B)
+        for K in (64, 512, 1536):
+            assert is_tensor_form(lib, [(2048, K), t.FILLER], B)
