@@ -372,8 +372,7 @@ gather_kernel(const __grid_constant__ GatherParamsT<NP> p) {
 constexpr int kClusterLoads = 9;                   // column loads per lane in registers (64 registers)
 // and in shared memory (S): 8 for a group of projections (4 CTAs per SM), 16
 // for a single projection's clusters of 12 or 16 (fewer CTAs, each with more
-// columns) and for the rows of a batch (rates up to 0.2: a warp's share of a
-// chunk of 1024 columns then still loads in one round)
+// columns) and for some batches of rows (rows_even below)
 template <int S>
 using ClusterSmem = UnitSmem<kGatherClusterWarps, kGatherClusterMaxCK, S>;
 
@@ -539,19 +538,26 @@ int capacity_for(int dev, bool lif, int CL, int S) {
   }
 }
 
-// The rows of a batch leave most SMs idle with clusters of 6, and at spike
-// rates up to 0.2 a warp's share of a chunk of 1024 columns takes two rounds
-// of loads with 8 shared-memory slots.  So a few rows (at most kSpreadMaxCtas
-// CTAs) take clusters of 12 with chunks of at least 384 columns, and more (at
-// most kRowsMaxCtas CTAs) clusters of 6 with 16 slots.  us a call at 1536 x 6144,
-// rates U(0.05, 0.2) / all 0.05, before and after: 2 rows 4.3 / 3.2 -> 3.6 /
-// 3.2, 4 rows 4.9 / 3.4 -> 4.6 / 3.35, 8 rows 6.0 / 3.8 -> 5.65 / 3.6, 12 rows
-// 7.9 / 4.9 -> 6.3 / 3.9.  Past the lines the other side is faster: 8 rows in
-// clusters of 12 take 5.2 but 4.3 at 0.05, 16 rows with 16 slots 7.3 against
-// 7.2.  The projections of a decode step keep clusters of 6 with 8 slots: at a
-// rate of 0.1 one round suffices (2 blocks: 3.8, in clusters of 16 4.05).
+// The rows of a batch leave most SMs idle with clusters of 6: a few rows (at
+// most kSpreadMaxCtas CTAs) take clusters of 12 with chunks of at least 384
+// columns.  Launches of about 1.5 CTAs per SM, and of 2 to 3 (rows_even),
+// take clusters of 6 with 16 slots: of these only three CTAs fit an SM, not
+// four, and so the clusters spread more evenly (the gain is the same at a rate
+// of 0.05, where the slots stay empty).  Time against clusters
+// of 6 with 8 slots, geometric means over 6 widths, 7 Ks and 2 to 48 rows, at
+// uniform rates 0.05 / 0.1 / 0.15 / 0.2 and rows of mixed rates U(0.05, 0.2):
+//   clusters of 12, CTAs <= 72     0.98 / 0.92 / 0.84 / 0.82, mixed 0.84
+//                   73 .. 120      1.08 / 1.00 / 0.91 / 0.90, mixed 0.89
+//                   121 .. 304     1.12 / 1.01 / 0.90 / 0.88, mixed 0.91 (not taken: low rates lose)
+//   16 slots, CTAs  <= 192         1.00 / 1.02 / 0.97 / 1.05, mixed 0.99 (not taken: 0.85 to 1.22)
+//                   216            0.85 / 0.84 / 0.79 / 0.84, mixed 0.84
+//                   288            0.93 / 0.97 / 0.92 / 1.02, mixed 0.97 (not taken: up to 1.22 at 0.2)
+//                   384, 432       0.86 / 0.90 / 0.83 / 0.93, mixed 0.88
+//                   576            1.00 (four CTAs per SM would not fit: 8 slots)
+// The projections of a decode step keep clusters of 6 with 8 slots (2 blocks:
+// 3.8 us, in clusters of 16 4.05).
 constexpr int kSpreadMaxCtas = 120;
-constexpr int kRowsMaxCtas = 228;
+constexpr bool rows_even(int ctas) { return (ctas >= 200 && ctas <= 256) || (ctas > 304 && ctas <= 456); }
 
 // Sets the chunking of a batch's rows for clusters of 12; false when they take
 // clusters of 6.
@@ -645,7 +651,7 @@ bool cluster_form(GatherParamsT<NP>& q, int dev, int* grid_x, int* grid_y, int* 
     if (q.prob[j].ncl > widest) widest = q.prob[j].ncl;
   }
   int S = CL > 8 ? 16 : 8;
-  if (rows && CL == 6 && total * CL <= kRowsMaxCtas && total <= capacity_for<NP>(dev, false, 6, 16)) S = 16;
+  if (rows && CL == 6 && rows_even(total * CL) && total <= capacity_for<NP>(dev, false, 6, 16)) S = 16;
   if (total > capacity_for<NP>(dev, q.lif_I != nullptr, CL, S)) return false;
   q.ncl_list = 0;
   if (NP > 1 && total <= kGatherMaxClusterList && widest <= 0xff) {
