@@ -384,9 +384,14 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
     } else {
       // Byte rows: one 16-byte copy per lane and K block, in kSmPhases commit
       // groups of blocks; a phase is folded (U8) and published as soon as its
-      // own copies have landed.
+      // own copies have landed.  With few rows several warps share the eight
+      // rows of one and take every share-th block (one warp per eight rows,
+      // as with 64, left six of eight idle at 16 rows: 2 byte rows of 300
+      // columns 4.4 -> 5.3 us).
       const int rr = lane >> 2, j = lane & 3;
-      const int r = 8 * e + rr;
+      const int share = TN == 16 ? 4 : TN == 32 ? 2 : 1;
+      const int skip = TN == 16 ? e >> 1 : TN == 32 ? e >> 2 : 8 * e < TN ? 0 : kGemmSmallMaxKB;   // (48: two have none)
+      const int r = 8 * (TN == 16 ? e & 1 : TN == 32 ? e & 3 : e) + rr;
       const uint8_t* row = r < a.T ? static_cast<const uint8_t*>(spike_row(a.spikes, a.fmt, r, a.ld)) : nullptr;
       uint8_t* slot = sX + r * 64 + ((j ^ ((r >> 1) & 3)) << 4);
       const auto copied = [&](int b, const uint8_t*& src) {   // block b of this lane goes by cp.async
@@ -397,7 +402,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
 #pragma unroll 1
       for (int ph = 0; ph < kSmPhases; ++ph) {
 #pragma unroll 1
-        for (int b = 4 * ph; b < min(nk, 4 * ph + 4) && r < TN; ++b) {
+        for (int b = 4 * ph + skip; b < min(nk, 4 * ph + 4); b += share) {
           const uint8_t* src;
           if (copied(b, src))
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + b * kSmXBlock)), "l"(src)
@@ -410,13 +415,14 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap mapW, const __grid_constan
       }
 #pragma unroll
       for (int ph = 0; ph < kSmPhases; ++ph) {
+        if (4 * ph >= nk) break;             // no fence and no barrier for phases without blocks
         if (ph == 0) asm volatile("cp.async.wait_group 3;" ::: "memory");
         else if (ph == 1) asm volatile("cp.async.wait_group 2;" ::: "memory");
         else if (ph == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
         else asm volatile("cp.async.wait_group 0;" ::: "memory");
         if (a.fmt == SP_SPIKES_U8) {         // any nonzero byte -> 1 (this lane's copies)
 #pragma unroll 1
-          for (int b = 4 * ph; b < min(nk, 4 * ph + 4) && r < TN; ++b) {
+          for (int b = 4 * ph + skip; b < min(nk, 4 * ph + 4); b += share) {
             const uint8_t* src;
             if (copied(b, src)) {
               uint4* p = reinterpret_cast<uint4*>(slot + b * kSmXBlock);

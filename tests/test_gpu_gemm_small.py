@@ -105,3 +105,26 @@ def test_one_hot_rows(down):
     acc, y = run(plan, to_dev(X), "u8", len(ks), 6144, 1536)
     want = np.stack([Qc[k].astype(np.int32) for k in ks])
     assert np.array_equal(acc.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("T", [8, 16, 32, 48, 64])
+@pytest.mark.parametrize("K", [60, 300, 1000, 2500, 4160, 8192])
+def test_byte_rows_shared_out(T, K):
+    """Byte rows over the ways their staging is shared out (4, 2 or 1 warps per
+    eight rows, 1 to 16 K blocks per CTA, whole and partial phases of them), at
+    an aligned and an odd row stride."""
+    N = 144
+    Qc, s, X = synth.random_case(340 + T, N, K, T=T, p=0.3)
+    plan = sp.Plan(to_dev(Qc), to_dev(s), N, K, ldw=Qc.shape[1], max_batch=T, gemm=True)
+    want_acc, want_y = oracle.project(Qc, s, N, K, X, "u8", ldq=Qc.shape[1])
+    for fmt, scale in (("u8", 7), ("bool8", 1)):
+        for ld in ((K + 15) // 16 * 16, K + 1 - K % 2):
+            rows = np.zeros((T, ld), np.uint8)
+            rows[:, :K] = X * scale
+            xd = to_dev(rows)
+            acc = torch.full((T, N), -7, dtype=torch.int32, device=DEV)
+            y = torch.full((T, N), -7.0, device=DEV)
+            plan.batched(xd, fmt, T, ld, acc, y, "gemm")
+            assert_parity(acc, y, want_acc, want_y, f"{fmt} ld {ld}")
+    assert plan.status() == sp.SP_OK
+    plan.close()
