@@ -31,9 +31,9 @@
 //               thread; tcgen05.commit frees ring slots and publishes
 //               accumulators
 //   warps 2-9   epilogue: warp w reads TMEM lane quarter w % 4 (32 rows);
-//               with K whole, warps 2-5 write 16-column blocks; with K split,
-//               warps 2-5 and 6-9 take alternate chunks of the partial and
-//               the two 16-column halves of every owned chunk
+//               with K whole, warps 2-5 and 6-9 write alternate 16-column
+//               blocks; with K split, they take alternate chunks of the
+//               partial and the two 16-column halves of every owned chunk
 // Whole K (enough output tiles for every SM): one CTA per SM, persistent over
 // 128 x 256 tiles; the epilogue of one tile overlaps the next tile's MMAs
 // (double-buffered accumulator) and writes acc / y through a shared-memory
@@ -212,7 +212,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], 4);          // one arrive per epilogue warp
+      mbar_init(&tempty[b], 8);          // one arrive per epilogue warp
     }
     mbar_init(done, 1);
     for (int j = 0; j < kMaxOwned; ++j) mbar_init(&pfull[j], 1);
@@ -340,39 +340,38 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
     }
   } else if (a.splits == 1) {
     publish();
-    if (warp < 6) {                           // the whole-K epilogue uses warps 2-5
-      // ------------------------------ epilogue (whole K) ------------------------
-      // Each warp owns one 32-row quarter of the tile (its TMEM lane quarter) and
-      // works alone: no barrier joins the epilogue warps, so a warp that gives up
-      // on a timed-out wait cannot strand the others.
-      const int q = warp & 3;
-      uint32_t* tr = s_tr + (size_t)(warp - 2) * 32 * TR16_STRIDE;
-      int ab = 0;
-      uint32_t aph = 0;
-      for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
-        int tile, mb, nb, kb0, kb1;
-        unit_coords(a, u, tile, mb, nb, kb0, kb1);
-        if (!mbar_wait(&tfull[ab], aph, lim)) {
-          *s_abort = 1;
-          if (lane == 0) atomicExch(a.p.err, kErrMbarTimeout);
-          break;
-        }
-        tc_fence_after();
-        const int row0 = mb * BM + q * 32;
-        for (int c = 0; c < BN; c += 16) {
-          uint32_t v[16];
-          tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + c), v);
-          if (a.p.fault == kFaultAbort) {    // test fault: the output stays unwritten
-            if (lane == 0) atomicExch(a.p.err, kErrInjected);
-            continue;
-          }
-          store_block16(a.p, tr, v, row0, nb * BN + c, column_scale(a.p, nb * BN + c + (lane & 15)));
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[ab]);
-        if (++ab == 2) { ab = 0; aph ^= 1u; }
+    // ------------------------------ epilogue (whole K) --------------------------
+    // Each warp owns one 32-row quarter of the tile (its TMEM lane quarter),
+    // every other 16-column block of it, and works alone: no barrier joins the
+    // epilogue warps, so a warp that gives up on a timed-out wait cannot strand
+    // the others.
+    const int q = warp & 3;
+    uint32_t* tr = s_tr + (size_t)(warp - 2) * 32 * TR16_STRIDE;
+    int ab = 0;
+    uint32_t aph = 0;
+    for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+      int tile, mb, nb, kb0, kb1;
+      unit_coords(a, u, tile, mb, nb, kb0, kb1);
+      if (!mbar_wait(&tfull[ab], aph, lim)) {
+        *s_abort = 1;
+        if (lane == 0) atomicExch(a.p.err, kErrMbarTimeout);
+        break;
       }
+      tc_fence_after();
+      const int row0 = mb * BM + q * 32;
+      for (int c = 16 * ((warp - 2) >> 2); c < BN; c += 32) {
+        uint32_t v[16];
+        tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + c), v);
+        if (a.p.fault == kFaultAbort) {      // test fault: the output stays unwritten
+          if (lane == 0) atomicExch(a.p.err, kErrInjected);
+          continue;
+        }
+        store_block16(a.p, tr, v, row0, nb * BN + c, column_scale(a.p, nb * BN + c + (lane & 15)));
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[ab]);
+      if (++ab == 2) { ab = 0; aph ^= 1u; }
     }
   } else {
     // ---------------- epilogue (split K): reduce-scatter through L2 -----------
