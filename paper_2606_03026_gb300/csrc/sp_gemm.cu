@@ -933,9 +933,12 @@ __device__ __forceinline__ bool bytes16_to_01(const uint8_t* x, const uint8_t* l
 // 16-byte aligned (base and leading dimension), so whole 16-column groups
 // load as one vector; other byte rows load the aligned words around a group
 // (single bytes only at the ends of the matrix and of a row).  The spikes are
-// counted on the way when a count is asked for: SP_AUTO then needs no pass of
-// its own over them.
-template <bool kVec>
+// counted on the way when a count is asked for (kCount): SP_AUTO then needs no
+// pass of its own over them.  (Without a count no block holds shared memory: a
+// GEMM CTA that starts early leaves room for five such blocks on its SM, for
+// four with it.  2048 rows of 6144 bytes: the pass costs 5.5 us of the call, 6.8
+// with the counting code in it.)
+template <bool kVec, bool kCount>
 __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, int64_t ld, int T,
                                     int K, int Kp, uint8_t* __restrict__ Xs, SpikeCount count) {
   pdl_launch_dependents();
@@ -977,10 +980,10 @@ __global__ void spikes_to_01_kernel(const void* __restrict__ spikes, int fmt, in
       }
     }
     // (the bytes are 0 / 1: adding the words keeps byte sums below 5)
-    active += (int)(((o.x + o.y + o.z + o.w) * 0x01010101u) >> 24);
+    if (kCount) active += (int)(((o.x + o.y + o.z + o.w) * 0x01010101u) >> 24);
     *reinterpret_cast<uint4*>(Xs + (int64_t)t * Kp + k) = o;
   }
-  if (count.dev) count_spikes(active, count, false);
+  if (kCount) count_spikes(active, count, false);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
@@ -1123,11 +1126,9 @@ cudaError_t launch_spikes_to_01(const void* spikes, int fmt, int64_t ld, int T, 
   if (blocks < 1) blocks = 1;
   const bool vec = fmt != SP_SPIKES_BITS32 && (reinterpret_cast<uintptr_t>(spikes) & 15u) == 0 &&
                    ld % 16 == 0;
-  if (vec)
-    return launch_pdl(spikes_to_01_kernel<true>, dim3((unsigned)blocks), dim3(threads), 0, s, spikes,
-                      fmt, ld, T, K, Kp, Xs, count);
-  return launch_pdl(spikes_to_01_kernel<false>, dim3((unsigned)blocks), dim3(threads), 0, s, spikes,
-                    fmt, ld, T, K, Kp, Xs, count);
+  const auto kernel = vec ? (count.dev ? spikes_to_01_kernel<true, true> : spikes_to_01_kernel<true, false>)
+                          : (count.dev ? spikes_to_01_kernel<false, true> : spikes_to_01_kernel<false, false>);
+  return launch_pdl(kernel, dim3((unsigned)blocks), dim3(threads), 0, s, spikes, fmt, ld, T, K, Kp, Xs, count);
 }
 
 namespace {
