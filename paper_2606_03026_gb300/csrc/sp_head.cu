@@ -50,6 +50,10 @@
 // to run beside a projection CTA: a projection CTA that had to wait for a
 // selection's SM held up the call by 7 us.
 //
+// Projection of one state beyond L2 (head_wide_kernel): there the ring's stream is
+// the slower one (5.3 TB/s at the margin, whatever its depth, its lane layout or
+// the work per chunk; the register loads 7), and the call takes register loads.
+//
 // Measured on 57,344 x 1536, back to back with three weight copies, us a call:
 // gate closed 21.5 (22.0 before this form: the weights 14 of it, the codes
 // 1.3, the selection and the two hand-offs 6), every call verified 24.3 (26.0);
@@ -73,6 +77,10 @@ constexpr size_t kHeadRingBytes = (size_t)kHeadWarps * kHeadRing * kHeadRows * k
 constexpr int kHeadLists = kHeadWarps / 2;    // lists of a projection CTA (one per pair of warps)
 constexpr int kHeadList = SPIKE_PROJ_HEAD_MAX_CAND;   // keys per list
 constexpr int kHeadMaxGrid = 160;             // projection CTAs of one call
+constexpr int kWideThreads = 1024;            // head_wide_kernel: a CTA per SM, 4 rows and a list per warp
+constexpr int kWideWarps = kWideThreads / 32;
+constexpr int kWideRows = 4;
+constexpr int64_t kWideBytes = (int64_t)110 << 20;
 constexpr int kSelThreads = 256;              // threads of a selection CTA
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelCluster = 4;                // selection CTAs of one hidden state
@@ -83,13 +91,14 @@ static_assert(kHeadList == 64, "a list is two keys per lane");
 static_assert(kHeadRingBytes + SPIKE_PROJ_HEAD_MAX_B * (SPIKE_PROJ_HEAD_MAX_K + kCodePad) <= 212 * 1024, "shared memory per CTA");
 static_assert((size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadLists * kHeadList * 8 <= kHeadRingBytes, "the lists fit the ring");
 static_assert(kHeadLists * kCtaLead == 64, "the pairs' leading keys: two per lane of one warp");
+static_assert(kWideWarps <= SPIKE_PROJ_HEAD_MAX_B * kHeadLists, "one state's lists fit the workspace");
 static_assert(kHeadMaxGrid <= kSelThreads, "one projection CTA per selection thread");
 static_assert(kHeadList == 2 * kSelWarps * kSelCluster, "two candidates per selection warp");
 
 typedef unsigned long long hkey;
 
-// Workspace: the lists (pair q of projection CTA c, hidden state b: list
-// (b * nctas + c) * kHeadLists + q), then each CTA's leading keys; all of it
+// Workspace: the lists (list q of projection CTA c, hidden state b: list
+// (b * nctas + c) * nlists + q), then each CTA's leading keys; all of it
 // is rewritten by every call.
 constexpr size_t kListBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadMaxGrid * kHeadLists * kHeadList * 8;
 constexpr size_t kLeadBytes = (size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadMaxGrid * kCtaLead * 8;
@@ -111,9 +120,10 @@ struct HeadParams {
   float* z;
   int64_t ld_z;
   int32_t B;
-  hkey* lists;             // one 64-key list per pair of projection warps and hidden state
+  hkey* lists;             // 64 keys each: one per pair of projection warps (or warp) and hidden state
   hkey* lead;              // the kCtaLead best keys of each projection CTA and hidden state
   int32_t nctas;           // CTAs of the projection kernel
+  int32_t nlists;          // lists of one of them
 };
 
 // Order-preserving bits of z (both zeros map to the bits of +0).
@@ -286,17 +296,17 @@ __device__ __forceinline__ void verify_rows2(const HeadParams& p, const float* h
   }
 }
 
-// Step 1: the CTA's warps are dealt out over the hidden states (kHeadThreads /
-// G threads each, G = B rounded up to a power of two); each group finds its
+// Step 1: the CTA's NT threads are dealt out over the hidden states (NT / G
+// each, G = B rounded up to a power of two); each group finds its
 // state's maximum |h|, and after one barrier every thread derives s_x and
 // writes codes four to a word, zero from K to Kpad.  h is read again for the
 // codes (from L1): kept in registers it made the code larger, and as the code
 // runs once per CTA its size showed (2.3 us instead of 1.3).
-template <int B, class Ring>
+template <int B, int NT, class Ring>
 __device__ __forceinline__ void head_codes(const HeadParams& p, int8_t* s_codes, float* s_red, float* s_sx,
                                            const Ring& issue_ring) {
   constexpr int G = B == 1 ? 1 : B == 2 ? 2 : 4;
-  constexpr int T = kHeadThreads / G;            // threads of one hidden state
+  constexpr int T = NT / G;                      // threads of one hidden state
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = (int)threadIdx.x / T, tt = (int)threadIdx.x % T;
   const float* hb = p.h + (int64_t)(b < B ? b : 0) * p.ldh;
@@ -424,7 +434,7 @@ head_kernel(const __grid_constant__ HeadParams p) {
   pdl_wait();
 
   // 1. activation scale and INT8 codes of each hidden state
-  head_codes<B>(p, s_codes, s_red, s_sx, [&]() {
+  head_codes<B, kHeadThreads>(p, s_codes, s_red, s_sx, [&]() {
 #pragma unroll 1
     for (int s = 0; s < kHeadRing; ++s) load();
   });
@@ -562,6 +572,90 @@ head_kernel(const __grid_constant__ HeadParams p) {
   }
 }
 
+// Steps 1-2 and the CTA's lists for one hidden state whose weights exceed what L2
+// keeps (kWideBytes): a warp owns units of 4 consecutive rows, lane l reads the
+// 16-byte chunks l, l + 32, ... of each row into registers (512 contiguous bytes
+// per instruction, 64 KB in flight per SM) and accumulates __dp4a products; every
+// warp has a list of its own.
+__global__ void __launch_bounds__(kWideThreads, 1)
+head_wide_kernel(const __grid_constant__ HeadParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  int8_t* s_codes = reinterpret_cast<int8_t*>(smem);       // [Kpad]
+  __shared__ float s_red[kWideWarps];
+  __shared__ float s_sx[1];
+  __shared__ hkey s_lead[kWideWarps * kCtaLead], s_lead2[kWideWarps];
+  static_assert(kWideWarps * kCtaLead == 256 && kWideWarps == 32, "leading keys in two steps of one warp each");
+
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wg = (int)blockIdx.x * kWideWarps + warp, nwarps = (int)gridDim.x * kWideWarps;
+  // the rows of the warp's first unit into L2 while the previous kernel ends
+  // (a prefetch hands no data to this kernel)
+  for (int r = wg * kWideRows; r < min((wg + 1) * kWideRows, p.V); ++r)
+    for (int off = lane * 128; off < p.K; off += 32 * 128)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p.W + (int64_t)r * p.ldw + off));
+  pdl_wait();
+  head_codes<1, kWideThreads>(p, s_codes, s_red, s_sx, []() {});
+
+  hkey la = 0ull, lb = 0ull, pend = 0ull;
+  int slot = 0, held = 0;                        // units since the last insert; inserts
+  const int nch = (p.K + 511) / 512;
+  for (int row0 = wg * kWideRows; row0 < p.V; row0 += nwarps * kWideRows) {
+    const int nrows = min(kWideRows, p.V - row0);
+    int acc[kWideRows] = {};
+    for (int c = 0; c < nch; ++c) {
+      const int k = 16 * (lane + 32 * c);
+      if (k >= p.K) continue;
+      // the row is ldw >= K bytes with ldw % 16 == 0: the 16 bytes at k lie
+      // inside it; bytes at or past K meet zero codes
+      uint4 w[kWideRows];
+#pragma unroll
+      for (int r = 0; r < kWideRows; ++r)
+        w[r] = r < nrows ? ld_weights16(p.W + (int64_t)(row0 + r) * p.ldw + k) : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 q = *reinterpret_cast<const uint4*>(s_codes + k);
+#pragma unroll
+      for (int r = 0; r < kWideRows; ++r) {
+        acc[r] = __dp4a((int)w[r].x, (int)q.x, acc[r]);
+        acc[r] = __dp4a((int)w[r].y, (int)q.y, acc[r]);
+        acc[r] = __dp4a((int)w[r].z, (int)q.z, acc[r]);
+        acc[r] = __dp4a((int)w[r].w, (int)q.w, acc[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kWideRows; ++r) {
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], d);
+      if (r < nrows) {
+        const float z = __fmul_rn(__ldg(p.scale + row0 + r), __fmul_rn(s_sx[0], __int2float_rn(acc[r])));
+        if (p.z && lane == r) p.z[row0 + r] = z;
+        if (lane == slot * kWideRows + r) pend = make_key(z, row0 + r);
+      }
+    }
+    if (++slot == 32 / kWideRows) {              // 32 pending keys
+      list_add32(la, lb, pend, held, lane);
+      pend = 0ull;
+      ++held;
+      slot = 0;
+    }
+  }
+  if (slot) list_add32(la, lb, pend, held, lane);
+  pdl_launch_dependents();
+  hkey* list = p.lists + ((int64_t)blockIdx.x * kWideWarps + warp) * kHeadList;
+  __stcg(list + lane, la);
+  __stcg(list + 32 + lane, lb);
+  const hkey k1 = best_of64(la, lb, lane);
+  if (lane < kCtaLead) s_lead[warp * kCtaLead + lane] = k1;
+  __syncthreads();
+  if (warp < kWideWarps * kCtaLead / 64) {
+    const hkey k2 = best_of64(s_lead[64 * warp + lane], s_lead[64 * warp + 32 + lane], lane);
+    if (lane < kCtaLead) s_lead2[warp * kCtaLead + lane] = k2;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const hkey k3 = best_of64(s_lead2[lane], 0ull, lane);
+    if (lane < kCtaLead) __stcg(p.lead + (int64_t)blockIdx.x * kCtaLead + lane, k3);
+  }
+}
+
 // Steps 3-6, a cluster of kSelCluster CTAs per hidden state.  Every CTA of
 // the cluster makes the same selection: the bound T (the 64th largest of the
 // projection CTAs' best keys, so at least 64 keys reach it), the keys >= T,
@@ -637,14 +731,14 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
     }
   }
   __syncthreads();
-  const hkey* lists = p.lists + (int64_t)b * nc * kHeadLists * kHeadList;
+  const hkey* lists = p.lists + (int64_t)b * nc * p.nlists * kHeadList;
   const int nlong = s_nlong;
   if (nlong <= kSelLong) {
     for (int j = 0; j < nlong; ++j) {
-      const hkey* L = lists + (int64_t)s_long[j] * kHeadLists * kHeadList;
-#pragma unroll
-      for (int e = 0; e < kHeadLists * kHeadList / kSelThreads; ++e) {
-        const hkey k = __ldcg(L + t + e * kSelThreads);
+      const hkey* L = lists + (int64_t)s_long[j] * p.nlists * kHeadList;
+#pragma unroll 2
+      for (int e = t; e < p.nlists * kHeadList; e += kSelThreads) {
+        const hkey k = __ldcg(L + e);
         if (k >= T) {
           const int i = atomicAdd(&s_nc, 1);
           if (i < kSelCand) s_cand[i] = k;
@@ -658,7 +752,7 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
     rank_place(s_cand, C, s_best);
   } else {
     hkey a = 0ull, c = 0ull;
-    for (int l = warp; l < nc * kHeadLists; l += kSelWarps) {
+    for (int l = warp; l < nc * p.nlists; l += kSelWarps) {
       const hkey* L = lists + (int64_t)l * kHeadList;
       hkey la = __ldcg(L + lane), lb = __ldcg(L + 32 + lane);
       sort64(la, lb, lane);                      // (lists of up to 64 keys are as they came)
@@ -756,7 +850,19 @@ cudaError_t launch_head_t(HeadParams p, int dev, int sms, cudaStream_t s) {
   if (grid > p.units) grid = p.units;
   if (grid > kHeadMaxGrid) grid = kHeadMaxGrid;
   p.nctas = grid;
-  e = launch_pdl(head_kernel<B>, dim3((unsigned)grid), dim3(kHeadThreads), smem, s, p);
+  p.nlists = kHeadLists;
+  // One state whose weights exceed what L2 keeps streams faster into registers,
+  // given two rounds of units for every warp.  us a call, ring / registers, gate
+  // closed: 57,344 x 2048 28.0 / 24.5, 57,344 x 4096 50.9 / 41.0, 150,000 x 1536
+  // 48.8 / 46.0, 128,256 x 2048 55.8 / 49.3 to 52.4, 151,936 x 1024 36.3 / 33.3;
+  // below, in L2, the ring: 70,000 x 1536 22.9 / 24.1; with few rows too: 13,000 x
+  // 8192 from HBM 31.2 / 36.7.
+  if (B == 1 && (int64_t)p.V * p.K >= kWideBytes && p.V >= 2 * kWideRows * kWideWarps * sms) {
+    p.nlists = kWideWarps;
+    e = launch_pdl(head_wide_kernel, dim3((unsigned)grid), dim3(kWideThreads), (size_t)p.Kpad + kCodePad, s, p);
+  } else {
+    e = launch_pdl(head_kernel<B>, dim3((unsigned)grid), dim3(kHeadThreads), smem, s, p);
+  }
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(B * kSelCluster, 1, 1);
@@ -804,7 +910,7 @@ cudaError_t launch_head(const HeadArgs& a, cudaStream_t s) {
   p.B = a.B;
   p.lists = static_cast<hkey*>(a.ws);
   p.lead = reinterpret_cast<hkey*>(static_cast<unsigned char*>(a.ws) + kListBytes);
-  p.nctas = 0;
+  p.nctas = p.nlists = 0;
   switch (a.B) {
     case 1: return launch_head_t<1>(p, dev, sms, s);
     case 2: return launch_head_t<2>(p, dev, sms, s);

@@ -185,6 +185,26 @@ def test_head_long_lists(B):
         check(run_head(head, h, tau, k_sel, V), Q, s, V, K, h, tau, k_sel, f"V={V} B={B}")
 
 
+@pytest.mark.parametrize("V,K", [(57_345, 2050), (150_001, 800), (400_003, 300)])
+def test_head_one_state_beyond_l2(V, K):
+    """One state whose weights L2 does not keep (the projection into registers):
+    ragged rows and columns, up to 64 rows per warp's list and more, equal
+    logits, and the best rows crowded into one CTA or a few."""
+    rng = synth.rng_for(7813, V, K)
+    ldw = (K + 15) // 16 * 16
+    Q = rng.integers(-127, 128, size=(V, ldw), dtype=np.int8)
+    s = (rng.uniform(0.5, 1.5, V) * (2.5 / 73 / math.sqrt(K))).astype(np.float32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    Qd = to_dev(Q)
+    h = rng.standard_normal((1, (K + 3) // 4 * 4)).astype(np.float32)
+    cta = np.arange(V) // 4 % (32 * sms) // 32
+    for ctas, hs, tau, k_sel in ((0, h, 0.0, 64), (0, h, np.inf, 64), (1, h, np.inf, 64), (40, h, np.inf, 16),
+                                 (0, np.zeros_like(h), np.inf, 64)):
+        sc = np.where(cta < ctas, s * np.float32(50), s).astype(np.float32)
+        head = sp.Head(Qd, to_dev(sc), K=K)
+        check(run_head(head, hs, tau, k_sel, V), Q, sc, V, K, hs, tau, k_sel, f"V={V} K={K} ctas={ctas} tau={tau}")
+
+
 @pytest.mark.parametrize("V,K", [(57344, 64), (9000, 64), (600, 512)])
 def test_head_candidates_in_few_units(V, K):
     """The best rows crowded into a few 16-row units, spread by the number of
