@@ -92,6 +92,7 @@ static_assert(kHeadRingBytes + SPIKE_PROJ_HEAD_MAX_B * (SPIKE_PROJ_HEAD_MAX_K + 
 static_assert((size_t)SPIKE_PROJ_HEAD_MAX_B * kHeadLists * kHeadList * 8 <= kHeadRingBytes, "the lists fit the ring");
 static_assert(kHeadLists * kCtaLead == 64, "the pairs' leading keys: two per lane of one warp");
 static_assert(kWideWarps <= SPIKE_PROJ_HEAD_MAX_B * kHeadLists, "one state's lists fit the workspace");
+static_assert(SPIKE_PROJ_HEAD_MAX_CAND * kCtaLead <= kSelCand, "the leading keys of 64 CTAs");
 static_assert(kHeadMaxGrid <= kSelThreads, "one projection CTA per selection thread");
 static_assert(kHeadList == 2 * kSelWarps * kSelCluster, "two candidates per selection warp");
 
@@ -656,6 +657,45 @@ head_wide_kernel(const __grid_constant__ HeadParams p) {
   }
 }
 
+// s_best <- the best 64 keys, descending, of s_cand[0 .. nshort) and of the lists
+// of n projection CTAs (those in s_long, or CTAs 0 .. n - 1); by a whole
+// selection CTA, with s_merge as scratch.  (A rare path: out of the way of the
+// code that every call runs through once.)
+__device__ __noinline__ void merge_lists(const hkey* lists, int nlists, const int* s_long, int n, const hkey* s_cand,
+                                         int nshort, hkey (*s_merge)[kHeadList], hkey* s_best) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  hkey a = 0ull, c = 0ull;
+  for (int i = 64 * warp; i < nshort; i += 64 * kSelWarps) {
+    hkey la = i + lane < nshort ? s_cand[i + lane] : 0ull;
+    hkey lb = i + 32 + lane < nshort ? s_cand[i + 32 + lane] : 0ull;
+    sort64(la, lb, lane);
+    list_merge(a, c, la, lb, lane);
+  }
+  for (int l = warp; l < n * nlists; l += kSelWarps) {
+    const hkey* L = lists + (int64_t)(s_long ? s_long[l / nlists] * nlists + l % nlists : l) * kHeadList;
+    hkey la = __ldcg(L + lane), lb = __ldcg(L + 32 + lane);
+    sort64(la, lb, lane);                        // (lists of up to 64 keys are as they came)
+    list_merge(a, c, la, lb, lane);
+  }
+  s_merge[warp][lane] = a;
+  s_merge[warp][32 + lane] = c;
+  __syncthreads();
+  if (warp == 0) {
+    for (int w = 1; w < kSelWarps; ++w) list_merge(a, c, s_merge[w][lane], s_merge[w][32 + lane], lane);
+    s_best[lane] = a;
+    s_best[32 + lane] = c;
+  }
+  __syncthreads();
+}
+
+// A sharper bound for the selection: *s_bound <- the 64th largest of the m keys
+// s_cand[0 .. m) (also a rare path).
+__device__ __noinline__ void sharper_bound(const hkey* s_cand, int m, hkey* s_bound) {
+  for (int i = threadIdx.x; i < m; i += kSelThreads)
+    if (s_cand[i] != 0ull && count_larger(s_cand, m, s_cand[i]) == kHeadList - 1) *s_bound = s_cand[i];
+  __syncthreads();
+}
+
 // Steps 3-6, a cluster of kSelCluster CTAs per hidden state.  Every CTA of
 // the cluster makes the same selection: the bound T (the 64th largest of the
 // projection CTAs' best keys, so at least 64 keys reach it), the keys >= T,
@@ -663,10 +703,10 @@ head_wide_kernel(const __grid_constant__ HeadParams p) {
 // leading keys all pass may have others in its lists, which are then read in
 // full.  The candidates are shared out (warp w of rank r recomputes 8 r + w
 // and 32 + 8 r + w), their logits meet in rank 0's shared memory, and rank 0
-// picks the token.  When the bound does not narrow the keys to at most
-// kSelCand, or more than kSelLong CTAs would be read in full (an adversarial
-// spread, e.g. equal logits everywhere), the warps merge every list instead:
-// slower, and exact either way.
+// picks the token.  Where more than kSelLong CTAs would be read in full a sharper
+// bound is taken; where more than kSelCand keys reach the bound the warps merge
+// the lists that hold them (or every list, when there is no bound): slower, and
+// exact either way.
 __global__ void __launch_bounds__(kSelThreads)
 head_select_kernel(const __grid_constant__ HeadParams p) {
   __shared__ hkey s_cand[kSelCand];
@@ -715,25 +755,51 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
   // this kernel's start its idle CTAs slowed the call (57,344 rows, one state,
   // tau 0.5: 24.6 against 24.0 us; four states 31.7 against 31.3).
   pdl_launch_dependents();
-  const hkey T = s_bound;
-  if (t < nc) {
-    int n = 0;
+  hkey T = s_bound;
+  // the leading keys >= T into s_cand; the CTAs whose lists may hold more
+  const auto gather_leads = [&]() {
+    if (t < nc) {
+      int n = 0;
 #pragma unroll
-    for (int e = 0; e < kCtaLead; ++e) n += lead[e] >= T;
-    if (n == kCtaLead) {                         // its lists may hold more
-      const int j = atomicAdd(&s_nlong, 1);
-      if (j < kSelLong) s_long[j] = t;
-    } else if (n > 0) {
-      const int i = atomicAdd(&s_nc, n);
+      for (int e = 0; e < kCtaLead; ++e) n += lead[e] >= T;
+      if (n == kCtaLead) {
+        const int j = atomicAdd(&s_nlong, 1);
+        if (j < kSelLong) s_long[j] = t;
+      } else if (n > 0) {
+        const int i = atomicAdd(&s_nc, n);
 #pragma unroll
-      for (int e = 0; e < kCtaLead - 1; ++e)
-        if (e < n && i + e < kSelCand) s_cand[i + e] = lead[e];
+        for (int e = 0; e < kCtaLead - 1; ++e)
+          if (e < n && i + e < kSelCand) s_cand[i + e] = lead[e];
+      }
     }
+    __syncthreads();
+  };
+  gather_leads();
+  if (s_nlong > kSelLong) {
+    // Best rows that are spread evenly, eight and more to a CTA, as equal logits
+    // are (3000 of them: 191 us a call by merging every list, 20 so): the bound is
+    // the 64th largest of all leading keys instead.  Those of 64 CTAs at most
+    // reach the first one, and at most eight CTAs reach this one in full.
+    __syncthreads();                             // every thread has read s_nlong
+    if (t == 0) s_nc = s_nlong = 0;
+    __syncthreads();
+    if (t < nc && lead[0] >= T) {
+      const int i = atomicAdd(&s_nc, kCtaLead);
+#pragma unroll
+      for (int e = 0; e < kCtaLead; ++e)
+        if (i + e < kSelCand) s_cand[i + e] = lead[e];
+    }
+    __syncthreads();
+    sharper_bound(s_cand, min(s_nc, kSelCand), &s_bound);   // (a barrier: s_nc and s_cand are read)
+    T = s_bound;
+    if (t == 0) s_nc = 0;
+    __syncthreads();
+    gather_leads();
   }
-  __syncthreads();
   const hkey* lists = p.lists + (int64_t)b * nc * p.nlists * kHeadList;
-  const int nlong = s_nlong;
-  if (nlong <= kSelLong) {
+  const int nlong = s_nlong, nshort = s_nc;      // (s_cand[0 .. nshort) are leading keys)
+  if (nlong > 0 && nlong <= kSelLong) {
+    __syncthreads();                             // every thread has read s_nc
     for (int j = 0; j < nlong; ++j) {
       const hkey* L = lists + (int64_t)s_long[j] * p.nlists * kHeadList;
 #pragma unroll 2
@@ -751,22 +817,12 @@ head_select_kernel(const __grid_constant__ HeadParams p) {
   if (C <= kSelCand && nlong <= kSelLong && C >= min(p.V, kHeadList)) {
     rank_place(s_cand, C, s_best);
   } else {
-    hkey a = 0ull, c = 0ull;
-    for (int l = warp; l < nc * p.nlists; l += kSelWarps) {
-      const hkey* L = lists + (int64_t)l * kHeadList;
-      hkey la = __ldcg(L + lane), lb = __ldcg(L + 32 + lane);
-      sort64(la, lb, lane);                      // (lists of up to 64 keys are as they came)
-      list_merge(a, c, la, lb, lane);
-    }
-    s_merge[warp][lane] = a;
-    s_merge[warp][32 + lane] = c;
-    __syncthreads();
-    if (warp == 0) {
-      for (int w = 1; w < kSelWarps; ++w) list_merge(a, c, s_merge[w][lane], s_merge[w][32 + lane], lane);
-      s_best[lane] = a;
-      s_best[32 + lane] = c;
-    }
-    __syncthreads();
+    // the lists of the CTAs that pass in full and the leading keys of the others,
+    // or every list
+    if (nlong <= kSelLong && C > kSelCand)
+      merge_lists(lists, p.nlists, s_long, nlong, s_cand, nshort, s_merge, s_best);
+    else
+      merge_lists(lists, p.nlists, nullptr, nc, s_cand, 0, s_merge, s_best);
   }
   const float g = __fsub_rn(key_z(s_best[0]), key_z(s_best[1]));
   const bool open = g < p.tau;

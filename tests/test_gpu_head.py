@@ -326,3 +326,28 @@ def test_head_weights_written_on_the_stream():
         head(hd, 4.0, 64, *out.values())
         got = {k: v.cpu().numpy() for k, v in out.items()}
         check(got, Q if i % 2 else -Q, s, V, K, h, 4.0, 64, f"call {i}")
+
+
+@pytest.mark.parametrize("V,K,B", [(3000, 256, 1), (9000, 64, 3), (57344, 64, 4), (1100, 40, 2)])
+def test_head_best_rows_spread_evenly(V, K, B):
+    """Eight and more of the best rows in each of many CTAs, so that the first
+    bound lets all of their leading keys pass and the sharper one is taken:
+    equal logits, and best rows boosted in the first 20 to 64 CTAs' units; many
+    calls in a row agree with the first."""
+    Q, s = small_case(7, V, K)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    unit = np.arange(V) // 16 % min(sms, -(-V // 16))
+    h = synth.rng_for(7814, V).standard_normal((B, (K + 3) // 4 * 4)).astype(np.float32)
+    for ctas in (0, 20, 64):
+        sc = np.where(unit < ctas, s * np.float32(50), s).astype(np.float32)
+        hs = h if ctas else np.zeros_like(h)
+        head = sp.Head(to_dev(Q), to_dev(sc), K=K)
+        first = run_head(head, hs, np.inf, 64, V)
+        check(first, Q, sc, V, K, hs, np.inf, 64, f"V={V} ctas={ctas}")
+        hd = to_dev(hs)
+        out = [torch.empty(200, *shape, dtype=dt, device=DEV)
+               for shape, dt in (((B,), torch.int32), ((B, 64), torch.int32))]
+        for i in range(200):
+            head(hd, np.inf, 64, out[0][i], None, None, out[1][i], None, None)
+        assert torch.all(out[0].cpu() == torch.from_numpy(first["token"]))
+        assert torch.all(out[1].cpu() == torch.from_numpy(first["cand"]))
