@@ -256,7 +256,8 @@ sp_status spike_proj_group_decode(sp_group_t group, const void *spikes,
  *         X[j] + t*ldx (t < T; words for BITS32, bytes for U8 and BOOL8).
  *         BOOL8 rows with a 16-byte aligned base and ldx % 16 == 0 are read
  *         in place; other rows go first through a 0/1 staging pass into the
- *         member plan's staging copy (one small launch per member).
+ *         member plan's staging copy (one small launch per member; a plan that
+ *         is a member again has a further copy, owned by the group).
  *   T     1 <= T <= every member plan's max_batch (else SP_ERANGE).
  *   ldx   row stride; ldx >= ceil(K_j/32) words (BITS32) or K_j bytes.
  *   acc   host array of `count` device pointers, member j's INT32 [T][N_j]

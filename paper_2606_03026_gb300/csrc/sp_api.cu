@@ -102,6 +102,10 @@ struct sp_group_s {
   int64_t rows_ld[kMaxProblems] = {};
   int32_t rows_T[kMaxProblems] = {};
   CUtensorMap rows_map[kMaxProblems];
+  // staging copy of a member whose plan is an earlier member too (that one has
+  // the plan's own), and its descriptor
+  uint8_t* xs[kMaxProblems] = {};
+  CUtensorMap xs_map[kMaxProblems];
 };
 
 namespace {
@@ -169,6 +173,7 @@ void group_free(sp_group_s* g) {
   if (!g) return;
   delete g->gemm;
   cudaFree(g->gpart);
+  for (uint8_t* xs : g->xs) cudaFree(xs);
   cudaFree(g->garrivals);
   cudaFree(g->ws);
   cudaFree(g->tickets);
@@ -704,6 +709,22 @@ sp_status spike_proj_group_create(sp_group_t* group, const sp_plan_t* plans, int
     group_free(g);
     return st;
   }
+  for (int j = 0; all_gemm && j < count; ++j) {
+    const sp_plan_s* p = plans[j];
+    bool again = false;
+    for (int i = 0; i < j; ++i) again = again || plans[i] == p;
+    if (!again) continue;
+    GemmMaps maps;
+    cudaError_t em = cudaSuccess;
+    if ((st = dev_alloc_zero(&g->xs[j], (size_t)p->xs_rows * p->Kp, s)) == SP_OK &&
+        (em = gemm_make_maps(g->xs[j], p->xs_rows, p->Wq, p->N, p->Kp, &maps)) != cudaSuccess)
+      st = cuda_fail(em);
+    if (st != SP_OK) {
+      group_free(g);
+      return st;
+    }
+    g->xs_map[j] = maps.a;
+  }
   g->params.ws = g->ws;
   g->params.tickets = g->tickets;
   g->params.err = g->err;
@@ -792,8 +813,9 @@ sp_status spike_proj_group_prefill(sp_group_t g, const void* const* X, sp_fmt fm
       }
       M.a = g->rows_map[j];
     } else {
-      SP_CUDA(launch_spikes_to_01(X[j], fmt, ldx, T, p->K, p->Kp, p->Xs, SpikeCount{}, s));
-      M.a = p->maps.a;
+      uint8_t* xs = g->xs[j] ? g->xs[j] : p->Xs;
+      SP_CUDA(launch_spikes_to_01(X[j], fmt, ldx, T, p->K, p->Kp, xs, SpikeCount{}, s));
+      M.a = g->xs[j] ? g->xs_map[j] : p->maps.a;
     }
     M.b = cl == 2 ? p->maps.b128 : p->maps.b;
     M.p.scale = p->scale;

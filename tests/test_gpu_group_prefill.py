@@ -267,6 +267,34 @@ def test_tail_ranges_one_after_another(T, shapes):
     group.close()
 
 
+@pytest.mark.parametrize("fmt", ["u8", "bits", "bool8"])
+def test_group_with_a_plan_twice(fmt):
+    """A plan that is two members of a group, each with rows of its own: staged
+    rows (u8, bits) do not meet in the plan's one staging copy."""
+    T, K = 140, 1000
+    members = make_members([(272, K, 288), (512, 700, 512)], T, seed=21)
+    order = [0, 1, 0, 0]
+    group = sp.Group([members[i][-1] for i in order])
+    X = [synth.bernoulli(synth.rng_for(7420, j), (T, K), 0.2) for j in range(len(order))]
+    if fmt == "bits":
+        xs_dev, ldx = [to_dev(synth.pack_bits(x)) for x in X], (K + 31) // 32
+    else:
+        ldx = 1008
+        xs_dev = []
+        for x in X:
+            r = np.zeros((T, ldx), np.uint8)
+            r[:, :K] = x
+            xs_dev.append(to_dev(r))
+    for rep in range(2):
+        accs, ys = run_group(group, [members[i] for i in order], xs_dev, fmt, T, ldx)
+        for j, i in enumerate(order):
+            Q, s, _, N, Ki, ldq, _ = members[i]
+            wa, wy = oracle.project(Q, s, N, Ki, X[j][:, :Ki], "u8", ldq=ldq)
+            assert_parity(accs[j], ys[j], wa, wy, f"member {j} rep {rep}")
+    assert group.status() == sp.SP_OK
+    group.close()
+
+
 def test_group_prefill_errors():
     members = make_members(RAGGED[:2], 8, seed=9)
     plain = sp.Plan(to_dev(members[0][0]), to_dev(members[0][1]), members[0][3], members[0][4],
