@@ -451,7 +451,7 @@ sp_status spike_proj_dense(const sp_dense *problems, int32_t count, int32_t B,
  * (Section 5, trace configuration; Appendix D).  The head's weights are a
  * continuous-input projection: W ROW-MAJOR INT8, row m (one vocabulary slot)
  * at W + m*ldw, K bytes used, with one FP32 scale per row.  For each hidden
- * state h, in ONE kernel launch:
+ * state h, in two kernel launches (projection and selection):
  *
  *   1. INT8 activations (the paper does not state the activation quantiser;
  *      this reads it as the weight rule of Section 2.3 applied to h):

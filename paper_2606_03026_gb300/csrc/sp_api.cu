@@ -378,12 +378,16 @@ sp_status run_gemm(sp_plan_s* p, const void* spikes, int fmt, int T, int64_t ld,
 //   GEMM, T <= 64 ~ 3.4 us + 0.33 us per K block of a CTA's K range
 //                   (ceil(Kp / 64 / S), S = the cluster size) + 0.045 us per row
 //   GEMM, T > 64  ~ max(11.3 us + 2 B N K ops / 1.4 PFLOP/s, 8.5 us + 0.55 us per 1024 of K)
-// (the GEMM only for SP_PLAN_GEMM plans).  The constants were fitted before
-// the kernels' latest speed-ups (both sides 0.2 to 1.3 us faster); measured
-// since, 1536 x 6144: gather (rows as a group) 3.6 / 4.6
-// / 5.6 / 6.4 us at B = 2 / 4 / 8 / 12, small-T GEMM 7.05 us at B = 16 and 8.5
-// at 64 (gather 16.2), the 128-row GEMM 10.9 us at B = 100; 1536 x 1536: the
-// gather up to B = 6, the small-T GEMM from B = 8 (5.7 us at 64).  The union
+// (the GEMM only for SP_PLAN_GEMM plans).  The kernels have become faster
+// since the fit.  Against both strategies timed (54 weight matrices of 256 x 256
+// to 4096 x 16384, rates 0.02 to 0.3), the choice costs 2 % over always taking
+// the faster one up to 64 rows.  At 65 to 173 rows it costs 18 %: there the
+// model is too high on both sides, the GEMM by 1.5 to 3.5 us (100 byte rows of
+// 1536 x 1536 9.4 us, model 11.6; 1536 x 6144 12.0, 12.6) and the gather of
+// small matrices by much more (100 rows of 512 x 512 3.7 us, model 12.2).  A
+// refit of the GEMM alone chooses worse (28 %); of both it chooses better (7 %),
+// but a gather of no columns is then mostly the faster one, and the calls that
+// do not wait for their count (below) would, for about 20 us each.  The union
 // fetch is never chosen automatically: it was slower than the per-token
 // gather at every batch size measured (its adds are ALU-bound, and the 126 MB
 // L2 serves the per-token re-reads of a 9.4 MB weight matrix).

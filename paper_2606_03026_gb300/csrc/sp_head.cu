@@ -54,10 +54,10 @@
 // the slower one (5.3 TB/s at the margin, whatever its depth, its lane layout or
 // the work per chunk; the register loads 7), and the call takes register loads.
 //
-// Measured on 57,344 x 1536, back to back with three weight copies, us a call:
-// gate closed 21.5 (22.0 before this form: the weights 14 of it, the codes
-// 1.3, the selection and the two hand-offs 6), every call verified 24.3 (26.0);
-// four states, every call verified 30.4 (60.6).
+// Measured on 57,344 x 1536, us a call through the binding: four states 31.7
+// (60.4 with a dp4a form per state and one selecting CTA), one state 23.1 to 24.1
+// (23.6: no gain; the weights are 14 of it, the codes 1.3, the selection and the
+// two hand-offs 6).
 #include "sp_internal.h"
 #include "sp_ptx.cuh"
 #include "sp_rows.cuh"
