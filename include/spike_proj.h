@@ -249,7 +249,9 @@ sp_status spike_proj_group_decode(sp_group_t group, const void *spikes,
  * 512-token prefill), for EVERY member of the group in ONE persistent launch:
  * the output tiles of all members (128 rows x 256 channels each) are shared
  * out over the SMs, and each tile runs over its whole K.  The members are
- * independent; nothing of member j reaches member i.  Results equal
+ * independent; nothing of member j reaches member i.  No CTA of the launch
+ * depends on another one's being resident (beside its partner of a CTA pair),
+ * so launches of several streams may share the device.  Results equal
  * spike_proj_prefill / spike_proj_batched on each member's plan, bit for bit.
  *
  *   X     host array of `count` device pointers; member j's rows at
